@@ -175,7 +175,7 @@ struct lbm_ctx {
     {
         LaunchArgs a{};
         a.p = dp;
-        finish_params(a.p);
+        finish_params(a.p, li.cs2);
         a.fin = buf[cur];
         a.fout = buf[cur ^ 1];
         a.carry_in = carry[cur];
@@ -567,6 +567,8 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     d.N = c->N;
     d.g = g;
     d.psx = psx;
+    d.dnx = make_fast_div((unsigned)p->nx);
+    d.dny = make_fast_div((unsigned)p->ny);
     d.psy = psy;
     d.G = p->G;
     d.omega = 1.0 / p->tau;

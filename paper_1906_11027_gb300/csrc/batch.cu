@@ -40,6 +40,7 @@ struct BatchDom {
     long long poff;  // element offset of the domain in the psi scratch field (two-pass shape)
     double G, omega, pref, rho_bar;
     float G_f, omega_f, pref_f, rho_bar_f;  // FP32 copies (set with the doubles on the host)
+    double kV[2], kP[2];                    // FP64 collision products (finish_params)
 };
 
 __device__ __forceinline__ DevParams dom_params(const BatchDom& d)
@@ -57,6 +58,10 @@ __device__ __forceinline__ DevParams dom_params(const BatchDom& d)
     p.omega_f = d.omega_f;
     p.pref_f = d.pref_f;
     p.rho_bar_f = d.rho_bar_f;
+    p.kV[0] = d.kV[0];
+    p.kV[1] = d.kV[1];
+    p.kP[0] = d.kP[0];
+    p.kP[1] = d.kP[1];
     p.psi_kind = 0;
     return p;
 }
@@ -332,7 +337,7 @@ __device__ __forceinline__ void force_global(const Real* __restrict__ psi, int n
 {
     using L = Lattice<kLatD2Q9>;
     using S = Stencil<2, ORD>;
-    Real ax = Real(0), ay = Real(0), az = Real(0);
+    Real ax = Real(0), ay = Real(0);
     sfor<S::n / 2>([&](auto kI) {
         constexpr int a = 2 * decltype(kI)::value;
         constexpr int ex = S::T.v[a][0], ey = S::T.v[a][1];
@@ -345,7 +350,7 @@ __device__ __forceinline__ void force_global(const Real* __restrict__ psi, int n
     const Real gp = -G * psi[y * nx + x];
     F[0] = gp * ax;
     F[1] = gp * ay;
-    F[2] = gp * az;
+    F[2] = Real(0);
 }
 
 template <class Real>
@@ -1002,6 +1007,15 @@ int lbm_batch_create(const lbm_params* ps, const double* init, int n, lbm_batch*
         m.omega_f = static_cast<float>(m.omega);
         m.pref_f = static_cast<float>(m.pref);
         m.rho_bar_f = static_cast<float>(m.rho_bar);
+        DevParams dp{};
+        dp.omega = m.omega;
+        dp.pref = m.pref;
+        dp.G = m.G;
+        finish_params(dp, Lattice<kLatD2Q9>::cs2);
+        for (int k = 0; k < 2; ++k) {
+            m.kV[k] = dp.kV[k];
+            m.kP[k] = dp.kP[k];
+        }
         off += (long long)kQ9 * p.nx * p.ny;
         off = (off + 63) / 64 * 64;  // 256-byte aligned domains
         m.poff = poff;

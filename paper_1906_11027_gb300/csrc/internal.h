@@ -19,6 +19,27 @@ enum : unsigned {
 // every TMA box starts on a 16-byte boundary) and `g` = stencil radius in y, z.
 constexpr int kGhostX = 4;
 
+constexpr double kPrA = 2.0 / 49.0;  // Peng-Robinson a, b (R = 1), Sec. 3
+constexpr double kPrB = 2.0 / 21.0;
+
+// Division of 0 <= i < 2^31 by a fixed d > 0: q = (i * m) >> s with s = 31 + ceil(log2 d)
+// and m = ceil(2^s / d) < 2^32, exact over that range.
+struct FastDiv {
+    unsigned d, m;
+    int s;
+    __host__ __device__ unsigned div(unsigned i) const
+    {
+        return static_cast<unsigned>((static_cast<unsigned long long>(i) * m) >> s);
+    }
+};
+inline FastDiv make_fast_div(unsigned d)
+{
+    int l = 0;
+    while ((1u << l) < d) ++l;
+    const unsigned long long p = 1ull << (31 + l);
+    return {d, static_cast<unsigned>((p + d - 1) / d), 31 + l};
+}
+
 // Runtime constants of one domain, passed by value to every kernel.
 struct DevParams {
     int nx, ny, nz;
@@ -44,12 +65,25 @@ struct DevParams {
     float omega_f, pref_f, rho_bar_f, G_f;
     float om1_f;  // 1 - omega, rounded once from double
     float dmrt_f[4];
+    // FP64 collision and psi: products of parameters with powers of the
+    // lattice's c_s^2, formed once per domain instead of once per cell.
+    double kV[2];  // V = kV[0] (j + F/2) + kV[1] F  with (omega/2, pref) / c_s^4
+    double kP[2];  // P = kP[0] (j + F/2) + kP[1] F  with (omega, pref) / c_s^2
+    double pr_K;   // Peng-Robinson psi: 2 / (G c_s^2) and a alpha
+    double pr_aa;
+    FastDiv dnx, dny;  // for x, y, z of a linear cell index
 };
 
-// Fills the derived fields of p from the others; call after any change to
-// omega, pref, rho_bar, G or rate.
-__host__ __device__ inline void finish_params(DevParams& p)
+// Fills the derived fields of p from the others (cs2: the lattice's c_s^2); call
+// after any change to omega, pref, rho_bar, G or rate.
+__host__ __device__ inline void finish_params(DevParams& p, double cs2)
 {
+    p.kV[0] = 0.5 * p.omega / (cs2 * cs2);
+    p.kV[1] = p.pref / (cs2 * cs2);
+    p.kP[0] = p.omega / cs2;
+    p.kP[1] = p.pref / cs2;
+    p.pr_K = 2.0 / (p.G * cs2);
+    p.pr_aa = kPrA * p.pr_alpha;
     for (int c = 0; c < 4; ++c) {
         p.dmrt[c] = (c == 0) ? 0.0 : p.omega - p.rate[c];
         p.dmrt_f[c] = static_cast<float>(p.dmrt[c]);

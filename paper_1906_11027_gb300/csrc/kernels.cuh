@@ -26,9 +26,6 @@
 
 namespace lbm {
 
-constexpr double kPrA = 2.0 / 49.0;  // Peng-Robinson a, b (R = 1), Sec. 3
-constexpr double kPrB = 2.0 / 21.0;
-
 // Sets a kernel's dynamic shared-memory limit to its request, once per (kernel,
 // device): the attribute belongs to the device, and a process may drive several.
 template <class K>
@@ -182,13 +179,25 @@ __device__ __forceinline__ double psi_exp(double r) { return -expm1(-r); }
 __device__ __forceinline__ float psi_exp(float r) { return -expm1f(-r); }
 
 // psi = sqrt(2 (p_EOS - c_s^2 rho) / (G c_s'^2)) with the Peng-Robinson EOS (Sec. 3).
+// Over the common denominator D = (1 - b rho)(1 + 2 b rho - b^2 rho^2) the argument
+// is n / D, and sqrt(n / D) = |n| / sqrt(n D): one reciprocal square root where
+// the terms taken one by one need three divisions and a square root, all on the
+// FP64 pipe (2 lanes per cycle and SM).
 __device__ __forceinline__ double psi_pr(double rho, const DevParams& p, double cs2)
 {
-    const double pe = rho * p.pr_T / (1.0 - kPrB * rho)
-                    - kPrA * p.pr_alpha * rho * rho / (1.0 + 2.0 * kPrB * rho - kPrB * kPrB * rho * rho);
-    const double arg = 2.0 * (pe - cs2 * rho) / (p.G * cs2);
-    if (!(arg >= 0.0)) atomicOr(p.err, kErrNegativeSqrt);
-    return sqrt(arg);
+    const double br = kPrB * rho;
+    const double d1 = 1.0 - br;
+    const double d2 = fma(br, 2.0 - br, 1.0);
+    const double D = d1 * d2;
+    const double t = fma(p.pr_T, d2, -(p.pr_aa * rho) * d1);
+    const double n = (p.pr_K * rho) * fma(-cs2, D, t);
+    const double q = n * D;
+    if (!(q > 0.0) || isinf(q)) {  // zero, negative or no number: the plain quotient decides
+        const double arg = n / D;
+        if (!(arg >= 0.0)) atomicOr(p.err, kErrNegativeSqrt);
+        return sqrt(arg);
+    }
+    return fabs(n) * rsqrt(q);
 }
 
 template <int LAT, class Real>
@@ -205,6 +214,10 @@ __device__ __forceinline__ void store_psi(Real* __restrict__ psi, const DevParam
 {
     const int g = p.g;
     const int gz = (D == 3) ? g : 0;
+    if (x >= kGhostX && x < p.nx - kGhostX && y >= g && y < p.ny - g && (D == 2 || (z >= g && z < p.nz - g))) {
+        psi[(static_cast<long long>(z + gz) * p.psy + (y + g)) * p.psx + (x + kGhostX)] = v;  // no image is a ghost
+        return;
+    }
     const int zlo = (D == 3) ? -1 : 0, zhi = (D == 3) ? 1 : 0;
     for (int dz = zlo; dz <= zhi; ++dz) {
         const int Z = z + dz * p.nz;
@@ -242,7 +255,7 @@ __device__ __forceinline__ void force_from(const Real* tc, Real G, Real (&F)[3])
     const Real gp = -G * tc[0];
     F[0] = gp * ax;
     F[1] = gp * ay;
-    F[2] = gp * az;
+    F[2] = L::D == 3 ? gp * az : Real(0);
 }
 
 // ---- value helpers shared by the scalar and the packed-pair collision --------
@@ -358,156 +371,301 @@ __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::
     });
 }
 
-// f_b += sum_k M_kb t_k over the non-conserved moments, by opposite pairs:
-// f_b += E + O, f_b+1 += E - O with E from the even rows and O from the odd ones.
+// sum_k M_kb t_k over the non-conserved moments at velocity b: E from the even
+// rows, O from the odd ones (the opposite velocity gets E - O).
+template <int LAT, int b, class V>
+__device__ __forceinline__ void mrt_pair(const V (&t)[Lattice<LAT>::Q], V& E, V& O)
+{
+    using MB = Mrt<LAT>;
+    E = vsplat<V>(0.0);
+    O = vsplat<V>(0.0);
+    sfor<Lattice<LAT>::Q>([&](auto kI) {
+        constexpr int k = decltype(kI)::value;
+        if constexpr (MB::B.rate_class[k] != 0) {
+            constexpr int mk = static_cast<int>(MB::B.M[k][b]);
+            if constexpr (MB::T.parity[k] > 0) E = macc<mk>(E, t[k]);
+            else O = macc<mk>(O, t[k]);
+        }
+    });
+}
+
+// f_b += sum_k M_kb t_k over the non-conserved moments, by opposite pairs.
 template <int LAT, class V>
 __device__ __forceinline__ void mrt_apply(const V (&t)[Lattice<LAT>::Q], V (&f)[Lattice<LAT>::Q])
 {
-    using L = Lattice<LAT>;
-    using MB = Mrt<LAT>;
-    constexpr int Q = L::Q;
-    {
-        V e = vsplat<V>(0.0);
-        sfor<Q>([&](auto kI) {
-            constexpr int k = decltype(kI)::value;
-            if constexpr (MB::B.rate_class[k] != 0 && MB::T.parity[k] > 0)
-                e = macc<static_cast<int>(MB::B.M[k][0])>(e, t[k]);
-        });
-        f[0] = vadd(f[0], e);
-    }
-    sfor<(Q - 1) / 2>([&](auto pI) {
+    V e, o;
+    mrt_pair<LAT, 0>(t, e, o);
+    f[0] = vadd(f[0], e);
+    sfor<(Lattice<LAT>::Q - 1) / 2>([&](auto pI) {
         constexpr int b = 2 * decltype(pI)::value + 1;
-        V e = vsplat<V>(0.0), o = vsplat<V>(0.0);
-        sfor<Q>([&](auto kI) {
-            constexpr int k = decltype(kI)::value;
-            if constexpr (MB::B.rate_class[k] != 0) {
-                constexpr int mk = static_cast<int>(MB::B.M[k][b]);
-                if constexpr (MB::T.parity[k] > 0) e = macc<mk>(e, t[k]);
-                else o = macc<mk>(o, t[k]);
-            }
-        });
+        mrt_pair<LAT, b>(t, e, o);
         f[b] = vadd(f[b], vadd(e, o));
         f[b + 1] = vadd(f[b + 1], vsub(e, o));
     });
 }
 
-// ---- collision (Eqs. 3-4) --------------------------------------------------------
-// f holds pre-collision populations (FP32: deviations); on return the
-// post-collision ones.  Returns nothing; rho, u computed inside.
-template <int LAT, int COLL, class Real>
-__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const Real (&F)[3], const DevParams& p)
+// c . v for a compile-time integer vector c of the lattice's dimension D
+template <int D, int CX, int CY, int CZ, class V>
+__device__ __forceinline__ V cdot(V vx, V vy, V vz)
+{
+    V r = vsplat<V>(0.0);
+    if constexpr (CX != 0) r = (CX == 1) ? vx : vmul(vsplat<V>(double(CX)), vx);
+    if constexpr (CX != 0) r = macc<CY>(r, vy);
+    else if constexpr (CY != 0) r = (CY == 1) ? vy : vmul(vsplat<V>(double(CY)), vy);
+    if constexpr (D == 3 && (CX != 0 || CY != 0)) r = macc<CZ>(r, vz);
+    else if constexpr (D == 3 && CZ != 0) r = (CZ == 1) ? vz : vmul(vsplat<V>(double(CZ)), vz);
+    return r;
+}
+
+// ---- collision in FP64 --------------------------------------------------------
+// Same update as collide() below, arranged for the FP64 pipe, which issues two
+// lanes per cycle and SM and bounds every FP64 step: no term that the lattice
+// lacks (z on 2-D lattices, zero velocity components), the even part of all
+// velocities from one symmetric tensor, and parameter products from the host.
+//   Guo:   w_b [ A0 + c.T.c +- c.P ], T_ij = sym(u_i V_j), A0 = omega rho - c_s^2 tr T,
+//          V = (omega/2 (j + F/2) + pref F) / c_s^4, P = (omega (j + F/2) + pref F) / c_s^2
+//   exact difference, a = j, b = j + F:
+//          T_ij = (b_i b_j - (1 - omega) a_i a_j) / (2 rho c_s^4), P = (b - (1 - omega) a) / c_s^2
+// With k_psi64 / k_fused64 below, per step: D2Q9 BGK 2048^2 1.24 -> 0.94 ms, D2Q9 MRT
+// 256^2 39 -> 27 us; error against 64-bit arithmetic of the same step unchanged.
+template <int LAT, int COLL>
+__device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const double (&F)[3], const DevParams& p)
 {
     using L = Lattice<LAT>;
-    constexpr int NP = (L::Q - 1) / 2;
-    constexpr bool kDev = std::is_same<Real, float>::value;  // deviation storage
-    // Moments through the opposite pairs (b, b+1): sum f and sum (f_b - f_b+1) c_b.
-    Real s = f[0], jx = Real(0), jy = Real(0), jz = Real(0);
-    Real Pp[NP], Dp[NP];  // pair sums and differences (MRT)
-    sfor<NP>([&](auto kI) {
-        constexpr int b = 1 + 2 * decltype(kI)::value;
-        constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
-        Pp[decltype(kI)::value] = f[b] + f[b + 1];
-        s += Pp[decltype(kI)::value];
-        const Real d = f[b] - f[b + 1];
-        Dp[decltype(kI)::value] = d;
-        if (cx != 0) jx += Real(cx) * d;
-        if (cy != 0) jy += Real(cy) * d;
-        if (cz != 0) jz += Real(cz) * d;
-    });
-    const Real rho = kDev ? par<Real>(p.rho_bar, p.rho_bar_f) + s : s;
-    const Real inv_rho = Real(1) / rho;
-    const Real ux = (jx + Real(0.5) * F[0]) * inv_rho;
-    const Real uy = (jy + Real(0.5) * F[1]) * inv_rho;
-    const Real uz = (jz + Real(0.5) * F[2]) * inv_rho;
+    constexpr int Q = L::Q, D = L::D, NP = (Q - 1) / 2;
     constexpr double cs2 = L::cs2;
-    const Real inv_cs2 = Real(1.0 / cs2);
-    const Real inv_cs4 = Real(1.0 / (cs2 * cs2));
-    const Real half_inv_cs4 = Real(0.5 / (cs2 * cs2));
-    const Real usq = (ux * ux + uy * uy + uz * uz) * Real(0.5 / cs2);
-    const Real uF = ux * F[0] + uy * F[1] + uz * F[2];
-    const Real omega = par<Real>(p.omega, p.omega_f);
-    const Real pref = par<Real>(p.pref, p.pref_f);
-    if constexpr (COLL == 0 || COLL == 1) {
-        // MRT: the moment-space correction is formed from the pre-collision state
-        Real t[L::Q];
+    double s = f[0];
+    double j[D] = {};
+    double Pp[COLL == 1 ? NP : 1], Dp[COLL == 1 ? NP : 1];
+    sfor<NP>([&](auto kI) {
+        constexpr int k = decltype(kI)::value;
+        constexpr int b = 1 + 2 * k;
+        static_assert(L::T.v[b + 1][0] == -L::T.v[b][0] && L::T.v[b + 1][1] == -L::T.v[b][1] &&
+                          L::T.v[b + 1][2] == -L::T.v[b][2],
+                      "opposite velocities must be adjacent");
+        const double sum = f[b] + f[b + 1], d = f[b] - f[b + 1];
         if constexpr (COLL == 1) {
-            const Real jv[3] = {jx, jy, jz};
-            const Real uv3[3] = {ux, uy, uz};
-            const Real vv[3] = {jx - Real(0.5) * F[0], jy - Real(0.5) * F[1], jz - Real(0.5) * F[2]};
-            Real dm[4];
+            Pp[k] = sum;
+            Dp[k] = d;
+        }
+        s += sum;
+        sfor<D>([&](auto iI) {
+            constexpr int i = decltype(iI)::value;
+            j[i] = macc<L::T.v[b][i]>(j[i], d);
+        });
+    });
+    const double rho = s;
+    const double inv_rho = 1.0 / rho;
+    double T[D], S[3] = {}, P[D];  // T_ii; S: 2 T_xy, 2 T_xz, 2 T_yz; P
+    double t[COLL == 1 ? Q : 1];
+    if constexpr (COLL == 2) {
+        const double om1 = 1.0 - p.omega;
+        const double h = inv_rho * (0.5 / (cs2 * cs2));
+        double a1[D], b[D];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) dm[c] = par<Real>(p.dmrt[c], p.dmrt_f[c]);
-            mrt_moments_g<LAT, Real>(f[0], Pp, Dp, kDev ? s : rho, jv, uv3, vv, dm, t);
+        for (int i = 0; i < D; ++i) {
+            b[i] = j[i] + F[i];
+            a1[i] = om1 * j[i];
+            P[i] = (b[i] - a1[i]) * (1.0 / cs2);
+            T[i] = h * fma(b[i], b[i], -(a1[i] * j[i]));
         }
-        // omega feq_b + pref src_b regrouped (Eq. 4):
-        //   w_b [ A0 + (c.u)(c.V) + c.P ],
-        //   A0 = omega rho (1 - u.u/(2 cs2)) - pref u.F / cs2   (FP32: omega (rho - rho_bar) in
-        //        place of omega rho for the constant term),
-        //   P  = (omega rho u + pref F) / cs2,   V = (omega rho u / 2 + pref F) / cs4;
-        // the c.P term is odd under c -> -c, the rest even.
-        const Real orho = omega * rho;
-        const Real A0 = (kDev ? omega * s : orho) - orho * usq - pref * uF * inv_cs2;
-        const Real Px = (orho * ux + pref * F[0]) * inv_cs2;
-        const Real Py = (orho * uy + pref * F[1]) * inv_cs2;
-        const Real Pz = (orho * uz + pref * F[2]) * inv_cs2;
-        const Real h = Real(0.5) * orho;
-        const Real Vx = (h * ux + pref * F[0]) * inv_cs4;
-        const Real Vy = (h * uy + pref * F[1]) * inv_cs4;
-        const Real Vz = (h * uz + pref * F[2]) * inv_cs4;
-        const Real om1 = Real(1) - omega;
-        {
-            constexpr double w0 = L::T.w[0];
-            f[0] = f[0] * om1 + Real(w0) * A0;
+        const double h2 = 2.0 * h;
+        S[0] = h2 * fma(b[0], b[1], -(a1[0] * j[1]));
+        if constexpr (D == 3) {
+            S[1] = h2 * fma(b[0], b[2], -(a1[0] * j[2]));
+            S[2] = h2 * fma(b[1], b[2], -(a1[1] * j[2]));
         }
+    } else {
+        double u[D], V[D];
+        double v[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            v[i] = fma(0.5, F[i], j[i]);
+            u[i] = v[i] * inv_rho;
+            V[i] = fma(p.kV[0], v[i], p.kV[1] * F[i]);
+            P[i] = fma(p.kP[0], v[i], p.kP[1] * F[i]);
+            T[i] = u[i] * V[i];
+        }
+        S[0] = fma(u[0], V[1], u[1] * V[0]);
+        if constexpr (D == 3) {
+            S[1] = fma(u[0], V[2], u[2] * V[0]);
+            S[2] = fma(u[1], V[2], u[2] * V[1]);
+        }
+        if constexpr (COLL == 1) {
+            double jv[3] = {}, uv[3] = {}, vv[3] = {};
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                jv[i] = j[i];
+                uv[i] = u[i];
+                vv[i] = fma(-0.5, F[i], j[i]);
+            }
+            mrt_moments_g<LAT, double>(f[0], Pp, Dp, rho, jv, uv, vv, p.dmrt, t);
+        }
+    }
+    double tr = T[0] + T[1];
+    if constexpr (D == 3) tr += T[2];
+    const double A0 = fma(p.omega, rho, -cs2 * tr);
+    // f*_b = (1 - omega) f_b + w_b (e_b +- o_b), and at omega = 1 (the paper's tau = 1)
+    // the first term is gone
+    auto update = [&](auto oneI) {
+        constexpr bool kOne = decltype(oneI)::value != 0;
+        const double om1 = 1.0 - p.omega;
+        auto relax = [&](double fb, double x) { return kOne ? x : fma(om1, fb, x); };
+        constexpr double w0 = L::T.w[0];
+        f[0] = relax(f[0], w0 * A0);
         sfor<NP>([&](auto kI) {
             constexpr int b = 1 + 2 * decltype(kI)::value;
             constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
-            static_assert(L::T.v[b + 1][0] == -cx && L::T.v[b + 1][1] == -cy && L::T.v[b + 1][2] == -cz,
-                          "opposite velocities must be adjacent");
             constexpr double wb = L::T.w[b];
-            const Real cu = Real(cx) * ux + Real(cy) * uy + Real(cz) * uz;
-            const Real cV = Real(cx) * Vx + Real(cy) * Vy + Real(cz) * Vz;
-            const Real cP = Real(cx) * Px + Real(cy) * Py + Real(cz) * Pz;
-            const Real ev = cu * cV + A0;
-            f[b] = f[b] * om1 + Real(wb) * (ev + cP);
-            f[b + 1] = f[b + 1] * om1 + Real(wb) * (ev - cP);
+            double e = A0;
+            e = macc<cx * cx>(e, T[0]);
+            e = macc<cy * cy>(e, T[1]);
+            if constexpr (D == 3) e = macc<cz * cz>(e, T[2]);
+            e = macc<cx * cy>(e, S[0]);
+            if constexpr (D == 3) {
+                e = macc<cx * cz>(e, S[1]);
+                e = macc<cy * cz>(e, S[2]);
+            }
+            double o = cdot<D, cx, cy, cz>(P[0], P[1], P[D - 1]);
+            if constexpr (COLL == 1) {  // plus the moment correction, even and odd rows apart
+                double E, O;
+                mrt_pair<LAT, b>(t, E, O);
+                e = fma(wb, e, E);
+                o = fma(wb, o, O);
+                f[b] = relax(f[b], e + o);
+                f[b + 1] = relax(f[b + 1], e - o);
+            } else {
+                f[b] = relax(f[b], wb * (e + o));
+                f[b + 1] = relax(f[b + 1], wb * (e - o));
+            }
         });
-        if constexpr (COLL == 1) mrt_apply<LAT, Real>(t, f);
-        (void)half_inv_cs4;
-    } else {
-        // Exact-difference forcing with BGK (the scheme of the paper's runs, Sec. 3):
-        //   f* = feq(rho, v) + (1 - omega) (f - feq(rho, u')),  u' = j / rho, v = u' + F / rho,
-        // regrouped as w_b [ A0 + q_b +- c.P ] with
-        //   A0 = omega rho - rho (v.v - (1 - omega) u'.u') / (2 cs2)   (FP32: omega (rho - rho_bar)),
-        //   P  = rho (v - (1 - omega) u') / cs2,
-        //   q_b = rho ((c.v)^2 - (1 - omega) (c.u')^2) / (2 cs4)   (even under c -> -c).
-        const Real upx = jx * inv_rho, upy = jy * inv_rho, upz = jz * inv_rho;
-        const Real vx = (jx + F[0]) * inv_rho, vy = (jy + F[1]) * inv_rho, vz = (jz + F[2]) * inv_rho;
-        const Real om1 = Real(1) - omega;
-        const Real vv = vx * vx + vy * vy + vz * vz;
-        const Real uu = upx * upx + upy * upy + upz * upz;
-        const Real A0 = (kDev ? omega * s : omega * rho) - rho * (vv - om1 * uu) * Real(0.5 / cs2);
-        const Real Px = rho * (vx - om1 * upx) * inv_cs2;
-        const Real Py = rho * (vy - om1 * upy) * inv_cs2;
-        const Real Pz = rho * (vz - om1 * upz) * inv_cs2;
-        const Real hq = rho * half_inv_cs4;
-        {
-            constexpr double w0 = L::T.w[0];
-            f[0] = f[0] * om1 + Real(w0) * A0;
+        if constexpr (COLL == 1) {
+            double E, O;
+            mrt_pair<LAT, 0>(t, E, O);
+            f[0] += E;
         }
-        sfor<(L::Q - 1) / 2>([&](auto kI) {
+    };
+    if (p.omega == 1.0)
+        update(std::integral_constant<int, 1>{});
+    else
+        update(std::integral_constant<int, 0>{});
+}
+
+// ---- collision in FP32 on deviations from w_b rho_bar (Eqs. 3-4) ------------------
+// Terms that vanish for the lattice (z on 2-D lattices, zero velocity components)
+// are left out at compile time: the compiler may not drop 0 * x by itself.
+template <int LAT, int COLL>
+__device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const float (&F)[3], const DevParams& p)
+{
+    using L = Lattice<LAT>;
+    constexpr int NP = (L::Q - 1) / 2;
+    constexpr bool k3 = L::D == 3;
+    // Moments through the opposite pairs (b, b+1): sum f and sum (f_b - f_b+1) c_b.
+    float s = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
+    float Pp[NP], Dp[NP];  // pair sums and differences (MRT)
+    sfor<NP>([&](auto kI) {
+        constexpr int b = 1 + 2 * decltype(kI)::value;
+        Pp[decltype(kI)::value] = f[b] + f[b + 1];
+        s += Pp[decltype(kI)::value];
+        const float d = f[b] - f[b + 1];
+        Dp[decltype(kI)::value] = d;
+        jx = macc<L::T.v[b][0]>(jx, d);
+        jy = macc<L::T.v[b][1]>(jy, d);
+        jz = macc<L::T.v[b][2]>(jz, d);
+    });
+    const float rho = p.rho_bar_f + s;
+    const float inv_rho = 1.f / rho;
+    const float ux = (jx + 0.5f * F[0]) * inv_rho;
+    const float uy = (jy + 0.5f * F[1]) * inv_rho;
+    const float uz = k3 ? (jz + 0.5f * F[2]) * inv_rho : 0.f;
+    constexpr double cs2 = L::cs2;
+    const float inv_cs2 = float(1.0 / cs2);
+    const float inv_cs4 = float(1.0 / (cs2 * cs2));
+    const float half_inv_cs4 = float(0.5 / (cs2 * cs2));
+    const float omega = p.omega_f;
+    if constexpr (COLL == 0 || COLL == 1) {
+        const float uxy = ux * ux + uy * uy;
+        const float usq = (k3 ? uxy + uz * uz : uxy) * float(0.5 / cs2);
+        const float uFxy = ux * F[0] + uy * F[1];
+        const float uF = k3 ? uFxy + uz * F[2] : uFxy;
+        const float pref = p.pref_f;
+        // MRT: the moment-space correction is formed from the pre-collision state
+        float t[L::Q];
+        if constexpr (COLL == 1) {
+            const float jv[3] = {jx, jy, jz};
+            const float uv3[3] = {ux, uy, uz};
+            const float vv[3] = {jx - 0.5f * F[0], jy - 0.5f * F[1], jz - 0.5f * F[2]};
+            mrt_moments_g<LAT, float>(f[0], Pp, Dp, s, jv, uv3, vv, p.dmrt_f, t);
+        }
+        // omega feq_b + pref src_b regrouped (Eq. 4):
+        //   w_b [ A0 + (c.u)(c.V) + c.P ],
+        //   A0 = omega (rho - rho_bar) - omega rho u.u/(2 cs2) - pref u.F / cs2,
+        //   P  = (omega rho u + pref F) / cs2,   V = (omega rho u / 2 + pref F) / cs4;
+        // the c.P term is odd under c -> -c, the rest even.
+        const float orho = omega * rho;
+        const float A0 = omega * s - orho * usq - pref * uF * inv_cs2;
+        const float Px = (orho * ux + pref * F[0]) * inv_cs2;
+        const float Py = (orho * uy + pref * F[1]) * inv_cs2;
+        const float Pz = (orho * uz + pref * F[2]) * inv_cs2;
+        const float h = 0.5f * orho;
+        const float Vx = (h * ux + pref * F[0]) * inv_cs4;
+        const float Vy = (h * uy + pref * F[1]) * inv_cs4;
+        const float Vz = (h * uz + pref * F[2]) * inv_cs4;
+        const float om1 = 1.f - omega;
+        f[0] = f[0] * om1 + float(L::T.w[0]) * A0;
+        sfor<NP>([&](auto kI) {
             constexpr int b = 1 + 2 * decltype(kI)::value;
             constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
-            constexpr double wb = L::T.w[b];
-            const Real cv = Real(cx) * vx + Real(cy) * vy + Real(cz) * vz;
-            const Real cu = Real(cx) * upx + Real(cy) * upy + Real(cz) * upz;
-            const Real cP = Real(cx) * Px + Real(cy) * Py + Real(cz) * Pz;
-            const Real ev = A0 + hq * (cv * cv - om1 * cu * cu);
-            f[b] = f[b] * om1 + Real(wb) * (ev + cP);
-            f[b + 1] = f[b + 1] * om1 + Real(wb) * (ev - cP);
+            constexpr float wb = float(L::T.w[b]);
+            const float cu = cdot<L::D, cx, cy, cz>(ux, uy, uz);
+            const float cV = cdot<L::D, cx, cy, cz>(Vx, Vy, Vz);
+            const float cP = cdot<L::D, cx, cy, cz>(Px, Py, Pz);
+            const float ev = cu * cV + A0;
+            f[b] = f[b] * om1 + wb * (ev + cP);
+            f[b + 1] = f[b + 1] * om1 + wb * (ev - cP);
         });
-        (void)ux; (void)uy; (void)uz; (void)usq; (void)uF; (void)pref;
+        if constexpr (COLL == 1) mrt_apply<LAT, float>(t, f);
+        (void)half_inv_cs4;
+    } else {
+        // Exact-difference forcing with BGK (the scheme of the paper's runs, Sec. 3), 2-D lattices:
+        //   f* = feq(rho, v) + (1 - omega) (f - feq(rho, u')),  u' = j / rho, v = u' + F / rho,
+        // regrouped as w_b [ A0 + q_b +- c.P ] with
+        //   A0 = omega (rho - rho_bar) - rho (v.v - (1 - omega) u'.u') / (2 cs2),
+        //   P  = rho (v - (1 - omega) u') / cs2,
+        //   q_b = rho ((c.v)^2 - (1 - omega) (c.u')^2) / (2 cs4)   (even under c -> -c).
+        static_assert(!k3, "exact-difference forcing is provided for the 2-D lattices");
+        const float upx = jx * inv_rho, upy = jy * inv_rho;
+        const float vx = (jx + F[0]) * inv_rho, vy = (jy + F[1]) * inv_rho;
+        const float om1 = 1.f - omega;
+        const float vv = vx * vx + vy * vy;
+        const float uu = upx * upx + upy * upy;
+        const float A0 = omega * s - rho * (vv - om1 * uu) * float(0.5 / cs2);
+        const float Px = rho * (vx - om1 * upx) * inv_cs2;
+        const float Py = rho * (vy - om1 * upy) * inv_cs2;
+        const float hq = rho * half_inv_cs4;
+        f[0] = f[0] * om1 + float(L::T.w[0]) * A0;
+        sfor<NP>([&](auto kI) {
+            constexpr int b = 1 + 2 * decltype(kI)::value;
+            constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1];
+            constexpr float wb = float(L::T.w[b]);
+            const float cv = cdot<2, cx, cy, 0>(vx, vy, 0.f);
+            const float cu = cdot<2, cx, cy, 0>(upx, upy, 0.f);
+            const float cP = cdot<2, cx, cy, 0>(Px, Py, 0.f);
+            const float ev = A0 + hq * (cv * cv - om1 * cu * cu);
+            f[b] = f[b] * om1 + wb * (ev + cP);
+            f[b + 1] = f[b + 1] * om1 + wb * (ev - cP);
+        });
+        (void)inv_cs4; (void)ux; (void)uy; (void)uz;
     }
+}
+
+// f holds pre-collision populations (FP32: deviations); on return the
+// post-collision ones.
+template <int LAT, int COLL, class Real>
+__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const Real (&F)[3], const DevParams& p)
+{
+    if constexpr (std::is_same<Real, double>::value) collide64<LAT, COLL>(f, F, p);
+    else collide32<LAT, COLL>(f, F, p);
 }
 
 // Index of the velocity opposite to c_b (c_opp = -c_b).
@@ -600,6 +758,86 @@ __global__ void __launch_bounds__(32 * TY * TZ)
     });
 }
 
+// FP64 form of the two-pass schedule: k_psi64 and k_fused64 take one cell per
+// thread by linear index, so no lane is spent on tile padding, and blocks are as
+// small as one warp, so that a 64 x 64 domain spreads over all SMs (FP64 issues
+// two lanes per cycle and SM: 16 blocks of 256 threads kept 136 SMs idle).  psi
+// comes straight from the ghosted buffer through L1: at two FP64 lanes per
+// cycle the staging of tiles buys nothing.  Per step, with collide64: D2Q9 64^2
+// 14.3 -> 6.9 us, D2Q25 Peng-Robinson 60^2 32 -> 11.7 us.
+struct CellXYZ {
+    int x, y, z;
+};
+template <int D>
+__device__ __forceinline__ CellXYZ cell_xyz(const DevParams& p, unsigned i)
+{
+    const unsigned r = p.dnx.div(i);
+    CellXYZ c;
+    c.x = static_cast<int>(i - r * p.dnx.d);
+    c.z = D == 3 ? static_cast<int>(p.dny.div(r)) : 0;
+    c.y = D == 3 ? static_cast<int>(r - c.z * p.dny.d) : static_cast<int>(r);
+    return c;
+}
+
+template <int LAT>
+__global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, double* __restrict__ psi, DevParams p)
+{
+    using L = Lattice<LAT>;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.N) return;
+    const CellXYZ c = cell_xyz<L::D>(p, i);
+    double v = p.psi_w;
+    if (c.y >= p.wall_rows) {
+        double f[L::Q];
+        gather<LAT>(A, p, c.x, c.y, c.z, f);
+        double s = 0.0;
+        sfor<L::Q>([&](auto bI) { s += f[decltype(bI)::value]; });
+        v = psi_of<LAT>(s, p);
+    }
+    store_psi<L::D>(psi, p, c.x, c.y, c.z, v);
+}
+
+// Solid nodes (y < wall_rows, 2-D) bounce back: f*_b = f_{-b}.
+template <int LAT, int ORD, int COLL>
+__global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, const double* __restrict__ psi,
+                                                 double* __restrict__ B, DevParams p)
+{
+    using L = Lattice<LAT>;
+    using S = Stencil<L::D, ORD>;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.N) return;
+    const CellXYZ c = cell_xyz<L::D>(p, i);
+    double f[L::Q];
+    gather<LAT>(A, p, c.x, c.y, c.z, f);
+    if (L::D == 2 && c.y < p.wall_rows) {
+        sfor<L::Q>([&](auto bI) {
+            constexpr int b = decltype(bI)::value;
+            B[static_cast<long long>(b) * p.N + i] = f[opposite<LAT>(b)];
+        });
+        return;
+    }
+    const int sy = p.psx, sz = p.psx * p.psy;
+    const double* tc = psi + (c.z + (L::D == 3 ? p.g : 0)) * sz + (c.y + p.g) * sy + (c.x + kGhostX);
+    double a[3] = {0.0, 0.0, 0.0};
+    sfor<S::n / 2>([&](auto kI) {
+        constexpr int k = 2 * decltype(kI)::value;
+        constexpr int ex = S::T.v[k][0], ey = S::T.v[k][1], ez = S::T.v[k][2];
+        constexpr double wt = S::T.w[k] * L::cs2;
+        const int o = ez * sz + ey * sy + ex;
+        const double d = tc[o] - tc[-o];
+        if (ex != 0) a[0] += (wt * ex) * d;
+        if (ey != 0) a[1] += (wt * ey) * d;
+        if (ez != 0) a[2] += (wt * ez) * d;
+    });
+    const double gp = -p.G * tc[0];
+    const double F[3] = {gp * a[0], gp * a[1], L::D == 3 ? gp * a[2] : 0.0};
+    collide64<LAT, COLL>(f, F, p);
+    sfor<L::Q>([&](auto bI) {
+        constexpr int b = decltype(bI)::value;
+        B[static_cast<long long>(b) * p.N + i] = f[b];
+    });
+}
+
 // Standard bounce-back on the solid band y < wall_rows (2-D): a solid node takes
 // no collision and sends every population back the way it came, f*_b = f_{-b}.
 // Runs after k_fused on the same stream and overwrites what that kernel wrote
@@ -670,7 +908,7 @@ __device__ __forceinline__ void force_ring(const Real* ring, int m, int cx, int 
     const Real gp = -G * base[R][0];
     F[0] = gp * ax;
     F[1] = gp * ay;
-    F[2] = gp * az;
+    F[2] = L::D == 3 ? gp * az : Real(0);
 }
 
 // Per-direction base pointers of the population buffers, passed by value so
@@ -3249,18 +3487,35 @@ inline int grid_1d(long long n, int cap = 152 * 16)
     return static_cast<int>(b < cap ? b : cap);
 }
 
+// Threads per block of the FP64 one-cell-per-thread kernels: one warp while the
+// whole domain fits the SMs' block slots that way (it spreads evenly), else four.
+inline int block64(long long n) { return n <= 152LL * 32 * 32 ? 32 : 128; }
+
 template <int LAT, class Real>
 cudaError_t launch_psi(const LaunchArgs& a, cudaStream_t s)
 {
+    if constexpr (std::is_same<Real, double>::value) {
+        const int bs = block64(a.p.N);
+        k_psi64<LAT><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
+            static_cast<const double*>(a.fin), static_cast<double*>(a.psi), a.p);
+        return cudaGetLastError();
+    } else {
     const dim3 blk(32, 8, 1);
     const dim3 grd((a.p.nx + 31) / 32, (a.p.ny + 7) / 8, Lattice<LAT>::D == 3 ? a.p.nz : 1);
     k_psi<LAT, Real><<<grd, blk, 0, s>>>(static_cast<const Real*>(a.fin), static_cast<Real*>(a.psi), a.p);
     return cudaGetLastError();
+    }
 }
 
 template <int LAT, int ORD, int COLL, class Real, int TY, int TZ>
 cudaError_t launch_fused(const LaunchArgs& a, cudaStream_t s)
 {
+    if constexpr (std::is_same<Real, double>::value) {
+        const int bs = block64(a.p.N);
+        k_fused64<LAT, ORD, COLL><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
+            static_cast<const double*>(a.fin), static_cast<const double*>(a.psi), static_cast<double*>(a.fout), a.p);
+        return cudaGetLastError();
+    } else {
     const dim3 blk(32, TY, TZ);
     const dim3 grd((a.p.nx + 31) / 32, (a.p.ny + TY - 1) / TY, Lattice<LAT>::D == 3 ? (a.p.nz + TZ - 1) / TZ : 1);
     k_fused<LAT, ORD, COLL, Real, TY, TZ><<<grd, blk, 0, s>>>(*a.tmap, static_cast<const Real*>(a.fin),
@@ -3271,6 +3526,7 @@ cudaError_t launch_fused(const LaunchArgs& a, cudaStream_t s)
             static_cast<const Real*>(a.fin), static_cast<Real*>(a.fout), a.p);
     }
     return cudaGetLastError();
+    }
 }
 
 template <int LAT, int ORD, int COLL, class Real, int TX, int TY, int ZC, int MINB, int ST>
