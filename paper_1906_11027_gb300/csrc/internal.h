@@ -157,21 +157,39 @@ cudaError_t launch_mean(const double* x, long long n, double* partials, int nblo
 // completes, through the step kernels' bounded wait, and sets kErrTimeout in *err.
 cudaError_t launch_wait_probe(unsigned* err, cudaStream_t s);
 
-// Warm-start network (mlp.cu): evaluates the network's density at T signed
-// distances evenly spaced over [-dmax, dmax] for (G, tau, order, R) into table_dev.
-// The network's distance input spans |d| <= kMlpDmax.
+// Warm-start network (mlp.cu): the network's density at T signed distances evenly
+// spaced over [-dmax, dmax] for (G, tau, order, r_in * R_dev[c]), c < ncand, into
+// tables_dev[c][T], on stream s.  The network's distance input spans |d| <= kMlpDmax.
 constexpr double kMlpDmax = 24.0;
 }  // namespace lbm
 struct lbm_mlp;
 namespace lbm {
-int mlp_profile_table(lbm_mlp* n, double G, double tau, double order, double R, int T, double dmax,
-                      float* table_dev);
+cudaError_t mlp_profile_tables(const lbm_mlp* n, double G, double tau, double order, const double* R_dev, double r_in,
+                               int ncand, int T, double dmax, float* tables_dev, cudaStream_t s);
 
-// Density field from a radial profile table (reduce.cu): rho0(cell) = table(r - R)
-// with r the periodic distance to the centre node, linear interpolation, clamped.
-cudaError_t launch_field_from_table(const DevParams& p, int dim, const float* table, int T, double dmax, double R,
-                                    double* rho0, cudaStream_t s);
-cudaError_t launch_add_constant(double* x, long long n, double c, cudaStream_t s);
+// Mass-matching search of the learned start (reduce.cu), kept on the device: a
+// radius bracket halved two times per round from three candidates, the midpoint
+// and the midpoints of both halves, so the halvings follow the plain bisection.
+struct RadiusSearch {
+    double cand[3];   // radii the next tables are made for (first round: the bracket's ends)
+    double lo, hi, mlo;
+    double m0;        // mean density to match
+    double Re, mm;    // last radius taken and its mean
+    int last;         // its candidate index
+    int ok;           // bracket valid and every mean finite
+    int round;        // 0: the bracket itself
+    unsigned done;    // blocks finished (last one updates)
+};
+// *st := start of a search over [lo, hi] for the mean res[0] (device).
+cudaError_t launch_search_start(RadiusSearch* st, const double* res, double lo, double hi, cudaStream_t s);
+// Means of the fields of the current candidates' tables, then one update of *st.
+// partials: 3 * (number of blocks) doubles of the reduction scratch.
+cudaError_t launch_search_round(const DevParams& p, int dim, const float* tables, int T, double dmax,
+                                RadiusSearch* st, double* partials, int nblocks_max, cudaStream_t s);
+// rho0(cell) = table(r - R_e) + (m0 - mm) with r the periodic distance to the
+// centre node, linear interpolation, clamped.
+cudaError_t launch_search_field(const DevParams& p, int dim, const float* tables, int T, double dmax,
+                                const RadiusSearch* st, double* rho0, cudaStream_t s);
 
 // Per-lattice lookup (defined in kernels_<lattice>.cu). Returns false if the
 // combination is not instantiated.

@@ -81,46 +81,155 @@ __device__ __forceinline__ double centre_offset(int i, int n)
     return d;
 }
 
-__global__ void k_field_from_table(DevParams p, int dim, const float* __restrict__ table, int T, double dmax,
-                                   double R, double* __restrict__ rho0)
+// Periodic distance of cell i to the centre node.
+__device__ __forceinline__ double centre_distance(const DevParams& p, int dim, long long i)
 {
+    const unsigned c = static_cast<unsigned>(i);
+    const unsigned r = p.dnx.div(c);
+    const int x = static_cast<int>(c - r * p.dnx.d);
+    const int z = dim == 3 ? static_cast<int>(p.dny.div(r)) : 0;
+    const int y = static_cast<int>(r) - z * p.ny;
+    const double dx = centre_offset(x, p.nx), dy = centre_offset(y, p.ny);
+    const double dz = dim == 3 ? centre_offset(z, p.nz) : 0.0;
+    return sqrt(dx * dx + dy * dy + dz * dz);
+}
+
+__device__ __forceinline__ double table_density(const float* __restrict__ table, int T, double dmax, double d)
+{
+    d = fmin(fmax(d, -dmax), dmax);
+    const double u = (d + dmax) / (2.0 * dmax) * (T - 1);
+    int k = static_cast<int>(floor(u));
+    if (k > T - 2) k = T - 2;
+    const double a = u - k;
+    return (1.0 - a) * static_cast<double>(table[k]) + a * static_cast<double>(table[k + 1]);
+}
+
+__global__ void k_search_start(RadiusSearch* st, const double* res, double lo, double hi)
+{
+    RadiusSearch s{};
+    s.cand[0] = lo;
+    s.cand[1] = hi;
+    s.cand[2] = hi;
+    s.lo = lo;
+    s.hi = hi;
+    s.m0 = res[0];
+    s.ok = 1;
+    *st = s;
+}
+
+__device__ void search_update(RadiusSearch& s, const double (&m)[3])
+{
+    if (s.round == 0) {
+        s.mlo = m[0];
+        s.ok = isfinite(m[0]) && isfinite(m[1]) && (m[0] - s.m0) * (m[1] - s.m0) < 0.0;
+    } else if (s.ok) {
+        int k = 0;
+        for (int it = 0; it < 2 && s.ok; ++it) {
+            s.Re = s.cand[k];
+            s.mm = m[k];
+            s.last = k;
+            if (!isfinite(s.mm)) {
+                s.ok = 0;
+            } else if ((s.mm - s.m0) * (s.mlo - s.m0) > 0.0) {
+                s.lo = s.Re;
+                s.mlo = s.mm;
+                k = 2;
+            } else {
+                s.hi = s.Re;
+                k = 1;
+            }
+        }
+    }
+    ++s.round;
+    s.cand[0] = 0.5 * (s.lo + s.hi);
+    s.cand[1] = 0.5 * (s.lo + s.cand[0]);
+    s.cand[2] = 0.5 * (s.cand[0] + s.hi);
+}
+
+// Block sums of the candidates' fields (the sums of k_block_sums on a stored
+// field, without the field); the last block adds the blocks in their order and
+// updates the search, so a round is two launches and no host read.  Bounded by
+// the FP64 distance and interpolation of 3 candidates per cell, whose distance
+// is formed once.
+__global__ void __launch_bounds__(256) k_search_round(DevParams p, int dim, const float* __restrict__ tables, int T,
+                                                      double dmax, RadiusSearch* st, double* partials)
+{
+    __shared__ double sh[256];
+    __shared__ bool is_last;
+    const double R[3] = {st->cand[0], st->cand[1], st->cand[2]};
+    const int nc = st->round == 0 ? 2 : 3;
+    double acc[3] = {0.0, 0.0, 0.0};
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < p.N;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int x = static_cast<int>(i % p.nx);
-        const long long r = i / p.nx;
-        const int y = static_cast<int>(r % p.ny);
-        const int z = static_cast<int>(r / p.ny);
-        const double dx = centre_offset(x, p.nx), dy = centre_offset(y, p.ny);
-        const double dz = dim == 3 ? centre_offset(z, p.nz) : 0.0;
-        double d = sqrt(dx * dx + dy * dy + dz * dz) - R;
-        d = fmin(fmax(d, -dmax), dmax);
-        const double u = (d + dmax) / (2.0 * dmax) * (T - 1);
-        int k = static_cast<int>(floor(u));
-        if (k > T - 2) k = T - 2;
-        const double a = u - k;
-        rho0[i] = (1.0 - a) * static_cast<double>(table[k]) + a * static_cast<double>(table[k + 1]);
+        const double r = centre_distance(p, dim, i);
+        for (int c = 0; c < nc; ++c) acc[c] += table_density(tables + c * T, T, dmax, r - R[c]);
+    }
+    auto tree = [&](double v) {
+        __syncthreads();
+        sh[threadIdx.x] = v;
+        __syncthreads();
+        for (int s = 128; s > 0; s >>= 1) {
+            if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+            __syncthreads();
+        }
+        return sh[0];
+    };
+    for (int c = 0; c < nc; ++c) {
+        const double v = tree(acc[c]);
+        if (threadIdx.x == 0) partials[static_cast<long long>(c) * gridDim.x + blockIdx.x] = v;
+    }
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    double m[3] = {0.0, 0.0, 0.0};
+    for (int c = 0; c < nc; ++c) {
+        double a = 0.0;
+        for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += 256)
+            a += __ldcg(partials + static_cast<long long>(c) * gridDim.x + b);
+        m[c] = tree(a) / static_cast<double>(p.N);
+    }
+    if (threadIdx.x == 0) {
+        RadiusSearch s = *st;
+        search_update(s, m);
+        s.done = 0;
+        *st = s;
     }
 }
 
-__global__ void k_add_constant(double* __restrict__ x, long long n, double c)
+__global__ void k_search_field(DevParams p, int dim, const float* __restrict__ tables, int T, double dmax,
+                               const RadiusSearch* __restrict__ st, double* __restrict__ rho0)
 {
-    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+    const double R = st->Re, shift = st->m0 - st->mm;
+    const float* table = tables + st->last * T;
+    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < p.N;
          i += static_cast<long long>(gridDim.x) * blockDim.x)
-        x[i] += c;
+        rho0[i] = table_density(table, T, dmax, centre_distance(p, dim, i) - R) + shift;
 }
 
-cudaError_t launch_field_from_table(const DevParams& p, int dim, const float* table, int T, double dmax, double R,
-                                    double* rho0, cudaStream_t s)
+cudaError_t launch_search_start(RadiusSearch* st, const double* res, double lo, double hi, cudaStream_t s)
 {
-    const long long nb = (p.N + 255) / 256;
-    k_field_from_table<<<static_cast<int>(nb < 2432 ? nb : 2432), 256, 0, s>>>(p, dim, table, T, dmax, R, rho0);
+    k_search_start<<<1, 1, 0, s>>>(st, res, lo, hi);
     return cudaGetLastError();
 }
 
-cudaError_t launch_add_constant(double* x, long long n, double c, cudaStream_t s)
+cudaError_t launch_search_round(const DevParams& p, int dim, const float* tables, int T, double dmax,
+                                RadiusSearch* st, double* partials, int nblocks_max, cudaStream_t s)
 {
-    const long long nb = (n + 255) / 256;
-    k_add_constant<<<static_cast<int>(nb < 2432 ? nb : 2432), 256, 0, s>>>(x, n, c);
+    long long nb = (p.N + 255) / 256;
+    if (nb > nblocks_max) nb = nblocks_max;
+    k_search_round<<<static_cast<int>(nb), 256, 0, s>>>(p, dim, tables, T, dmax, st, partials);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_search_field(const DevParams& p, int dim, const float* tables, int T, double dmax,
+                                const RadiusSearch* st, double* rho0, cudaStream_t s)
+{
+    const long long nb = (p.N + 255) / 256;
+    k_search_field<<<static_cast<int>(nb < 2432 ? nb : 2432), 256, 0, s>>>(p, dim, tables, T, dmax, st, rho0);
     return cudaGetLastError();
 }
 
