@@ -133,6 +133,7 @@ struct lbm_ctx {
     int cur;      // index of the buffer holding the current state
     void* psi;
     size_t psi_bytes;
+    double* rho;  // FP64: density written by the psi kernel for the collision
     double* partials;
     double* res;
     unsigned* err;
@@ -175,12 +176,13 @@ struct lbm_ctx {
     {
         LaunchArgs a{};
         a.p = dp;
-        finish_params(a.p, li.cs2);
+        finish_params(a.p);
         a.fin = buf[cur];
         a.fout = buf[cur ^ 1];
         a.carry_in = carry[cur];
         a.carry_out = carry[cur ^ 1];
         a.psi = psi;
+        a.rho = rho;
         a.tmap = &tmap;
         a.partials = partials;
         a.nblocks_max = kNBlocksMax;
@@ -546,11 +548,12 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     c->buf[0] = c->dalloc(fbytes);
     c->buf[1] = c->dalloc(fbytes);
     c->psi = c->dalloc(c->psi_bytes);
+    if (!fp32) c->rho = static_cast<double*>(c->dalloc(sizeof(double) * c->N));
     c->partials = static_cast<double*>(c->dalloc(sizeof(double) * kNBlocksMax * kObsWidth));
     c->res_len = kResLine + p->nx + 8;
     c->res = static_cast<double*>(c->dalloc(sizeof(double) * c->res_len));
     c->err = static_cast<unsigned*>(c->dalloc(256));
-    if (!c->buf[0] || !c->buf[1] || !c->psi || !c->partials || !c->res || !c->err)
+    if (!c->buf[0] || !c->buf[1] || !c->psi || (!fp32 && !c->rho) || !c->partials || !c->res || !c->err)
         return cleanup(fail(LBM_ENOMEM, "device allocation of %zu bytes failed", 2 * fbytes + c->psi_bytes));
     if (cudaMallocHost(&c->host_res, sizeof(double) * c->res_len) != cudaSuccess)
         return cleanup(fail(LBM_ENOMEM, "pinned host allocation failed"));
@@ -578,6 +581,8 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     if (p->psi == LBM_PSI_PENG_ROBINSON) {
         d.pr_T = p->T_over_Tc * pr_critical_temperature();
         d.pr_alpha = pr_alpha(p->T_over_Tc);
+        d.pr_K = 2.0 / (p->G * li.cs2);
+        d.pr_aa = kPrA * d.pr_alpha;
     }
     d.rate[0] = 1.0 / p->tau;
     d.rate[1] = p->s_e;
@@ -621,6 +626,7 @@ int lbm_destroy(lbm_ctx* c)
     c->dfree(c->carry[0]);
     c->dfree(c->carry[1]);
     c->dfree(c->psi);
+    c->dfree(c->rho);
     c->dfree(c->partials);
     c->dfree(c->res);
     c->dfree(c->err);

@@ -40,7 +40,7 @@ struct BatchDom {
     long long poff;  // element offset of the domain in the psi scratch field (two-pass shape)
     double G, omega, pref, rho_bar;
     float G_f, omega_f, pref_f, rho_bar_f;  // FP32 copies (set with the doubles on the host)
-    double kV[2], kP[2];                    // FP64 collision products (finish_params)
+    Coll64 c64;                             // FP64 collision products
 };
 
 __device__ __forceinline__ DevParams dom_params(const BatchDom& d)
@@ -58,10 +58,7 @@ __device__ __forceinline__ DevParams dom_params(const BatchDom& d)
     p.omega_f = d.omega_f;
     p.pref_f = d.pref_f;
     p.rho_bar_f = d.rho_bar_f;
-    p.kV[0] = d.kV[0];
-    p.kV[1] = d.kV[1];
-    p.kP[0] = d.kP[0];
-    p.kP[1] = d.kP[1];
+    p.c64 = d.c64;
     p.psi_kind = 0;
     return p;
 }
@@ -105,8 +102,7 @@ __device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, co
         Real* dst = ring + ring_slot(m, NS) * E;
         Real f[Q];
         gather_off<kLatD2Q9, Real, RE>(P, ixo, mo, zero, f);
-        Real s = Real(0);
-        sfor<Q>([&](auto bI) { s += f[decltype(bI)::value]; });
+        const Real s = sum_f<kLatD2Q9>(f);
         dst[tid + R] = psi_of<kLatD2Q9>(std::is_same<Real, float>::value ? Real(p.rho_bar) + s : s, p);
         Real* st = stash + static_cast<unsigned>(m + 4 * NST) % NST * (Q * TX) + tid;
         sfor<Q>([&](auto bI) {
@@ -116,8 +112,7 @@ __device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, co
         if (has_halo) {
             Real h[Q];
             gather_off<kLatD2Q9, Real, RE>(P, hxo, mo, zero, h);
-            Real sh = Real(0);
-            sfor<Q>([&](auto bI) { sh += h[decltype(bI)::value]; });
+            const Real sh = sum_f<kLatD2Q9>(h);
             dst[hex] = psi_of<kLatD2Q9>(std::is_same<Real, float>::value ? Real(p.rho_bar) + sh : sh, p);
         }
     };
@@ -133,8 +128,8 @@ __device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, co
                 constexpr int b = decltype(bI)::value;
                 f[b] = st[b * TX];
             });
-            Real F[3];
-            force_ring<kLatD2Q9, ORD, Real, EX, E, NS>(ring, m, tid + R, 0, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<kLatD2Q9, ORD, Real, EX, E, NS>(ring, m, tid + R, 0, F);
             collide<kLatD2Q9, 0>(f, F, p);
             const int c = m * p.nx + ix;
             sfor<Q>([&](auto bI) {
@@ -274,8 +269,8 @@ __device__ __forceinline__ void batch_item_seg(const float* __restrict__ A, floa
         if (active) {
             float f[Q];
             load_cell(stage_of(m), tid, f);
-            float F[3];
-            force_ring<kLatD2Q9, ORD, float, EX, EX, NS>(ring, m, tid + R, 0, p.G_f, F);
+            ForceSum<float> F;
+            force_ring<kLatD2Q9, ORD, float, EX, EX, NS>(ring, m, tid + R, 0, F);
             collide<kLatD2Q9, 0>(f, F, p);
             const long long c = static_cast<long long>(m) * p.nx + x0 + tid;
             sfor<Q>([&](auto bI) {
@@ -332,25 +327,19 @@ __global__ void __launch_bounds__(TX + 32) k_batch_step_seg(const BatchDom* __re
 // results are bitwise the same) and collides.  Work item = 256 consecutive cells
 // of one domain.
 template <int ORD, class Real>
-__device__ __forceinline__ void force_global(const Real* __restrict__ psi, int nx, int ny, int x, int y, Real G,
-                                             Real (&F)[3])
+__device__ __forceinline__ void force_global(const Real* __restrict__ psi, int nx, int ny, int x, int y,
+                                             ForceSum<Real>& F)
 {
-    using L = Lattice<kLatD2Q9>;
     using S = Stencil<2, ORD>;
-    Real ax = Real(0), ay = Real(0);
+    F = ForceSum<Real>{};
     sfor<S::n / 2>([&](auto kI) {
         constexpr int a = 2 * decltype(kI)::value;
         constexpr int ex = S::T.v[a][0], ey = S::T.v[a][1];
-        constexpr double wt = S::T.w[a] * L::cs2;
         const Real d = psi[wrap_near(y + ey, ny) * nx + wrap_near(x + ex, nx)] -
                        psi[wrap_near(y - ey, ny) * nx + wrap_near(x - ex, nx)];
-        if (ex != 0) ax += Real(wt * ex) * d;
-        if (ey != 0) ay += Real(wt * ey) * d;
+        force_add<kLatD2Q9, ORD, a>(F, d);
     });
-    const Real gp = -G * psi[y * nx + x];
-    F[0] = gp * ax;
-    F[1] = gp * ay;
-    F[2] = Real(0);
+    F.psi = psi[y * nx + x];
 }
 
 template <class Real>
@@ -368,8 +357,7 @@ __global__ void __launch_bounds__(256) k_batch_psi2(const BatchDom* __restrict__
         const int x = static_cast<int>(i % p.nx), y = static_cast<int>(i / p.nx);
         Real f[kQ9];
         gather<kLatD2Q9>(pool_in + d.off, p, x, y, 0, f);
-        Real s = Real(0);
-        sfor<kQ9>([&](auto bI) { s += f[decltype(bI)::value]; });
+        const Real s = sum_f<kLatD2Q9>(f);
         psi_pool[d.poff + i] = psi_of<kLatD2Q9>(std::is_same<Real, float>::value ? Real(p.rho_bar) + s : s, p);
     }
 }
@@ -381,8 +369,8 @@ __device__ __forceinline__ void fused2_cell(const Real* __restrict__ A, const Re
     const int x = static_cast<int>(i % p.nx), y = static_cast<int>(i / p.nx);
     Real f[kQ9];
     gather<kLatD2Q9>(A, p, x, y, 0, f);
-    Real F[3];
-    force_global<ORD, Real>(psi, p.nx, p.ny, x, y, par<Real>(p.G, p.G_f), F);
+    ForceSum<Real> F;
+    force_global<ORD, Real>(psi, p.nx, p.ny, x, y, F);
     collide<kLatD2Q9, 0>(f, F, p);
     sfor<kQ9>([&](auto bI) {
         constexpr int b = decltype(bI)::value;
@@ -1011,10 +999,11 @@ int lbm_batch_create(const lbm_params* ps, const double* init, int n, lbm_batch*
         dp.omega = m.omega;
         dp.pref = m.pref;
         dp.G = m.G;
-        finish_params(dp, Lattice<kLatD2Q9>::cs2);
-        for (int k = 0; k < 2; ++k) {
-            m.kV[k] = dp.kV[k];
-            m.kP[k] = dp.kP[k];
+        switch (m.order) {
+        case 4: m.c64 = fill_c64<kLatD2Q9, 4, 0>(dp); break;
+        case 6: m.c64 = fill_c64<kLatD2Q9, 6, 0>(dp); break;
+        case 8: m.c64 = fill_c64<kLatD2Q9, 8, 0>(dp); break;
+        default: m.c64 = fill_c64<kLatD2Q9, 10, 0>(dp); break;
         }
         off += (long long)kQ9 * p.nx * p.ny;
         off = (off + 63) / 64 * 64;  // 256-byte aligned domains

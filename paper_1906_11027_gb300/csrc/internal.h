@@ -40,6 +40,18 @@ inline FastDiv make_fast_div(unsigned d)
     return {d, static_cast<unsigned>((p + d - 1) / d), 31 + l};
 }
 
+// Parameter products of the FP64 collision (collide64), formed once per launch on
+// the host.  w: weight of the lattice's largest shell, w1: first force weight
+// times c_s^2 (the force sums come divided by it).
+struct Coll64 {
+    double g, gh;    // -G w1, half of it
+    double k0, k1;   // w omega / (2 c_s^2), -G w1 w pref / c_s^2
+    double w, omega, om1;  // w, omega, 1 - omega
+    double kb, kj;   // exact difference: w / c_s^2, w (1 - omega) / c_s^2
+    double hT;       // exact difference: w / (2 c_s^2)
+    double dmn[19];  // MRT: (omega - s_k) / |M_k|^2
+};
+
 // Runtime constants of one domain, passed by value to every kernel.
 struct DevParams {
     int nx, ny, nz;
@@ -65,25 +77,16 @@ struct DevParams {
     float omega_f, pref_f, rho_bar_f, G_f;
     float om1_f;  // 1 - omega, rounded once from double
     float dmrt_f[4];
-    // FP64 collision and psi: products of parameters with powers of the
-    // lattice's c_s^2, formed once per domain instead of once per cell.
-    double kV[2];  // V = kV[0] (j + F/2) + kV[1] F  with (omega/2, pref) / c_s^4
-    double kP[2];  // P = kP[0] (j + F/2) + kP[1] F  with (omega, pref) / c_s^2
     double pr_K;   // Peng-Robinson psi: 2 / (G c_s^2) and a alpha
     double pr_aa;
+    Coll64 c64;        // FP64 collision products, set by the launchers (fill_c64)
     FastDiv dnx, dny;  // for x, y, z of a linear cell index
 };
 
-// Fills the derived fields of p from the others (cs2: the lattice's c_s^2); call
-// after any change to omega, pref, rho_bar, G or rate.
-__host__ __device__ inline void finish_params(DevParams& p, double cs2)
+// Fills the derived fields of p from the others; call after any change to
+// omega, pref, rho_bar, G or rate.
+__host__ __device__ inline void finish_params(DevParams& p)
 {
-    p.kV[0] = 0.5 * p.omega / (cs2 * cs2);
-    p.kV[1] = p.pref / (cs2 * cs2);
-    p.kP[0] = p.omega / cs2;
-    p.kP[1] = p.pref / cs2;
-    p.pr_K = 2.0 / (p.G * cs2);
-    p.pr_aa = kPrA * p.pr_alpha;
     for (int c = 0; c < 4; ++c) {
         p.dmrt[c] = (c == 0) ? 0.0 : p.omega - p.rate[c];
         p.dmrt_f[c] = static_cast<float>(p.dmrt[c]);
@@ -105,6 +108,7 @@ struct LaunchArgs {
     double* partials;      // reduction scratch
     int nblocks_max;       // capacity of partials (blocks)
     double* res;           // reduction result (see api.cu for the slots)
+    double* rho;           // density of every cell (FP64 two-pass schedule)
     double* dbuf0;         // double work buffers (N or Q*N)
     double* dbuf1;
     int mode;              // init profile: 0 droplet, 1 flat

@@ -174,8 +174,97 @@ __device__ __forceinline__ void gather(const Real* __restrict__ A, const DevPara
     });
 }
 
+// sum_b f_b.  FP64 takes the opposite pairs, the order every FP64 kernel shares;
+// the one-cell-per-thread FP32 kernels add in index order.
+template <int LAT, class Real>
+__device__ __forceinline__ Real sum_f(const Real (&f)[Lattice<LAT>::Q])
+{
+    constexpr int Q = Lattice<LAT>::Q;
+    if constexpr (std::is_same<Real, double>::value) {
+        Real s = f[0];
+        sfor<(Q - 1) / 2>([&](auto kI) {
+            constexpr int b = 1 + 2 * decltype(kI)::value;
+            s += f[b] + f[b + 1];
+        });
+        return s;
+    } else {
+        Real s = Real(0);
+        sfor<Q>([&](auto bI) { s += f[decltype(bI)::value]; });
+        return s;
+    }
+}
+
 // ---- psi -------------------------------------------------------------------------
-__device__ __forceinline__ double psi_exp(double r) { return -expm1(-r); }
+// 1 - exp(-j/64) and exp(-j/64) to the last bit, for psi_exp below: powers of
+// exp(-1/64) in double-double arithmetic, evaluated by the compiler.
+struct DD {
+    double h, l;
+};
+constexpr DD dd_sum(double a, double b)  // |a| >= |b|
+{
+    const double s = a + b;
+    return {s, b - (s - a)};
+}
+constexpr DD dd_mul(DD a, DD b)
+{
+    auto split = [](double v) {  // Dekker: v = hi + lo with 26-bit halves
+        const double t = 134217729.0 * v;
+        const double hi = t - (t - v);
+        return DD{hi, v - hi};
+    };
+    const DD x = split(a.h), y = split(b.h);
+    const double p = a.h * b.h;
+    const double e = ((x.h * y.h - p) + x.h * y.l + x.l * y.h) + x.l * y.l;
+    return dd_sum(p, e + (a.h * b.l + a.l * b.h));
+}
+struct ExpTable {
+    double2 v[1024];  // {exp(-j/64), 1 - exp(-j/64)}
+};
+constexpr ExpTable make_exp_table()
+{
+    // exp(-1/64) = 1 - (1/64)(1 - (1/64)/2 (1 - (1/64)/3 (...))): 1/n to double-double
+    DD q{1.0, 0.0};
+    for (int n = 14; n >= 1; --n) {
+        const double r = 1.0 / (64.0 * n);
+        // 1/(64 n) - r, exactly rounded: r n 64 = 1 + tiny
+        DD inv{r, 0.0};
+        const DD rn = dd_mul(inv, DD{64.0 * n, 0.0});
+        inv.l = ((1.0 - rn.h) - rn.l) * r;
+        const DD t = dd_mul(q, inv);
+        const DD u = dd_sum(1.0, -t.h);
+        q = dd_sum(u.h, u.l - t.l);
+    }
+    ExpTable T{};
+    DD e{1.0, 0.0};
+    for (int j = 0; j < 1024; ++j) {
+        const DD c = dd_sum(1.0, -e.h);
+        T.v[j].x = e.h;
+        T.v[j].y = c.h + (c.l - e.l);
+        e = dd_mul(e, q);
+    }
+    return T;
+}
+__device__ const ExpTable kExpTable = make_exp_table();
+
+// 1 - exp(-r).  Table and polynomial: r = j/64 + x, |x| <= 1/128,
+// 1 - exp(-r) = (1 - e_j) + e_j (1 - exp(-x)), the last factor by its Taylor
+// polynomial (next term 2^-54 of the value): 10 operations of the FP64 pipe where
+// expm1 takes 19 (D2Q9 psi pass at 2048^2: 0.24 -> 0.15 ms).
+__device__ __forceinline__ double psi_exp(double r)
+{
+    if (static_cast<unsigned>(__double2hiint(r)) >= 0x402f0000u) return -expm1(-r);  // not in [0, 15.5)
+    constexpr double magic = 6755399441055744.0;  // 1.5 * 2^52: the sum holds round(64 r) in its low word
+    const double t = fma(r, 64.0, magic);
+    const int j = __double2loint(t);
+    const double x = fma(t - magic, -1.0 / 64.0, r);
+    double c = fma(x, -1.0 / 720.0, 1.0 / 120.0);
+    c = fma(c, x, -1.0 / 24.0);
+    c = fma(c, x, 1.0 / 6.0);
+    c = fma(c, x, -0.5);
+    c = fma(c, x, 1.0);
+    const double2 e = __ldg(&kExpTable.v[j]);
+    return fma(e.x, c * x, e.y);
+}
 __device__ __forceinline__ float psi_exp(float r) { return -expm1f(-r); }
 
 // psi = sqrt(2 (p_EOS - c_s^2 rho) / (G c_s'^2)) with the Peng-Robinson EOS (Sec. 3).
@@ -235,27 +324,44 @@ __device__ __forceinline__ void store_psi(Real* __restrict__ psi, const DevParam
 }
 
 // ---- force (Eq. 1) from a psi view with compile-time strides -------------------
-template <int LAT, int ORD, class Real, int SX, int SY>
-__device__ __forceinline__ void force_from(const Real* tc, Real G, Real (&F)[3])
+// F = -G psi a: the stencil sum a and psi of the cell, kept apart.  In FP64 the
+// sum is divided by the first weight, whose product with G the host forms
+// (Coll64), which saves one multiplication per component.
+template <class Real>
+struct ForceSum {
+    Real a[3];
+    Real psi;
+};
+// Adds the pair (e_A, -e_A) with difference d = psi(x + e_A) - psi(x - e_A).  The axis
+// vectors lead each component, so theirs starts its sum.
+template <int LAT, int ORD, int A, class Real>
+__device__ __forceinline__ void force_add(ForceSum<Real>& F, Real d)
 {
-    using L = Lattice<LAT>;
-    using S = Stencil<L::D, ORD>;
+    using S = Stencil<Lattice<LAT>::D, ORD>;
+    constexpr bool k64 = std::is_same<Real, double>::value;
+    constexpr double w = k64 ? S::T.w[A] / S::T.w[0] : S::T.w[A] * Lattice<LAT>::cs2;  // c_s^2-scaled force weight
+    constexpr bool axis = S::T.v[A][0] * S::T.v[A][0] + S::T.v[A][1] * S::T.v[A][1] + S::T.v[A][2] * S::T.v[A][2] == 1;
+    sfor<3>([&](auto iI) {
+        constexpr int i = decltype(iI)::value;
+        constexpr int e = S::T.v[A][i];
+        if constexpr (k64 && axis && e == 1) F.a[i] = d;
+        else if constexpr (e != 0) F.a[i] += Real(w * e) * d;
+    });
+}
+
+template <int LAT, int ORD, class Real, int SX, int SY>
+__device__ __forceinline__ void force_from(const Real* tc, ForceSum<Real>& F)
+{
+    using S = Stencil<Lattice<LAT>::D, ORD>;
     // Opposite stencil vectors are adjacent: each pair contributes
     // w e (psi(x + e) - psi(x - e)).
-    Real ax = Real(0), ay = Real(0), az = Real(0);
+    F = ForceSum<Real>{};
     sfor<S::n / 2>([&](auto kI) {
         constexpr int a = 2 * decltype(kI)::value;
-        constexpr int ex = S::T.v[a][0], ey = S::T.v[a][1], ez = S::T.v[a][2];
-        constexpr double wt = S::T.w[a] * L::cs2;  // c_s^2-scaled force weight
-        const Real d = tc[(ez * SY + ey) * SX + ex] - tc[-((ez * SY + ey) * SX + ex)];
-        if (ex != 0) ax += Real(wt * ex) * d;
-        if (ey != 0) ay += Real(wt * ey) * d;
-        if (ez != 0) az += Real(wt * ez) * d;
+        constexpr int o = (S::T.v[a][2] * SY + S::T.v[a][1]) * SX + S::T.v[a][0];
+        force_add<LAT, ORD, a>(F, tc[o] - tc[-o]);
     });
-    const Real gp = -G * tc[0];
-    F[0] = gp * ax;
-    F[1] = gp * ay;
-    F[2] = L::D == 3 ? gp * az : Real(0);
+    F.psi = tc[0];
 }
 
 // ---- value helpers shared by the scalar and the packed-pair collision --------
@@ -265,6 +371,9 @@ __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ double vsub(double a, double b) { return a - b; }
 __device__ __forceinline__ float vsub(float a, float b) { return a - b; }
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ double vneg(double a) { return -a; }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ double vmul(double a, double b) { return a * b; }
 __device__ __forceinline__ float vmul(float a, float b) { return a * b; }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
@@ -287,6 +396,17 @@ __device__ __forceinline__ V macc(V acc, V x)
     else if constexpr (C == -1) return vsub(acc, x);
     else return vfma(vsplat<V>(double(C)), x, acc);
 }
+// C x + acc, or C x where nothing has been summed yet
+template <bool FIRST, int C, class V>
+__device__ __forceinline__ V macc1(V acc, V x)
+{
+    if constexpr (!FIRST) return macc<C>(acc, x);
+    else if constexpr (C == 0) return acc;
+    else if constexpr (C == 1) return x;
+    else if constexpr (C == -1) return vneg(x);
+    else return vmul(vsplat<V>(double(C)), x);
+}
+
 // A scalar parameter in the kernel's precision (FP32 kernels read the FP32 copy).
 template <class Real>
 __device__ __forceinline__ Real par(double d, float f)
@@ -309,10 +429,40 @@ __device__ __forceinline__ Real par(double d, float f)
 //   odd rows:  m_k(g) = m_k(f) - B_k.j/cs2
 // with v = j - F/2 (= rho u - F) and rho' = rho, or rho - rho_bar for FP32
 // deviations (whose m_k(f) lacks the rho_bar A_k of the stored offset).
-template <int LAT, class V>
+//
+// dm: omega - s per rate class (ND = 4), or that over |M_k|^2 per row (FP64, from
+// the host).  In FP64 a row that is constant on the shells takes the shells' sums,
+// which such rows share.
+template <int LAT>
+constexpr bool mrt_row_by_shell(int k)
+{
+    using L = Lattice<LAT>;
+    for (int b = 1; b < L::Q; ++b)
+        for (int q = 1; q < L::Q; ++q)
+            if (L::T.w[b] == L::T.w[q] && Mrt<LAT>::B.M[k][b] != Mrt<LAT>::B.M[k][q]) return false;
+    return true;
+}
+// first pair with a nonzero entry in row k
+template <int LAT>
+constexpr int first_pair(int k)
+{
+    for (int q = 0; q < (Lattice<LAT>::Q - 1) / 2; ++q)
+        if (Mrt<LAT>::B.M[k][2 * q + 1] != 0.0) return q;
+    return -1;
+}
+// first pair of pair n's shell
+template <int LAT>
+constexpr int shell_head(int n)
+{
+    for (int q = 0; q < n; ++q)
+        if (Lattice<LAT>::T.w[2 * q + 1] == Lattice<LAT>::T.w[2 * n + 1]) return q;
+    return n;
+}
+
+template <int LAT, class V, int ND>
 __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::Q - 1) / 2],
                                               const V (&D)[(Lattice<LAT>::Q - 1) / 2], V r0, const V (&j)[3],
-                                              const V (&u)[3], const V (&v)[3], const V (&dm)[4],
+                                              const V (&u)[3], const V (&v)[3], const V (&dm)[ND],
                                               V (&t)[Lattice<LAT>::Q])
 {
     using L = Lattice<LAT>;
@@ -321,10 +471,18 @@ __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::
     constexpr int NP = (Q - 1) / 2;
     constexpr int DIM = L::D;
     constexpr double cs2 = L::cs2;
+    constexpr bool k64 = std::is_same<V, double>::value;
     V uv = vmul(u[0], v[0]);
     uv = vfma(u[1], v[1], uv);
     if constexpr (DIM == 3) uv = vfma(u[2], v[2], uv);
     const V e0 = vfma(uv, vsplat<V>(-0.5 / cs2), r0);
+    V SS[NP];  // shell sums, at the shell's first pair
+    if constexpr (k64)
+        sfor<NP>([&](auto pI) {
+            constexpr int pp = decltype(pI)::value, h = shell_head<LAT>(pp);
+            if constexpr (h == pp) SS[pp] = P[pp];
+            else SS[h] = vadd(SS[h], P[pp]);
+        });
     sfor<Q>([&](auto kI) {
         constexpr int k = decltype(kI)::value;
         constexpr int rc = MB::B.rate_class[k];
@@ -335,12 +493,19 @@ __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::
             if constexpr (par_k > 0) {
                 constexpr int m0 = static_cast<int>(MB::B.M[k][0]);
                 static_assert(double(m0) == MB::B.M[k][0], "integer basis");
-                m = macc<m0>(m, f0);
+                m = macc1<true, m0>(m, f0);
+                constexpr bool by_shell = k64 && mrt_row_by_shell<LAT>(k);
+                constexpr int first = first_pair<LAT>(k);
                 sfor<NP>([&](auto pI) {
                     constexpr int pp = decltype(pI)::value;
                     constexpr int mk = static_cast<int>(MB::B.M[k][2 * pp + 1]);
                     static_assert(double(mk) == MB::B.M[k][2 * pp + 1], "integer basis");
-                    m = macc<mk>(m, P[pp]);
+                    constexpr bool f1 = m0 == 0 && pp == first;
+                    if constexpr (by_shell) {
+                        if constexpr (shell_head<LAT>(pp) == pp) m = macc1<f1, mk>(m, SS[pp]);
+                    } else {
+                        m = macc1<f1, mk>(m, P[pp]);
+                    }
                 });
                 constexpr double A = MB::T.A[k];
                 if constexpr (A != 0.0) m = vfma(vsplat<V>(-A), e0, m);
@@ -353,11 +518,12 @@ __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::
                     });
                 });
             } else {
+                constexpr int first = first_pair<LAT>(k);
                 sfor<NP>([&](auto pI) {
                     constexpr int pp = decltype(pI)::value;
                     constexpr int mk = static_cast<int>(MB::B.M[k][2 * pp + 1]);
                     static_assert(double(mk) == MB::B.M[k][2 * pp + 1], "integer basis");
-                    m = macc<mk>(m, D[pp]);
+                    m = macc1<pp == first, mk>(m, D[pp]);
                 });
                 sfor<DIM>([&](auto iI) {
                     constexpr int i = decltype(iI)::value;
@@ -365,8 +531,12 @@ __device__ __forceinline__ void mrt_moments_g(V f0, const V (&P)[(Lattice<LAT>::
                     if constexpr (bc != 0.0) m = vfma(vsplat<V>(-bc / cs2), j[i], m);
                 });
             }
-            constexpr double inv_norm = MB::B.inv_norm[k];
-            t[k] = vmul(dm[rc], vmul(vsplat<V>(inv_norm), m));
+            if constexpr (ND == 4) {
+                constexpr double inv_norm = MB::B.inv_norm[k];
+                t[k] = vmul(dm[rc], vmul(vsplat<V>(inv_norm), m));
+            } else {
+                t[k] = vmul(dm[k], m);
+            }
         }
     });
 }
@@ -418,24 +588,142 @@ __device__ __forceinline__ V cdot(V vx, V vy, V vz)
 }
 
 // ---- collision in FP64 --------------------------------------------------------
-// Same update as collide() below, arranged for the FP64 pipe, which issues two
-// lanes per cycle and SM and bounds every FP64 step: no term that the lattice
-// lacks (z on 2-D lattices, zero velocity components), the even part of all
-// velocities from one symmetric tensor, and parameter products from the host.
-//   Guo:   w_b [ A0 + c.T.c +- c.P ], T_ij = sym(u_i V_j), A0 = omega rho - c_s^2 tr T,
-//          V = (omega/2 (j + F/2) + pref F) / c_s^4, P = (omega (j + F/2) + pref F) / c_s^2
-//   exact difference, a = j, b = j + F:
-//          T_ij = (b_i b_j - (1 - omega) a_i a_j) / (2 rho c_s^4), P = (b - (1 - omega) a) / c_s^2
-// With k_psi64 / k_fused64 below, per step: D2Q9 BGK 2048^2 1.24 -> 0.94 ms, D2Q9 MRT
-// 256^2 39 -> 27 us; error against 64-bit arithmetic of the same step unchanged.
-template <int LAT, int COLL>
-__device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const double (&F)[3], const DevParams& p)
+// Same update as collide32() below, arranged for the FP64 pipe: one operation of
+// a warp holds it for 19 cycles (64 on one sub-partition alone), whatever lanes are
+// active, so the operation count is the time.  Left out or folded away: terms that the lattice
+// lacks, sums that start at zero, products of parameters (Coll64, from the host),
+// powers of two (exponent arithmetic on the integer pipe), and at omega = 1 (the
+// paper's tau = 1) the old population.  Everything carries the factor w of the
+// largest shell; shell ratio r = w_b / w:
+//   Guo:   f*_b = (1 - omega) f_b + r [ A0 + c.T.c / c_s^2 +- c.P ],  v = j + F/2, u = v / rho,
+//          V = w (omega/2 v + pref F) / c_s^2, P = V + w omega/2 v / c_s^2,
+//          T_ij = sym(u_i V_j), A0 = w (omega rho) - tr T
+//   exact difference, b = j + F:
+//          T_ij = w (b_i b_j - (1 - omega) j_i j_j) / (2 rho c_s^2), P = w (b - (1 - omega) j) / c_s^2
+// Error against 64-bit arithmetic of the same steps: as before (4e-16 to 2e-15 after
+// 130 steps on every lattice and collision).
+
+// x * 2^K on the integer pipe.  Zero, a result below 2^-1022 (to zero), infinities
+// and NaN are kept apart.
+template <int K>
+__device__ __forceinline__ double scale2(double x)
+{
+    if constexpr (K == 0) return x;
+    const int hi = __double2hiint(x);
+    const int e = hi & 0x7ff00000;
+    const bool live = K < 0 ? e > (-K << 20) : e != 0;
+    int h = live ? hi + K * (1 << 20) : hi & 0x80000000;
+    int lo = live ? __double2loint(x) : 0;
+    const bool big = K < 0 ? e == 0x7ff00000 : e >= 0x7ff00000 - (K << 20);
+    if (big) {
+        h = K > 0 && e != 0x7ff00000 ? (hi & 0x80000000) | 0x7ff00000 : hi;
+        lo = K > 0 && e != 0x7ff00000 ? 0 : __double2loint(x);
+    }
+    return __hiloint2double(h, lo);
+}
+// x * r for a compile-time r
+constexpr int log2_of(double r)
+{
+    for (int k = -8; k <= 8; ++k)
+        if (r == (k < 0 ? 1.0 / double(1 << (k < 0 ? -k : 0)) : double(1 << (k < 0 ? 0 : k)))) return k;
+    return 99;
+}
+// weight of shell b over the largest shell's
+template <int LAT>
+constexpr double base_weight()
+{
+    using L = Lattice<LAT>;
+    double best = 0.0;
+    int most = 0;
+    for (int b = 1; b < L::Q; ++b) {
+        int n = 0;
+        for (int k = 1; k < L::Q; ++k) n += L::T.w[k] == L::T.w[b];
+        if (n > most) {
+            most = n;
+            best = L::T.w[b];
+        }
+    }
+    return best;
+}
+// w_b / w.  The ratios are multiples of 1/32, so they are exact.  The rest
+// velocity's, where it is no power of two, closes the sum: w (r_0 + sum r_b) is the
+// sum of the table's weights although w itself is rounded, or the mass would
+// drift by that rounding every step.
+// (second term: what r_0 itself loses by rounding).
+template <int LAT>
+constexpr DD weight_ratio2(int b)
+{
+    using L = Lattice<LAT>;
+    auto at = [](int k) {
+        const double q = 32.0 * (L::T.w[k] / base_weight<LAT>());
+        return static_cast<double>(static_cast<long long>(q + 0.5)) / 32.0;
+    };
+    const double r = at(b);
+    if (b > 0 || log2_of(r) != 99) return DD{r, 0.0};
+    constexpr double w = base_weight<LAT>();
+    double others = 0.0;
+    DD sum{L::T.w[0], 0.0};
+    for (int k = 1; k < L::Q; ++k) {
+        others += at(k);
+        const DD s = dd_sum(sum.h, L::T.w[k]);  // the running sum is the larger term from w_0 on (Q >= 13)
+        sum = DD{s.h, sum.l + s.l};
+    }
+    const double inv = 1.0 / w;
+    const DD x = dd_mul(DD{inv, 0.0}, DD{w, 0.0});
+    return dd_sum(inv - others, (((sum.h - x.h) - x.l) + sum.l) * inv);
+}
+template <int LAT>
+constexpr double weight_ratio(int b)
+{
+    return weight_ratio2<LAT>(b).h;
+}
+
+template <int LAT, int ORD, int COLL>
+Coll64 fill_c64(const DevParams& p)
+{
+    constexpr double cs2 = Lattice<LAT>::cs2, w = base_weight<LAT>();
+    constexpr double w1 = Stencil<Lattice<LAT>::D, ORD>::T.w[0] * cs2;
+    Coll64 c{};
+    c.g = -p.G * w1;
+    c.gh = 0.5 * c.g;
+    c.k0 = w * p.omega / (2.0 * cs2);
+    c.k1 = c.g * w * p.pref / cs2;
+    c.w = w;
+    c.omega = p.omega;
+    c.om1 = 1.0 - p.omega;
+    c.kb = w / cs2;
+    c.kj = w * c.om1 / cs2;
+    c.hT = 0.5 * w / cs2;
+    if constexpr (COLL == 1)
+        for (int k = 0; k < Lattice<LAT>::Q; ++k)
+            c.dmn[k] = p.dmrt[Mrt<LAT>::B.rate_class[k]] * Mrt<LAT>::B.inv_norm[k];
+    return c;
+}
+template <int LAT, int ORD, int COLL>
+DevParams params64(DevParams p)
+{
+    p.c64 = fill_c64<LAT, ORD, COLL>(p);
+    return p;
+}
+
+// First MRT row of a parity (k < 0: none) with a nonzero entry at velocity b.
+template <int LAT>
+constexpr int mrt_first(int b, int parity)
+{
+    for (int k = 0; k < Lattice<LAT>::Q; ++k)
+        if (Mrt<LAT>::B.rate_class[k] != 0 && Mrt<LAT>::T.parity[k] == parity && Mrt<LAT>::B.M[k][b] != 0.0) return k;
+    return -1;
+}
+
+template <int LAT, int COLL, bool ONE>
+__device__ __forceinline__ void collide64_at(double (&f)[Lattice<LAT>::Q], const ForceSum<double>& F, double rho,
+                                             const DevParams& p)
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q, D = L::D, NP = (Q - 1) / 2;
-    constexpr double cs2 = L::cs2;
-    double s = f[0];
-    double j[D] = {};
+    constexpr double ics2 = 1.0 / L::cs2;
+    const Coll64& c = p.c64;
+    double j[D];
     double Pp[COLL == 1 ? NP : 1], Dp[COLL == 1 ? NP : 1];
     sfor<NP>([&](auto kI) {
         constexpr int k = decltype(kI)::value;
@@ -443,47 +731,57 @@ __device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const do
         static_assert(L::T.v[b + 1][0] == -L::T.v[b][0] && L::T.v[b + 1][1] == -L::T.v[b][1] &&
                           L::T.v[b + 1][2] == -L::T.v[b][2],
                       "opposite velocities must be adjacent");
-        const double sum = f[b] + f[b + 1], d = f[b] - f[b + 1];
+        static_assert(k >= D || (L::T.v[b][k] == 1 && L::T.w[b] == L::T.w[1]), "the unit vectors lead");
+        const double d = f[b] - f[b + 1];
         if constexpr (COLL == 1) {
-            Pp[k] = sum;
+            Pp[k] = f[b] + f[b + 1];
             Dp[k] = d;
         }
-        s += sum;
-        sfor<D>([&](auto iI) {
-            constexpr int i = decltype(iI)::value;
-            j[i] = macc<L::T.v[b][i]>(j[i], d);
-        });
+        if constexpr (k < D) j[k] = d;
+        else
+            sfor<D>([&](auto iI) {
+                constexpr int i = decltype(iI)::value;
+                j[i] = macc<L::T.v[b][i]>(j[i], d);
+            });
     });
-    const double rho = s;
     const double inv_rho = 1.0 / rho;
-    double T[D], S[3] = {}, P[D];  // T_ii; S: 2 T_xy, 2 T_xz, 2 T_yz; P
+    double T[D], S[3] = {}, P[D];  // T_ii; T_xy, T_xz, T_yz (Guo: their symmetric sums); P
+    constexpr double s2 = COLL == 2 ? 2.0 * ics2 : ics2;  // factor of S in c.T.c / c_s^2
     double t[COLL == 1 ? Q : 1];
     if constexpr (COLL == 2) {
-        const double om1 = 1.0 - p.omega;
-        const double h = inv_rho * (0.5 / (cs2 * cs2));
+        const double h = inv_rho * c.hT;
+        const double gp = c.g * F.psi;
         double a1[D], b[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            b[i] = j[i] + F[i];
-            a1[i] = om1 * j[i];
-            P[i] = (b[i] - a1[i]) * (1.0 / cs2);
-            T[i] = h * fma(b[i], b[i], -(a1[i] * j[i]));
+            b[i] = fma(gp, F.a[i], j[i]);
+            if constexpr (ONE) {
+                P[i] = c.kb * b[i];
+                T[i] = h * (b[i] * b[i]);
+            } else {
+                a1[i] = c.om1 * j[i];
+                P[i] = c.kb * (b[i] - a1[i]);
+                T[i] = h * fma(b[i], b[i], -(a1[i] * j[i]));
+            }
         }
-        const double h2 = 2.0 * h;
-        S[0] = h2 * fma(b[0], b[1], -(a1[0] * j[1]));
+        auto off = [&](int i, int k) {
+            if constexpr (ONE) return h * (b[i] * b[k]);
+            else return h * fma(b[i], b[k], -(a1[i] * j[k]));
+        };
+        S[0] = off(0, 1);
         if constexpr (D == 3) {
-            S[1] = h2 * fma(b[0], b[2], -(a1[0] * j[2]));
-            S[2] = h2 * fma(b[1], b[2], -(a1[1] * j[2]));
+            S[1] = off(0, 2);
+            S[2] = off(1, 2);
         }
     } else {
-        double u[D], V[D];
-        double v[D];
+        double u[D], V[D], v[D];
+        const double gp = c.gh * F.psi, kp = c.k1 * F.psi;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            v[i] = fma(0.5, F[i], j[i]);
+            v[i] = fma(gp, F.a[i], j[i]);
             u[i] = v[i] * inv_rho;
-            V[i] = fma(p.kV[0], v[i], p.kV[1] * F[i]);
-            P[i] = fma(p.kP[0], v[i], p.kP[1] * F[i]);
+            V[i] = fma(c.k0, v[i], kp * F.a[i]);
+            P[i] = fma(c.k0, v[i], V[i]);
             T[i] = u[i] * V[i];
         }
         S[0] = fma(u[0], V[1], u[1] * V[0]);
@@ -497,81 +795,109 @@ __device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const do
             for (int i = 0; i < D; ++i) {
                 jv[i] = j[i];
                 uv[i] = u[i];
-                vv[i] = fma(-0.5, F[i], j[i]);
+                vv[i] = fma(-gp, F.a[i], j[i]);
             }
-            mrt_moments_g<LAT, double>(f[0], Pp, Dp, rho, jv, uv, vv, p.dmrt, t);
+            mrt_moments_g<LAT, double, 19>(f[0], Pp, Dp, rho, jv, uv, vv, c.dmn, t);
         }
     }
     double tr = T[0] + T[1];
     if constexpr (D == 3) tr += T[2];
-    const double A0 = fma(p.omega, rho, -cs2 * tr);
-    // f*_b = (1 - omega) f_b + w_b (e_b +- o_b), and at omega = 1 (the paper's tau = 1)
-    // the first term is gone
-    auto update = [&](auto oneI) {
-        constexpr bool kOne = decltype(oneI)::value != 0;
-        const double om1 = 1.0 - p.omega;
-        auto relax = [&](double fb, double x) { return kOne ? x : fma(om1, fb, x); };
-        constexpr double w0 = L::T.w[0];
-        f[0] = relax(f[0], w0 * A0);
-        sfor<NP>([&](auto kI) {
-            constexpr int b = 1 + 2 * decltype(kI)::value;
-            constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
-            constexpr double wb = L::T.w[b];
-            double e = A0;
-            e = macc<cx * cx>(e, T[0]);
-            e = macc<cy * cy>(e, T[1]);
-            if constexpr (D == 3) e = macc<cz * cz>(e, T[2]);
-            e = macc<cx * cy>(e, S[0]);
-            if constexpr (D == 3) {
-                e = macc<cx * cz>(e, S[1]);
-                e = macc<cy * cz>(e, S[2]);
-            }
-            double o = cdot<D, cx, cy, cz>(P[0], P[1], P[D - 1]);
-            if constexpr (COLL == 1) {  // plus the moment correction, even and odd rows apart
-                double E, O;
-                mrt_pair<LAT, b>(t, E, O);
-                e = fma(wb, e, E);
-                o = fma(wb, o, O);
-                f[b] = relax(f[b], e + o);
-                f[b + 1] = relax(f[b + 1], e - o);
-            } else {
-                f[b] = relax(f[b], wb * (e + o));
-                f[b + 1] = relax(f[b + 1], wb * (e - o));
-            }
-        });
-        if constexpr (COLL == 1) {
-            double E, O;
-            mrt_pair<LAT, 0>(t, E, O);
-            f[0] += E;
-        }
+    // omega rho is rounded by itself: a rounded product w omega would leave the mass
+    // off by its error every step
+    const double A0 = fma(c.w, ONE ? rho : c.omega * rho, -tr);
+    auto relax = [&](double fb, double x) { return ONE ? x : fma(c.om1, fb, x); };
+    auto ratio = [&](auto bI, double x) {
+        constexpr double r = weight_ratio<LAT>(decltype(bI)::value);
+        constexpr int k = log2_of(r);
+        if constexpr (k != 99) return scale2<k>(x);
+        else return r * x;
     };
+    sfor<NP>([&](auto kI) {
+        constexpr int b = 1 + 2 * decltype(kI)::value;
+        constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
+        double e = A0;
+        if constexpr (cx != 0) e = fma(cx * cx * ics2, T[0], e);
+        if constexpr (cy != 0) e = fma(cy * cy * ics2, T[1], e);
+        if constexpr (cz != 0) e = fma(cz * cz * ics2, T[D - 1], e);
+        if constexpr (cx * cy != 0) e = fma(cx * cy * s2, S[0], e);
+        if constexpr (cx * cz != 0) e = fma(cx * cz * s2, S[1], e);
+        if constexpr (cy * cz != 0) e = fma(cy * cz * s2, S[2], e);
+        double o = cdot<D, cx, cy, cz>(P[0], P[1], P[D - 1]);
+        if constexpr (COLL == 1) {  // plus the moment correction, even and odd rows apart
+            double E = 0.0, O = 0.0;
+            constexpr int ke = mrt_first<LAT>(b, 1), ko = mrt_first<LAT>(b, -1);
+            sfor<Q>([&](auto qI) {
+                constexpr int k = decltype(qI)::value;
+                if constexpr (Mrt<LAT>::B.rate_class[k] != 0) {
+                    constexpr int mk = static_cast<int>(Mrt<LAT>::B.M[k][b]);
+                    if constexpr (Mrt<LAT>::T.parity[k] > 0) E = macc1<k == ke, mk>(E, t[k]);
+                    else O = macc1<k == ko, mk>(O, t[k]);
+                }
+            });
+            constexpr double r = weight_ratio<LAT>(b);
+            if constexpr (ke >= 0) e = r == 1.0 ? e + E : fma(r, e, E); else e = ratio(std::integral_constant<int, b>{}, e);
+            if constexpr (ko >= 0) o = r == 1.0 ? o + O : fma(r, o, O); else o = ratio(std::integral_constant<int, b>{}, o);
+            f[b] = relax(f[b], e + o);
+            f[b + 1] = relax(f[b + 1], e - o);
+        } else {
+            f[b] = relax(f[b], ratio(std::integral_constant<int, b>{}, e + o));
+            f[b + 1] = relax(f[b + 1], ratio(std::integral_constant<int, b>{}, e - o));
+        }
+    });
+    constexpr DD r0 = weight_ratio2<LAT>(0);
+    if constexpr (r0.l != 0.0) f[0] = relax(f[0], fma(r0.h, A0, r0.l * A0));
+    else f[0] = relax(f[0], ratio(std::integral_constant<int, 0>{}, A0));
+    if constexpr (COLL == 1) {
+        double E = 0.0;
+        constexpr int ke = mrt_first<LAT>(0, 1);
+        sfor<Q>([&](auto qI) {
+            constexpr int k = decltype(qI)::value;
+            if constexpr (Mrt<LAT>::B.rate_class[k] != 0 && Mrt<LAT>::T.parity[k] > 0)
+                E = macc1<k == ke, static_cast<int>(Mrt<LAT>::B.M[k][0])>(E, t[k]);
+        });
+        f[0] += E;
+    }
+}
+
+template <int LAT, int COLL>
+__device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const ForceSum<double>& F, double rho,
+                                          const DevParams& p)
+{
     if (p.omega == 1.0)
-        update(std::integral_constant<int, 1>{});
+        collide64_at<LAT, COLL, true>(f, F, rho, p);
     else
-        update(std::integral_constant<int, 0>{});
+        collide64_at<LAT, COLL, false>(f, F, rho, p);
 }
 
 // ---- collision in FP32 on deviations from w_b rho_bar (Eqs. 3-4) ------------------
-// Terms that vanish for the lattice (z on 2-D lattices, zero velocity components)
-// are left out at compile time: the compiler may not drop 0 * x by itself.
+// On 2-D lattices the z terms are left out at compile time (the compiler may not
+// drop 0 * x by itself); the other expressions keep the form and order that fix
+// their rounding.
 template <int LAT, int COLL>
-__device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const float (&F)[3], const DevParams& p)
+__device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const ForceSum<float>& Fs, const DevParams& p)
 {
     using L = Lattice<LAT>;
     constexpr int NP = (L::Q - 1) / 2;
     constexpr bool k3 = L::D == 3;
+    const float gp = -p.G_f * Fs.psi;
+    const float F[3] = {gp * Fs.a[0], gp * Fs.a[1], k3 ? gp * Fs.a[2] : 0.f};
+    auto dot = [](float cx, float vx, float cy, float vy, float cz, float vz) {
+        if constexpr (k3) return cx * vx + cy * vy + cz * vz;
+        else return cx * vx + cy * vy;
+    };
     // Moments through the opposite pairs (b, b+1): sum f and sum (f_b - f_b+1) c_b.
     float s = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
     float Pp[NP], Dp[NP];  // pair sums and differences (MRT)
     sfor<NP>([&](auto kI) {
         constexpr int b = 1 + 2 * decltype(kI)::value;
+        constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
         Pp[decltype(kI)::value] = f[b] + f[b + 1];
         s += Pp[decltype(kI)::value];
         const float d = f[b] - f[b + 1];
         Dp[decltype(kI)::value] = d;
-        jx = macc<L::T.v[b][0]>(jx, d);
-        jy = macc<L::T.v[b][1]>(jy, d);
-        jz = macc<L::T.v[b][2]>(jz, d);
+        if (cx != 0) jx += float(cx) * d;
+        if (cy != 0) jy += float(cy) * d;
+        if (cz != 0) jz += float(cz) * d;
     });
     const float rho = p.rho_bar_f + s;
     const float inv_rho = 1.f / rho;
@@ -582,20 +908,18 @@ __device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const flo
     const float inv_cs2 = float(1.0 / cs2);
     const float inv_cs4 = float(1.0 / (cs2 * cs2));
     const float half_inv_cs4 = float(0.5 / (cs2 * cs2));
+    const float usq = dot(ux, ux, uy, uy, uz, uz) * float(0.5 / cs2);
+    const float uF = dot(ux, F[0], uy, F[1], uz, F[2]);
     const float omega = p.omega_f;
+    const float pref = p.pref_f;
     if constexpr (COLL == 0 || COLL == 1) {
-        const float uxy = ux * ux + uy * uy;
-        const float usq = (k3 ? uxy + uz * uz : uxy) * float(0.5 / cs2);
-        const float uFxy = ux * F[0] + uy * F[1];
-        const float uF = k3 ? uFxy + uz * F[2] : uFxy;
-        const float pref = p.pref_f;
         // MRT: the moment-space correction is formed from the pre-collision state
         float t[L::Q];
         if constexpr (COLL == 1) {
             const float jv[3] = {jx, jy, jz};
             const float uv3[3] = {ux, uy, uz};
             const float vv[3] = {jx - 0.5f * F[0], jy - 0.5f * F[1], jz - 0.5f * F[2]};
-            mrt_moments_g<LAT, float>(f[0], Pp, Dp, s, jv, uv3, vv, p.dmrt_f, t);
+            mrt_moments_g<LAT, float, 4>(f[0], Pp, Dp, s, jv, uv3, vv, p.dmrt_f, t);
         }
         // omega feq_b + pref src_b regrouped (Eq. 4):
         //   w_b [ A0 + (c.u)(c.V) + c.P ],
@@ -616,13 +940,13 @@ __device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const flo
         sfor<NP>([&](auto kI) {
             constexpr int b = 1 + 2 * decltype(kI)::value;
             constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1], cz = L::T.v[b][2];
-            constexpr float wb = float(L::T.w[b]);
-            const float cu = cdot<L::D, cx, cy, cz>(ux, uy, uz);
-            const float cV = cdot<L::D, cx, cy, cz>(Vx, Vy, Vz);
-            const float cP = cdot<L::D, cx, cy, cz>(Px, Py, Pz);
+            constexpr double wb = L::T.w[b];
+            const float cu = dot(float(cx), ux, float(cy), uy, float(cz), uz);
+            const float cV = dot(float(cx), Vx, float(cy), Vy, float(cz), Vz);
+            const float cP = dot(float(cx), Px, float(cy), Py, float(cz), Pz);
             const float ev = cu * cV + A0;
-            f[b] = f[b] * om1 + wb * (ev + cP);
-            f[b + 1] = f[b + 1] * om1 + wb * (ev - cP);
+            f[b] = f[b] * om1 + float(wb) * (ev + cP);
+            f[b + 1] = f[b + 1] * om1 + float(wb) * (ev - cP);
         });
         if constexpr (COLL == 1) mrt_apply<LAT, float>(t, f);
         (void)half_inv_cs4;
@@ -647,24 +971,24 @@ __device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const flo
         sfor<NP>([&](auto kI) {
             constexpr int b = 1 + 2 * decltype(kI)::value;
             constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1];
-            constexpr float wb = float(L::T.w[b]);
-            const float cv = cdot<2, cx, cy, 0>(vx, vy, 0.f);
-            const float cu = cdot<2, cx, cy, 0>(upx, upy, 0.f);
-            const float cP = cdot<2, cx, cy, 0>(Px, Py, 0.f);
+            constexpr double wb = L::T.w[b];
+            const float cv = dot(float(cx), vx, float(cy), vy, 0.f, 0.f);
+            const float cu = dot(float(cx), upx, float(cy), upy, 0.f, 0.f);
+            const float cP = dot(float(cx), Px, float(cy), Py, 0.f, 0.f);
             const float ev = A0 + hq * (cv * cv - om1 * cu * cu);
-            f[b] = f[b] * om1 + wb * (ev + cP);
-            f[b + 1] = f[b + 1] * om1 + wb * (ev - cP);
+            f[b] = f[b] * om1 + float(wb) * (ev + cP);
+            f[b + 1] = f[b + 1] * om1 + float(wb) * (ev - cP);
         });
-        (void)inv_cs4; (void)ux; (void)uy; (void)uz;
+        (void)inv_cs4; (void)ux; (void)uy; (void)uz; (void)usq; (void)uF; (void)pref;
     }
 }
 
 // f holds pre-collision populations (FP32: deviations); on return the
 // post-collision ones.
 template <int LAT, int COLL, class Real>
-__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const Real (&F)[3], const DevParams& p)
+__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const ForceSum<Real>& F, const DevParams& p)
 {
-    if constexpr (std::is_same<Real, double>::value) collide64<LAT, COLL>(f, F, p);
+    if constexpr (std::is_same<Real, double>::value) collide64<LAT, COLL>(f, F, sum_f<LAT>(f), p);
     else collide32<LAT, COLL>(f, F, p);
 }
 
@@ -748,8 +1072,8 @@ __global__ void __launch_bounds__(32 * TY * TZ)
     }
     if (!active) return;
     const Real* tc = tile + ((tz + (D == 3 ? R : 0)) * SY + (ty + R)) * SX + (tx + kGhostX);
-    Real F[3];
-    force_from<LAT, ORD, Real, SX, SY>(tc, par<Real>(p.G, p.G_f), F);
+    ForceSum<Real> F;
+    force_from<LAT, ORD, Real, SX, SY>(tc, F);
     collide<LAT, COLL>(f, F, p);
     const long long c = cell_of(p, x, y, z);
     sfor<L::Q>([&](auto bI) {
@@ -763,8 +1087,11 @@ __global__ void __launch_bounds__(32 * TY * TZ)
 // small as one warp, so that a 64 x 64 domain spreads over all SMs (FP64 issues
 // two lanes per cycle and SM: 16 blocks of 256 threads kept 136 SMs idle).  psi
 // comes straight from the ghosted buffer through L1: at two FP64 lanes per
-// cycle the staging of tiles buys nothing.  Per step, with collide64: D2Q9 64^2
-// 14.3 -> 6.9 us, D2Q25 Peng-Robinson 60^2 32 -> 11.7 us.
+// cycle the staging of tiles buys nothing.  k_psi64 keeps the density for
+// k_fused64, whose BGK or exact-difference collision needs no sum then.  Per step, with
+// collide64: D2Q9 64^2 14.3 -> 5.7 us, D2Q25 Peng-Robinson 60^2 32 -> 10.3 us, D2Q9 MRT
+// 256^2 39 -> 22 us, D2Q9 2048^2 1.24 -> 0.58 ms (54 operations where there were 155 in
+// plain form, and 18 for psi where there were 32).
 struct CellXYZ {
     int x, y, z;
 };
@@ -780,7 +1107,8 @@ __device__ __forceinline__ CellXYZ cell_xyz(const DevParams& p, unsigned i)
 }
 
 template <int LAT>
-__global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, double* __restrict__ psi, DevParams p)
+__global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, double* __restrict__ psi,
+                                               double* __restrict__ rho, DevParams p)
 {
     using L = Lattice<LAT>;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -790,8 +1118,8 @@ __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, dou
     if (c.y >= p.wall_rows) {
         double f[L::Q];
         gather<LAT>(A, p, c.x, c.y, c.z, f);
-        double s = 0.0;
-        sfor<L::Q>([&](auto bI) { s += f[decltype(bI)::value]; });
+        const double s = sum_f<LAT>(f);
+        rho[i] = s;
         v = psi_of<LAT>(s, p);
     }
     store_psi<L::D>(psi, p, c.x, c.y, c.z, v);
@@ -800,7 +1128,7 @@ __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, dou
 // Solid nodes (y < wall_rows, 2-D) bounce back: f*_b = f_{-b}.
 template <int LAT, int ORD, int COLL>
 __global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, const double* __restrict__ psi,
-                                                 double* __restrict__ B, DevParams p)
+                                                 const double* __restrict__ rho, double* __restrict__ B, DevParams p)
 {
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;
@@ -818,20 +1146,14 @@ __global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, c
     }
     const int sy = p.psx, sz = p.psx * p.psy;
     const double* tc = psi + (c.z + (L::D == 3 ? p.g : 0)) * sz + (c.y + p.g) * sy + (c.x + kGhostX);
-    double a[3] = {0.0, 0.0, 0.0};
+    ForceSum<double> F{};
     sfor<S::n / 2>([&](auto kI) {
         constexpr int k = 2 * decltype(kI)::value;
-        constexpr int ex = S::T.v[k][0], ey = S::T.v[k][1], ez = S::T.v[k][2];
-        constexpr double wt = S::T.w[k] * L::cs2;
-        const int o = ez * sz + ey * sy + ex;
-        const double d = tc[o] - tc[-o];
-        if (ex != 0) a[0] += (wt * ex) * d;
-        if (ey != 0) a[1] += (wt * ey) * d;
-        if (ez != 0) a[2] += (wt * ez) * d;
+        const int o = S::T.v[k][2] * sz + S::T.v[k][1] * sy + S::T.v[k][0];
+        force_add<LAT, ORD, k>(F, tc[o] - tc[-o]);
     });
-    const double gp = -p.G * tc[0];
-    const double F[3] = {gp * a[0], gp * a[1], L::D == 3 ? gp * a[2] : 0.0};
-    collide64<LAT, COLL>(f, F, p);
+    F.psi = tc[0];
+    collide64<LAT, COLL>(f, F, rho[i], p);
     sfor<L::Q>([&](auto bI) {
         constexpr int b = decltype(bI)::value;
         B[static_cast<long long>(b) * p.N + i] = f[b];
@@ -885,7 +1207,7 @@ __device__ __forceinline__ int wrap_any(int i, int n)
 }
 
 template <int LAT, int ORD, class Real, int EX, int E, int NS>
-__device__ __forceinline__ void force_ring(const Real* ring, int m, int cx, int cy, Real G, Real (&F)[3])
+__device__ __forceinline__ void force_ring(const Real* ring, int m, int cx, int cy, ForceSum<Real>& F)
 {
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;
@@ -893,22 +1215,15 @@ __device__ __forceinline__ void force_ring(const Real* ring, int m, int cx, int 
     const Real* base[2 * R + 1];
 #pragma unroll
     for (int s = 0; s < 2 * R + 1; ++s) base[s] = ring + ring_slot(m - R + s, NS) * E + cy * EX + cx;
-    Real ax = Real(0), ay = Real(0), az = Real(0);
+    F = ForceSum<Real>{};
     sfor<S::n / 2>([&](auto kI) {
         constexpr int a = 2 * decltype(kI)::value;
         constexpr int ex = S::T.v[a][0], ey = S::T.v[a][1], ez = S::T.v[a][2];
         constexpr int dm = (L::D == 3) ? ez : ey;  // offset along the marching axis
         constexpr int dq = (L::D == 3) ? ey : 0;   // in-plane offset of the second axis
-        constexpr double wt = S::T.w[a] * L::cs2;
-        const Real d = base[dm + R][dq * EX + ex] - base[R - dm][-(dq * EX + ex)];
-        if (ex != 0) ax += Real(wt * ex) * d;
-        if (ey != 0) ay += Real(wt * ey) * d;
-        if (ez != 0) az += Real(wt * ez) * d;
+        force_add<LAT, ORD, a>(F, base[dm + R][dq * EX + ex] - base[R - dm][-(dq * EX + ex)]);
     });
-    const Real gp = -G * base[R][0];
-    F[0] = gp * ax;
-    F[1] = gp * ay;
-    F[2] = L::D == 3 ? gp * az : Real(0);
+    F.psi = base[R][0];
 }
 
 // Per-direction base pointers of the population buffers, passed by value so
@@ -1043,8 +1358,7 @@ __global__ void __launch_bounds__(TX * TY, MINB)
                 gather_off<LAT, Real, RE>(P, ixo, iyo, mo, fnxt);
             else
                 gather_off<LAT, Real, RE>(P, ixo, mo, zero, fnxt);
-            Real s = Real(0);
-            sfor<Q>([&](auto bI) { s += fnxt[decltype(bI)::value]; });
+            const Real s = sum_f<LAT>(fnxt);
             const Real rho = std::is_same<Real, float>::value ? Real(p.rho_bar) + s : s;
             dst[i_slot] = psi_of<LAT>(rho, p);
             if (kSmem) {
@@ -1061,8 +1375,7 @@ __global__ void __launch_bounds__(TX * TY, MINB)
                 gather_off<LAT, Real, RE>(P, hxo, hyo, mo, f);
             else
                 gather_off<LAT, Real, RE>(P, hxo, mo, zero, f);
-            Real s = Real(0);
-            sfor<Q>([&](auto bI) { s += f[decltype(bI)::value]; });
+            const Real s = sum_f<LAT>(f);
             const Real rho = std::is_same<Real, float>::value ? Real(p.rho_bar) + s : s;
             dst[h_slot] = psi_of<LAT>(rho, p);
         }
@@ -1095,8 +1408,8 @@ __global__ void __launch_bounds__(TX * TY, MINB)
                 else
                     gather_off<LAT, Real, RE>(P, ixo, mo, zero, fcur);
             }
-            Real F[3];
-            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, F);
             collide<LAT, COLL>(fcur, F, p);
             const int c = m * mscale + cell_xy;
             sfor<Q>([&](auto bI) {
@@ -1266,8 +1579,8 @@ __global__ void __launch_bounds__(NX * TY + (PROD ? 32 : 0), 1)
         if (issuer)
             for (; next <= last && next <= m + R + NSTG; ++next) issue(next);
         if (active) {
-            Real F[3];
-            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, ty + R, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, ty + R, F);
             collide<LAT, COLL>(fcur, F, p);
             const int c = m * plane + cell_xy;
             sfor<Q>([&](auto bI) {
@@ -1448,8 +1761,8 @@ __global__ void __launch_bounds__(NX * TY + 32, 1)
             // after the item's last slab the next item's first slabs start loading
             if (producer) issue_upto(consumed);
             if (active) {
-                Real F[3];
-                force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, ty + R, par<Real>(p.G, p.G_f), F);
+                ForceSum<Real> F;
+                force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, ty + R, F);
                 collide<LAT, COLL>(fcur, F, p);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
@@ -1599,8 +1912,8 @@ __global__ void __launch_bounds__(TX + 32, 1)
         if (active) {
             Real f[Q];
             load_cell(stage_of(m), tid, f);
-            Real F[3];
-            force_ring<LAT, ORD, Real, EX, EX, NS>(ring, m, tid + R, 0, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, EX, NS>(ring, m, tid + R, 0, F);
             collide<LAT, COLL>(f, F, p);
             const int c = m * p.nx + x0 + tid;
             sfor<Q>([&](auto bI) {
@@ -1747,8 +2060,8 @@ __global__ void __launch_bounds__(TX * TY, MINB)
                 constexpr int b = decltype(bI)::value;
                 f[b] = fi[b * NT];
             });
-            Real F[3];
-            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, F);
             collide<LAT, COLL>(f, F, p);
             const int c = m * mscale + cell_xy;
             sfor<Q>([&](auto bI) {
@@ -1890,8 +2203,8 @@ __global__ void __launch_bounds__(TX * TY, MINB)
                 constexpr int b = decltype(bI)::value;
                 f[b] = st[b * NT];
             });
-            Real F[3];
-            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, par<Real>(p.G, p.G_f), F);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, E, NS>(ring, m, tx + R, (D == 3) ? ty + R : 0, F);
             collide<LAT, COLL>(f, F, p);
             const int c = m * mscale + cell_xy;
             sfor<Q>([&](auto bI) {
@@ -1977,7 +2290,7 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
         const float2 uv3[3] = {ux, uy, uz};
         const float2 vv[3] = {fma2(p2(-0.5f), F[0], jx), fma2(p2(-0.5f), F[1], jy), fma2(p2(-0.5f), F[2], jz)};
         const float2 dm[4] = {p2(p.dmrt_f[0]), p2(p.dmrt_f[1]), p2(p.dmrt_f[2]), p2(p.dmrt_f[3])};
-        mrt_moments_g<LAT, float2>(f[0], Pp, Dp, s, jv, uv3, vv, dm, t);
+        mrt_moments_g<LAT, float2, 4>(f[0], Pp, Dp, s, jv, uv3, vv, dm, t);
     }
     const float2 usq = k3 ? mul2(fma2(ux, ux, fma2(uy, uy, mul2(uz, uz))), p2(float(0.5 / cs2)))
                           : mul2(fma2(ux, ux, mul2(uy, uy)), p2(float(0.5 / cs2)));
@@ -3497,7 +3810,7 @@ cudaError_t launch_psi(const LaunchArgs& a, cudaStream_t s)
     if constexpr (std::is_same<Real, double>::value) {
         const int bs = block64(a.p.N);
         k_psi64<LAT><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
-            static_cast<const double*>(a.fin), static_cast<double*>(a.psi), a.p);
+            static_cast<const double*>(a.fin), static_cast<double*>(a.psi), a.rho, a.p);
         return cudaGetLastError();
     } else {
     const dim3 blk(32, 8, 1);
@@ -3513,7 +3826,8 @@ cudaError_t launch_fused(const LaunchArgs& a, cudaStream_t s)
     if constexpr (std::is_same<Real, double>::value) {
         const int bs = block64(a.p.N);
         k_fused64<LAT, ORD, COLL><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
-            static_cast<const double*>(a.fin), static_cast<const double*>(a.psi), static_cast<double*>(a.fout), a.p);
+            static_cast<const double*>(a.fin), static_cast<const double*>(a.psi), a.rho,
+            static_cast<double*>(a.fout), params64<LAT, ORD, COLL>(a.p));
         return cudaGetLastError();
     } else {
     const dim3 blk(32, TY, TZ);
@@ -3542,7 +3856,8 @@ cudaError_t launch_onepass(const LaunchArgs& a, cudaStream_t s)
     const int nm = k3 ? a.p.nz : a.p.ny;
     const long long nblocks = static_cast<long long>(ntx) * nty * ((nm + ZC - 1) / ZC);
     const auto P = make_pops<Real, Lattice<LAT>::Q>(a.fin, a.fout, a.p.N);
-    kern<<<static_cast<unsigned>(nblocks), TX * TY, dyn, s>>>(P, a.p, ntx, nty);
+    kern<<<static_cast<unsigned>(nblocks), TX * TY, dyn, s>>>(
+        P, std::is_same<Real, double>::value ? params64<LAT, ORD, COLL>(a.p) : a.p, ntx, nty);
     return cudaGetLastError();
 }
 
