@@ -133,7 +133,7 @@ struct lbm_ctx {
     int cur;      // index of the buffer holding the current state
     void* psi;
     size_t psi_bytes;
-    double* rho;  // FP64: density written by the psi kernel for the collision
+    double* rho;  // FP64: density written by the psi kernel for the collision (in psi's allocation)
     double* partials;
     double* res;
     unsigned* err;
@@ -141,7 +141,7 @@ struct lbm_ctx {
     size_t res_len;
     CUtensorMap tmap;
     KernelSet ks;
-    DevParams dp;
+    DevParams64 dp;
     int64_t step;
     cudaGraphExec_t graph;
     bool graph_valid;
@@ -547,13 +547,15 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     const size_t fbytes = (size_t)li.Q * c->N * c->elem;
     c->buf[0] = c->dalloc(fbytes);
     c->buf[1] = c->dalloc(fbytes);
-    c->psi = c->dalloc(c->psi_bytes);
-    if (!fp32) c->rho = static_cast<double*>(c->dalloc(sizeof(double) * c->N));
+    // psi and, in FP64, the density after it
+    const size_t psi_room = (c->psi_bytes + 255) / 256 * 256;
+    c->psi = c->dalloc(fp32 ? c->psi_bytes : psi_room + sizeof(double) * c->N);
+    if (c->psi && !fp32) c->rho = reinterpret_cast<double*>(static_cast<char*>(c->psi) + psi_room);
     c->partials = static_cast<double*>(c->dalloc(sizeof(double) * kNBlocksMax * kObsWidth));
     c->res_len = kResLine + p->nx + 8;
     c->res = static_cast<double*>(c->dalloc(sizeof(double) * c->res_len));
     c->err = static_cast<unsigned*>(c->dalloc(256));
-    if (!c->buf[0] || !c->buf[1] || !c->psi || (!fp32 && !c->rho) || !c->partials || !c->res || !c->err)
+    if (!c->buf[0] || !c->buf[1] || !c->psi || !c->partials || !c->res || !c->err)
         return cleanup(fail(LBM_ENOMEM, "device allocation of %zu bytes failed", 2 * fbytes + c->psi_bytes));
     if (cudaMallocHost(&c->host_res, sizeof(double) * c->res_len) != cudaSuccess)
         return cleanup(fail(LBM_ENOMEM, "pinned host allocation failed"));
@@ -563,7 +565,7 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
         cudaMemsetAsync(c->err, 0, 256, c->stream) != cudaSuccess)
         return cleanup(fail(LBM_ECUDA, "memset failed"));
 
-    DevParams& d = c->dp;
+    DevParams64& d = c->dp;
     d.nx = p->nx;
     d.ny = p->ny;
     d.nz = nz;
@@ -626,7 +628,6 @@ int lbm_destroy(lbm_ctx* c)
     c->dfree(c->carry[0]);
     c->dfree(c->carry[1]);
     c->dfree(c->psi);
-    c->dfree(c->rho);
     c->dfree(c->partials);
     c->dfree(c->res);
     c->dfree(c->err);

@@ -43,9 +43,10 @@ struct BatchDom {
     Coll64 c64;                             // FP64 collision products
 };
 
-__device__ __forceinline__ DevParams dom_params(const BatchDom& d)
+template <class Real>
+__device__ __forceinline__ typename ParamsOf<Real>::T dom_params(const BatchDom& d)
 {
-    DevParams p{};
+    typename ParamsOf<Real>::T p{};
     p.nx = d.nx;
     p.ny = d.ny;
     p.nz = 1;
@@ -58,15 +59,75 @@ __device__ __forceinline__ DevParams dom_params(const BatchDom& d)
     p.omega_f = d.omega_f;
     p.pref_f = d.pref_f;
     p.rho_bar_f = d.rho_bar_f;
-    p.c64 = d.c64;
+    if constexpr (std::is_same<Real, double>::value) p.c64 = d.c64;
     p.psi_kind = 0;
     return p;
+}
+
+// Operations with their rounding spelled out (the compiler may not contract them),
+// on one cell or a packed pair of cells.
+__device__ __forceinline__ float xadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float xmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float xfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float xrcp(float a) { return __frcp_rn(a); }  // = 1.f / a
+__device__ __forceinline__ float2 xadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 xmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 xfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 xrcp(float2 a) { return make_float2(xrcp(a.x), xrcp(a.y)); }
+
+// D2Q9 BGK collision on FP32 deviations: collide32's expressions with every rounding
+// fixed, so that all FP32 shapes, one cell or two per thread, give the same bits.
+// a: force sums of ForceSum, psi of the cell(s).
+template <class V>
+__device__ __forceinline__ void collide_batch(V (&f)[kQ9], V ax, V ay, V psi, const DevParams& p)
+{
+    auto c = [](float v) { return vsplat<V>(v); };
+    auto sub = [&](V u, V v) { return xadd(u, vneg(v)); };
+    const V gp = xmul(c(-p.G_f), psi);
+    const V Fx = xmul(gp, ax), Fy = xmul(gp, ay);
+    V s = f[0];
+    const V d1 = sub(f[1], f[2]), d2 = sub(f[3], f[4]), d3 = sub(f[5], f[6]), d4 = sub(f[7], f[8]);
+#pragma unroll
+    for (int b = 1; b < kQ9; b += 2) s = xadd(s, xadd(f[b], f[b + 1]));
+    const V jx = xadd(xadd(d1, d3), d4), jy = sub(xadd(d2, d3), d4);
+    const V rho = xadd(c(p.rho_bar_f), s);
+    const V inv = xrcp(rho);
+    const V ux = xmul(xfma(c(0.5f), Fx, jx), inv), uy = xmul(xfma(c(0.5f), Fy, jy), inv);
+    constexpr double cs2 = Lattice<kLatD2Q9>::cs2;
+    const V ic2 = c(static_cast<float>(1.0 / cs2)), ic4 = c(static_cast<float>(1.0 / (cs2 * cs2)));
+    const V om = c(p.omega_f), pref = c(p.pref_f), om1 = c(__fadd_rn(1.f, -p.omega_f));
+    const V usq = xmul(xfma(ux, ux, xmul(uy, uy)), c(static_cast<float>(0.5 / cs2)));
+    const V uF = xfma(ux, Fx, xmul(uy, Fy));
+    const V orho = xmul(om, rho);
+    const V nq = xmul(xmul(c(-1.f), orho), usq);
+    const V A0 = xfma(xmul(xmul(c(-1.f), pref), uF), ic2, xfma(om, s, nq));
+    const V Px = xmul(xfma(pref, Fx, xmul(orho, ux)), ic2), Py = xmul(xfma(pref, Fy, xmul(orho, uy)), ic2);
+    const V h = xmul(c(0.5f), orho);
+    const V Vx = xmul(xfma(pref, Fx, xmul(h, ux)), ic4), Vy = xmul(xfma(pref, Fy, xmul(h, uy)), ic4);
+    const V w0 = c(static_cast<float>(4.0 / 9.0)), w1 = c(static_cast<float>(1.0 / 9.0)),
+            w2 = c(static_cast<float>(1.0 / 36.0));
+    f[0] = xfma(f[0], om1, xmul(w0, A0));
+    auto pair = [&](int b, V cu, V cV, V cP, V w) {
+        const V e = xfma(cu, cV, A0);
+        f[b] = xfma(f[b], om1, xmul(w, xadd(e, cP)));
+        f[b + 1] = xfma(f[b + 1], om1, xmul(w, sub(e, cP)));
+    };
+    pair(1, ux, Vx, Px, w1);
+    pair(3, uy, Vy, Py, w1);
+    pair(5, xadd(ux, uy), xadd(Vx, Vy), xadd(Px, Py), w2);
+    pair(7, sub(ux, uy), sub(Vx, Vy), sub(Px, Py), w2);
+}
+template <class Real>
+__device__ __forceinline__ void collide_any(Real (&f)[kQ9], const ForceSum<Real>& F, const typename ParamsOf<Real>::T& p)
+{
+    if constexpr (std::is_same<Real, float>::value) collide_batch<float>(f, F.a[0], F.a[1], F.psi, p);
+    else collide<kLatD2Q9, 0>(f, F, p);
 }
 
 // One (tile, chunk) of one domain: the 2-D one-pass march with a shared-memory
 // stash.  ring: [NS][EX] psi, stash: [R + 1][Q][TX] populations.
 template <int ORD, class Real, int TX, int ZC>
-__device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, const DevParams& p, int x0, int m0,
+__device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, const typename ParamsOf<Real>::T& p, int x0, int m0,
                            Real* ring, Real* stash)
 {
     using L = Lattice<kLatD2Q9>;
@@ -130,7 +191,7 @@ __device__ void batch_item(const Real* __restrict__ A, Real* __restrict__ Bo, co
             });
             ForceSum<Real> F;
             force_ring<kLatD2Q9, ORD, Real, EX, E, NS>(ring, m, tid + R, 0, F);
-            collide<kLatD2Q9, 0>(f, F, p);
+            collide_any(f, F, p);
             const int c = m * p.nx + ix;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -153,7 +214,7 @@ __global__ void __launch_bounds__(TX) k_batch_step(const BatchDom* __restrict__ 
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         const int4 w = items[it];
         const BatchDom d = doms[w.x];
-        const DevParams p = dom_params(d);
+        const auto p = dom_params<Real>(d);
         const Real* A = pool_in + d.off;
         Real* Bo = pool_out + d.off;
         const int x0 = w.y * TX, m0 = w.z * ZC;
@@ -271,7 +332,7 @@ __device__ __forceinline__ void batch_item_seg(const float* __restrict__ A, floa
             load_cell(stage_of(m), tid, f);
             ForceSum<float> F;
             force_ring<kLatD2Q9, ORD, float, EX, EX, NS>(ring, m, tid + R, 0, F);
-            collide<kLatD2Q9, 0>(f, F, p);
+            collide_any(f, F, p);
             const long long c = static_cast<long long>(m) * p.nx + x0 + tid;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -303,7 +364,7 @@ __global__ void __launch_bounds__(TX + 32) k_batch_step_seg(const BatchDom* __re
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         const int4 w = items[it];
         const BatchDom d = doms[w.x];
-        const DevParams p = dom_params(d);
+        const auto p = dom_params<float>(d);
         const float* A = pool_in + d.off;
         float* Bo = pool_out + d.off;
         const int x0 = w.y * TX, m0 = w.z * ZC;
@@ -351,7 +412,7 @@ __global__ void __launch_bounds__(256) k_batch_psi2(const BatchDom* __restrict__
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         const int4 w = items[it];
         const BatchDom d = doms[w.x];
-        const DevParams p = dom_params(d);
+        const auto p = dom_params<Real>(d);
         const long long i = static_cast<long long>(w.y) * 256 + threadIdx.x;
         if (i >= p.N) continue;
         const int x = static_cast<int>(i % p.nx), y = static_cast<int>(i / p.nx);
@@ -364,14 +425,14 @@ __global__ void __launch_bounds__(256) k_batch_psi2(const BatchDom* __restrict__
 
 template <int ORD, class Real>
 __device__ __forceinline__ void fused2_cell(const Real* __restrict__ A, const Real* __restrict__ psi,
-                                            Real* __restrict__ Bo, const DevParams& p, long long i)
+                                            Real* __restrict__ Bo, const typename ParamsOf<Real>::T& p, long long i)
 {
     const int x = static_cast<int>(i % p.nx), y = static_cast<int>(i / p.nx);
     Real f[kQ9];
     gather<kLatD2Q9>(A, p, x, y, 0, f);
     ForceSum<Real> F;
     force_global<ORD, Real>(psi, p.nx, p.ny, x, y, F);
-    collide<kLatD2Q9, 0>(f, F, p);
+    collide_any(f, F, p);
     sfor<kQ9>([&](auto bI) {
         constexpr int b = decltype(bI)::value;
         Bo[static_cast<long long>(b) * p.N + i] = f[b];
@@ -388,7 +449,7 @@ __global__ void __launch_bounds__(256) k_batch_fused2(const BatchDom* __restrict
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         const int4 w = items[it];
         const BatchDom d = doms[w.x];
-        const DevParams p = dom_params(d);
+        const auto p = dom_params<Real>(d);
         const long long i = static_cast<long long>(w.y) * 256 + threadIdx.x;
         if (i >= p.N) continue;
         const Real* A = pool_in + d.off;
@@ -403,10 +464,292 @@ __global__ void __launch_bounds__(256) k_batch_fused2(const BatchDom* __restrict
     }
 }
 
+// ---- resident shape (FP32, even nx): a domain lives in the shared memory of a cluster --
+// Many steps per launch without touching HBM or L2 in between: a cluster of C blocks
+// holds one domain, each block a band of rows with one halo row of populations and R
+// halo rows of psi on each side, and wrapped columns left and right.  A step is two
+// phases:
+//   1. every thread pulls its cells' populations into registers and writes psi;
+//   2. it forms the force from psi, collides and writes the populations back in place.
+// What a neighbouring band needs (the psi rows, the three populations that leave
+// through an edge row) goes straight into that block's halo through distributed shared
+// memory, and one cluster barrier ends each phase, so a step costs no launch and no
+// global traffic.  A thread takes the x-adjacent pair of cells of one column pair in up
+// to kResRows rows: packed FP32 instructions, 8-byte shared accesses, addresses that
+// differ by constants.  The per-cell arithmetic is that of the other shapes, bit for bit.
+// Two warps per sub-partition with 255 registers each (8 rows of populations held across
+// the barrier) beat four with spills or a branch per row.  Bound by the latency of
+// shared-memory loads and packed instructions at that occupancy: 4096 cells of one SM
+// take 4.6 us per step (order 4) to 5.6 us (order 10), 134 GLUPS with every SM busy;
+// clusters of 16 leave part of a GPC idle (16 domains of 256^2: 69 GLUPS).  40 droplets of
+// 64^2 to 256^2: 27 us per step with tile128_rows16, 15 us here; 5 of them 10.6 -> 5.4 us.
+constexpr int kResThreads = 256;
+constexpr int kResRows = 8;       // most rows per thread (144 registers of populations)
+constexpr int kResMaxCluster = 16;
+
+// (every thread arrives; the waits end because all blocks of a cluster run together and
+// take the same number of steps)
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_remote(uint32_t addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_remote(uint32_t addr, float2 v)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+
+// Band of block `rank` of C: rows [y0, y0 + rows).
+__host__ __device__ inline void band_of(int ny, int C, int rank, int& y0, int& rows)
+{
+    const int q = ny / C, rem = ny % C;
+    rows = q + (rank < rem ? 1 : 0);
+    y0 = rank * q + (rank < rem ? rank : rem);
+}
+// Columns on each side: of the populations (one wrapped, one for 8-byte pairs) and of
+// psi (R rounded up to pairs).
+constexpr int kResPad = 2;
+__host__ __device__ constexpr int psi_pad(int R) { return (R + 1) / 2 * 2; }
+// Shared memory of a block: populations [maxrows + 2][9][nx + 2 kResPad], psi
+// [maxrows + 2R][nx + 2 psi_pad].
+__host__ __device__ inline size_t resident_bytes(int nx, int maxrows, int R)
+{
+    return sizeof(float) * (static_cast<size_t>(maxrows + 2) * kQ9 * (nx + 2 * kResPad) +
+                            static_cast<size_t>(maxrows + 2 * R) * (nx + 2 * psi_pad(R)));
+}
+
+// Rows that each thread takes: what a band needs, rounded up to 1, 2, 4 or 8 (more: the
+// band does not fit).
+__host__ __device__ inline int resident_rows_per_thread(int nx, int ny, int C)
+{
+    const int maxrows = (ny + C - 1) / C, per_col = kResThreads / (nx / 2);
+    const int m = (maxrows + per_col - 1) / per_col;
+    return m > 4 ? (m > kResRows ? m : 8) : m == 3 ? 4 : m;
+}
+
+// M: rows per thread.  A band's last strip of rows is moved up to end with the band, so
+// every working thread has M rows and the compiler may interleave them; rows that two
+// threads share get the same values from both.
+template <int ORD, int M>
+__device__ __forceinline__ void resident_domain(const BatchDom& d, const float* __restrict__ A0, float* __restrict__ B0,
+                                                float* smem, int rank, int C, int nsteps)
+{
+    using L = Lattice<kLatD2Q9>;
+    using S = Stencil<2, ORD>;
+    constexpr int R = S::radius;
+    constexpr int Q = kQ9;
+    constexpr int XP = kResPad, PP = psi_pad(R);
+    const auto p = dom_params<float>(d);
+    const int nx = d.nx, ny = d.ny;
+    int y0, rows;
+    band_of(ny, C, rank, y0, rows);
+    const int maxrows = (ny + C - 1) / C;
+    const int SX = nx + 2 * XP, RS = Q * SX;  // population row: [9][SX]
+    const int PS = nx + 2 * PP;
+    float* A = smem;
+    float* psi = smem + (maxrows + 2) * RS;
+    const int N = nx * ny;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    constexpr int kWarps = kResThreads / 32;
+
+    // the band with its halo rows and wrapped columns, a warp per row of one direction
+    for (int k = warp; k < (rows + 2) * Q; k += kWarps) {
+        const int r = k / Q, b = k - r * Q;
+        const float* src = A0 + b * N + wrap_near(y0 + r - 1, ny) * nx;
+        float* dst = A + r * RS + b * SX;
+        for (int c = lane; c < SX; c += 32) dst[c] = src[wrap_near(c - XP, nx)];
+    }
+    // this thread's rows of its column pair
+    const int half = nx / 2;
+    const int per_col = kResThreads / half;  // threads per column pair (half <= kResThreads)
+    const int strip = tid / half, x = 2 * (tid - strip * half);
+    const bool active = strip < per_col && strip * M < rows;
+    const int r0 = strip * M < rows - M ? strip * M : rows - M;
+    const int up = rank == 0 ? C - 1 : rank - 1, dn = rank + 1 == C ? 0 : rank + 1;
+    int yu, rows_up;
+    band_of(ny, C, up, yu, rows_up);
+    // this column pair in the halo rows of the neighbouring bands
+    const uint32_t A_up = map_rank(smem_u32(A + (rows_up + 1) * RS + x + XP), up);
+    const uint32_t A_dn = map_rank(smem_u32(A + x + XP), dn);
+    const uint32_t psi_up = map_rank(smem_u32(psi + (rows_up + R) * PS + x + PP), up);
+    const uint32_t psi_dn = map_rank(smem_u32(psi + x + PP), dn);
+    const bool left = x == 0, right = x == nx - 2;
+    const bool wrap_r = x < PP, wrap_l = x >= nx - PP;  // psi columns repeated past the right / left end
+    const float rho_bar = static_cast<float>(p.rho_bar);
+    float* const a = A + (r0 + 1) * RS + x + XP;
+    float* const ps = psi + (r0 + R) * PS + x + PP;
+    auto ld2 = [](const float* q) { return *reinterpret_cast<const float2*>(q); };
+    auto st2 = [](float* q, float2 v) { *reinterpret_cast<float2*>(q) = v; };
+    auto sync = [&]() {
+        if (C == 1) __syncthreads();
+        else cluster_sync();
+    };
+    __syncthreads();
+    sync();  // every block of the cluster runs and holds its band
+
+    for (int step = 0; step < nsteps; ++step) {
+        float2 f[M][Q];
+        if (active) {
+            float2 v[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                float2 s = make_float2(0.f, 0.f);
+                sfor<Q>([&](auto bI) {
+                    constexpr int b = decltype(bI)::value;
+                    constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1];
+                    const float* q = a + (i - cy) * RS + b * SX;
+                    if constexpr (cx == 0) f[i][b] = ld2(q);
+                    else f[i][b] = make_float2(q[-cx], q[1 - cx]);
+                    s = xadd(s, f[i][b]);
+                });
+                v[i] = make_float2(psi_exp(__fadd_rn(rho_bar, s.x)), psi_exp(__fadd_rn(rho_bar, s.y)));
+            }
+#pragma unroll
+            for (int i = 0; i < M; ++i) st2(ps + i * PS, v[i]);
+            if (wrap_r || wrap_l) {
+                const int o = wrap_r ? nx : -nx;
+#pragma unroll
+                for (int i = 0; i < M; ++i) st2(ps + i * PS + o, v[i]);
+            }
+            if (r0 < R) {
+#pragma unroll
+                for (int i = 0; i < M; ++i)
+                    if (r0 + i < R) {
+                        const uint32_t q = psi_up + 4u * ((r0 + i) * PS);
+                        st_remote(q, v[i]);
+                        if (wrap_r) st_remote(q + 4u * nx, v[i]);
+                        if (wrap_l) st_remote(q - 4u * nx, v[i]);
+                    }
+            }
+            if (r0 + M > rows - R) {
+#pragma unroll
+                for (int i = 0; i < M; ++i)
+                    if (r0 + i >= rows - R) {
+                        const uint32_t q = psi_dn + 4u * ((r0 + i - rows + R) * PS);
+                        st_remote(q, v[i]);
+                        if (wrap_r) st_remote(q + 4u * nx, v[i]);
+                        if (wrap_l) st_remote(q - 4u * nx, v[i]);
+                    }
+            }
+        }
+        sync();
+        if (active) {
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                // psi of the pair shifted by (ex, ey), from aligned 8-byte loads
+                auto tap = [&](auto exI, auto eyI) {
+                    constexpr int ex = decltype(exI)::value, ey = decltype(eyI)::value;
+                    const float* q = ps + (i + ey) * PS + ex;
+                    if constexpr (ex % 2 == 0) return ld2(q);
+                    else return make_float2(ld2(q - 1).y, ld2(q + 1).x);
+                };
+                float2 ax = make_float2(0.f, 0.f), ay = ax;
+                sfor<S::n / 2>([&](auto kI) {
+                    constexpr int k = 2 * decltype(kI)::value;
+                    constexpr int ex = S::T.v[k][0], ey = S::T.v[k][1];
+                    constexpr double wt = S::T.w[k] * L::cs2;
+                    const float2 dp =
+                        xadd(tap(std::integral_constant<int, ex>{}, std::integral_constant<int, ey>{}),
+                             vneg(tap(std::integral_constant<int, -ex>{}, std::integral_constant<int, -ey>{})));
+                    if constexpr (ex != 0) ax = xfma(vsplat<float2>(wt * ex), dp, ax);
+                    if constexpr (ey != 0) ay = xfma(vsplat<float2>(wt * ey), dp, ay);
+                });
+                collide_batch<float2>(f[i], ax, ay, ld2(ps + i * PS), p);
+            }
+#pragma unroll
+            for (int i = 0; i < M; ++i)
+                sfor<Q>([&](auto bI) { st2(a + i * RS + decltype(bI)::value * SX, f[i][decltype(bI)::value]); });
+            if (right) {
+#pragma unroll
+                for (int i = 0; i < M; ++i)
+                    sfor<Q>([&](auto bI) {
+                        constexpr int b = decltype(bI)::value, cx = L::T.v[b][0];
+                        if constexpr (cx == 1) a[i * RS + b * SX + 1 - nx] = f[i][b].y;
+                    });
+            }
+            if (left) {
+#pragma unroll
+                for (int i = 0; i < M; ++i)
+                    sfor<Q>([&](auto bI) {
+                        constexpr int b = decltype(bI)::value, cx = L::T.v[b][0];
+                        if constexpr (cx == -1) a[i * RS + b * SX + nx] = f[i][b].x;
+                    });
+            }
+            // what leaves the band, into the neighbours' halo rows
+            auto leave = [&](uint32_t h, const float2 v, auto cxI) {
+                constexpr int cx = decltype(cxI)::value;
+                st_remote(h, v);
+                if (cx == 1 && right) st_remote(h + 4u - 4u * nx, v.y);
+                if (cx == -1 && left) st_remote(h + 4u * nx, v.x);
+            };
+            if (r0 == 0)
+                sfor<Q>([&](auto bI) {
+                    constexpr int b = decltype(bI)::value, cx = L::T.v[b][0], cy = L::T.v[b][1];
+                    if constexpr (cy == -1) leave(A_up + 4u * (b * SX), f[0][b], std::integral_constant<int, cx>{});
+                });
+            if (r0 == rows - M)
+                sfor<Q>([&](auto bI) {
+                    constexpr int b = decltype(bI)::value, cx = L::T.v[b][0], cy = L::T.v[b][1];
+                    if constexpr (cy == 1) leave(A_dn + 4u * (b * SX), f[M - 1][b], std::integral_constant<int, cx>{});
+                });
+        }
+        sync();
+    }
+    // the band back to the pool
+    for (int k = warp; k < rows * Q; k += kWarps) {
+        const int r = k / Q, b = k - r * Q;
+        const float* src = A + (r + 1) * RS + b * SX + XP;
+        float* dst = B0 + b * N + (y0 + r) * nx;
+        for (int c = lane; c < nx; c += 32) dst[c] = src[c];
+    }
+}
+
+template <int ORD>
+__device__ __forceinline__ void resident_rows(const BatchDom& d, const float* A0, float* B0, float* smem, int rank,
+                                              int C, int nsteps)
+{
+    switch (resident_rows_per_thread(d.nx, d.ny, C)) {
+    case 8: resident_domain<ORD, 8>(d, A0, B0, smem, rank, C, nsteps); break;
+    case 4: resident_domain<ORD, 4>(d, A0, B0, smem, rank, C, nsteps); break;
+    case 2: resident_domain<ORD, 2>(d, A0, B0, smem, rank, C, nsteps); break;
+    default: resident_domain<ORD, 1>(d, A0, B0, smem, rank, C, nsteps); break;
+    }
+}
+
+// One cluster per listed domain; every block of a cluster takes the same way through.
+__global__ void __launch_bounds__(kResThreads, 1) k_batch_resident(const BatchDom* __restrict__ doms,
+                                                                   const int* __restrict__ list, int C,
+                                                                   const float* __restrict__ pool_in,
+                                                                   float* __restrict__ pool_out, int nsteps)
+{
+    extern __shared__ __align__(128) unsigned char dyn_smem[];
+    float* smem = reinterpret_cast<float*>(dyn_smem);
+    const int rank = static_cast<int>(blockIdx.x) % C;
+    const BatchDom d = doms[list[blockIdx.x / C]];
+    if (!d.active) return;
+    const float* A0 = pool_in + d.off;
+    float* B0 = pool_out + d.off;
+    switch (d.order) {
+    case 4: resident_rows<4>(d, A0, B0, smem, rank, C, nsteps); break;
+    case 6: resident_rows<6>(d, A0, B0, smem, rank, C, nsteps); break;
+    case 8: resident_rows<8>(d, A0, B0, smem, rank, C, nsteps); break;
+    default: resident_rows<10>(d, A0, B0, smem, rank, C, nsteps); break;
+    }
+}
+
 // Per-cell macroscopic values of domain d at cell i (pulled populations, psi of
 // the neighbourhood recomputed from the populations; used by the observables).
 template <int ORD, class Real>
-__device__ void batch_cell_obs(const Real* __restrict__ A, const DevParams& p, int x, int y, double& rho,
+__device__ void batch_cell_obs(const Real* __restrict__ A, const typename ParamsOf<Real>::T& p, int x, int y, double& rho,
                                double (&mom)[3])
 {
     using L = Lattice<kLatD2Q9>;
@@ -456,7 +799,7 @@ __global__ void __launch_bounds__(256) k_batch_obs(const BatchDom* __restrict__ 
     if (d >= ndom) return;
     const BatchDom dm = doms[d];
     if (only_active && !dm.active) return;  // a retired domain keeps its last observables
-    const DevParams p = dom_params(dm);
+    const auto p = dom_params<Real>(dm);
     const Real* A = pool + dm.off + (cur_of[d] ? pool_stride : 0);
     double v[kObsWidth] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     bool bad = false;
@@ -502,7 +845,7 @@ __global__ void k_batch_obs_final(const BatchDom* __restrict__ doms, const Real*
         }
     for (int k = 0; k < kObsWidth; ++k) res[d * 8 + k] = acc[k];
     const BatchDom dm = doms[d];
-    const DevParams p = dom_params(dm);
+    const auto p = dom_params<Real>(dm);
     const Real* A = pool + dm.off + (cur_of[d] ? pool_stride : 0);
     auto rho_at = [&](int x, int y) {
         Real f[kQ9];
@@ -523,7 +866,7 @@ __global__ void k_batch_init(const BatchDom* __restrict__ doms, const double* __
     const int d = blockIdx.y;
     if (d >= ndom) return;
     const BatchDom dm = doms[d];
-    const DevParams p = dom_params(dm);
+    const auto p = dom_params<Real>(dm);
     const double rl = init[4 * d], rg = init[4 * d + 1], R = init[4 * d + 2], W = init[4 * d + 3];
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < p.N;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -540,6 +883,41 @@ __global__ void k_batch_init(const BatchDom* __restrict__ doms, const double* __
             const double v = std::is_same<Real, float>::value ? wb * (rho0 - p.rho_bar) : wb * rho0;
             pool[dm.off + static_cast<long long>(b) * p.N + i] = static_cast<Real>(v);
         });
+    }
+}
+
+// State I/O of one domain: f = pre-collision populations in double [9][ny][nx],
+// A the pool's storage (A_b(y) = f_b(y + c_b), FP32 less w_b rho_bar).  On the host the
+// pull took 1.3 ms per 256 x 256 domain, here 10 us.
+template <bool GET, class Real>
+__global__ void __launch_bounds__(256) k_batch_io(int nx, int ny, double rho_bar, Real* __restrict__ A,
+                                                  double* __restrict__ f)
+{
+    using L = Lattice<kLatD2Q9>;
+    constexpr bool kDev = std::is_same<Real, float>::value;
+    const long long N = static_cast<long long>(nx) * ny;
+    const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+    if (i >= kQ9 * N) return;
+    const int b = static_cast<int>(i / N);
+    const int y = static_cast<int>((i - b * N) / nx), x = static_cast<int>(i - b * N - static_cast<long long>(y) * nx);
+    int cx = 0, cy = 0;
+    double w = 0.0;
+    sfor<kQ9>([&](auto bI) {
+        constexpr int q = decltype(bI)::value;
+        constexpr int vx = L::T.v[q][0], vy = L::T.v[q][1];
+        constexpr double wq = L::T.w[q];
+        if (b == q) {
+            cx = vx;
+            cy = vy;
+            w = wq;
+        }
+    });
+    if (GET) {
+        const double v = static_cast<double>(A[b * N + static_cast<long long>(wrap_near(y - cy, ny)) * nx + wrap_near(x - cx, nx)]);
+        f[i] = kDev ? v + w * rho_bar : v;
+    } else {
+        const double v = f[b * N + static_cast<long long>(wrap_near(y + cy, ny)) * nx + wrap_near(x + cx, nx)];
+        A[i] = static_cast<Real>(kDev ? v - w * rho_bar : v);
     }
 }
 
@@ -616,6 +994,18 @@ struct lbm_batch {
     bool pinned;    // a shape was pinned by lbm_batch_set_schedule (never re-tuned)
     long long tuned_cells;  // active cells when the shape was last tuned
     std::vector<double> tune_ms;  // ms per step of each shape (< 0: not timed)
+    // resident shape: domains by cluster size, largest first, each class on a stream
+    // of its own so that the classes share the GPU
+    struct ResClass {
+        int C, first, count;  // list[first .. first + count)
+        size_t bytes;         // shared memory of a block
+    };
+    std::vector<ResClass> res;
+    int* d_list;
+    cudaStream_t aux[kResMaxCluster];
+    cudaEvent_t ev_fork, ev_join[kResMaxCluster];
+    void* io;            // device copy of one domain's populations in double (state I/O)
+    size_t io_bytes;
 
     void* dalloc(size_t bytes)
     {
@@ -648,6 +1038,7 @@ struct BatchVariant {
     int (*occupancy)(int fp32);
     bool staged;   // bulk-copy staging: FP32 only, every nx a multiple of 4
     bool per_cell; // two-pass shape: items are 256 consecutive cells, not (tile, row chunk)
+    bool resident; // steps a domain many times per launch inside a cluster: FP32 only, every domain must fit
 };
 
 template <int TX, int ZC>
@@ -736,22 +1127,132 @@ int occupancy_twopass(int fp32)
     return std::min(a, c);
 }
 
+// Whether bands of an nx x ny domain over C blocks fit the threads' rows and the shared
+// memory; every band has the rows that its threads take at once.
+bool resident_fits(int nx, int ny, int R, int C)
+{
+    const int M = resident_rows_per_thread(nx, ny, C);
+    return M <= kResRows && ny / C >= std::max(R, M) && resident_bytes(nx, (ny + C - 1) / C, R) <= 227 * 1024;
+}
+
+// Blocks of the cluster that holds an nx x ny domain with a stencil of radius R: the
+// fewest whose bands fit the threads' rows and the shared memory, times at most
+// `spread` (to use SMs that would stand idle).  0: none does.
+int resident_cluster(int nx, int ny, int R, int spread)
+{
+    if (nx % 2 != 0 || nx / 2 > kResThreads) return 0;
+    for (int C = 1; C <= kResMaxCluster && ny / C >= R; ++C) {
+        if (!resident_fits(nx, ny, R, C)) continue;
+        for (int S = std::min({C * spread, kResMaxCluster, ny / R}); S > C; --S)
+            if (resident_fits(nx, ny, R, S)) return S;
+        return C;
+    }
+    return 0;
+}
+
+int radius_of(int order) { return order == 4 ? 1 : order == 10 ? 3 : 2; }
+
+cudaLaunchConfig_t resident_config(int C, int count, size_t bytes, cudaStream_t s, cudaLaunchAttribute* attr)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(C * count));
+    cfg.blockDim = dim3(kResThreads);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = static_cast<unsigned>(C);
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// FP32, and every domain fits a cluster of a size that the device can hold.
+bool resident_applies(const lbm_batch* b)
+{
+    if (!b->fp32) return false;
+    bool seen[kResMaxCluster + 1] = {};
+    int most = 0;
+    for (const auto& m : b->doms) {
+        const int C = resident_cluster(m.nx, m.ny, radius_of(m.order), 1);
+        if (C == 0) return false;
+        seen[C] = true;
+        most = std::max(most, resident_cluster(m.nx, m.ny, radius_of(m.order), kResMaxCluster));
+    }
+    seen[most] = true;  // domains spread at most this far
+    if (cudaFuncSetAttribute(k_batch_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(k_batch_resident, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    for (int C = 1; C <= kResMaxCluster; ++C) {
+        if (!seen[C]) continue;
+        cudaLaunchAttribute attr{};
+        const cudaLaunchConfig_t cfg = resident_config(C, 1, 227 * 1024, nullptr, &attr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_batch_resident, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            return false;
+        }
+    }
+    return true;
+}
+
+cudaError_t resident_launch_class(lbm_batch* b, const lbm_batch::ResClass& k, int parity, int n, cudaStream_t s)
+{
+    cudaLaunchAttribute attr{};
+    const cudaLaunchConfig_t cfg = resident_config(k.C, k.count, k.bytes, s, &attr);
+    return cudaLaunchKernelEx(&cfg, k_batch_resident, static_cast<const BatchDom*>(b->d_doms),
+                              static_cast<const int*>(b->d_list + k.first), k.C,
+                              static_cast<const float*>(b->pool[parity]),
+                              static_cast<float*>(b->pool[parity ^ (n & 1)]), n);
+}
+
+// n steps of every active domain: one launch per cluster size, forked from and joined
+// to the batch's stream.
+cudaError_t launch_resident(lbm_batch* b, int parity, int64_t n)
+{
+    constexpr int64_t kMost = 4096;  // steps per launch
+    while (n > 0) {
+        const int k = static_cast<int>(std::min(n, kMost));
+        cudaError_t e = cudaSuccess;
+        if (b->res.size() == 1) {
+            e = resident_launch_class(b, b->res[0], parity, k, b->stream);
+            if (e != cudaSuccess) return e;
+        } else {
+            if ((e = cudaEventRecord(b->ev_fork, b->stream)) != cudaSuccess) return e;
+            for (size_t i = 0; i < b->res.size(); ++i) {
+                if ((e = cudaStreamWaitEvent(b->aux[i], b->ev_fork, 0)) != cudaSuccess) return e;
+                if ((e = resident_launch_class(b, b->res[i], parity, k, b->aux[i])) != cudaSuccess) return e;
+                if ((e = cudaEventRecord(b->ev_join[i], b->aux[i])) != cudaSuccess) return e;
+                if ((e = cudaStreamWaitEvent(b->stream, b->ev_join[i], 0)) != cudaSuccess) return e;
+            }
+        }
+        parity ^= k & 1;
+        n -= k;
+    }
+    return cudaSuccess;
+}
+
 const BatchVariant kBatchVariants[] = {
-    {"tile64_rows16", 64, 16, &launch_variant<64, 16>, &occupancy_variant<64, 16>, false, false},
-    {"tile32_rows16", 32, 16, &launch_variant<32, 16>, &occupancy_variant<32, 16>, false, false},
-    {"tile32_rows32", 32, 32, &launch_variant<32, 32>, &occupancy_variant<32, 32>, false, false},
-    {"tile64_rows8", 64, 8, &launch_variant<64, 8>, &occupancy_variant<64, 8>, false, false},
-    {"tile64_rows32", 64, 32, &launch_variant<64, 32>, &occupancy_variant<64, 32>, false, false},
-    {"tile128_rows16", 128, 16, &launch_variant<128, 16>, &occupancy_variant<128, 16>, false, false},
-    {"tile128_rows32", 128, 32, &launch_variant<128, 32>, &occupancy_variant<128, 32>, false, false},
-    {"staged64_rows32", 64, 32, &launch_seg<64, 32, 8>, &occupancy_seg<64, 32, 8>, true, false},
-    {"staged128_rows32", 128, 32, &launch_seg<128, 32, 8>, &occupancy_seg<128, 32, 8>, true, false},
-    {"staged128_rows64", 128, 64, &launch_seg<128, 64, 8>, &occupancy_seg<128, 64, 8>, true, false},
-    {"staged256_rows64", 256, 64, &launch_seg<256, 64, 8>, &occupancy_seg<256, 64, 8>, true, false},
-    {"staged64_rows1024", 64, 1024, &launch_seg<64, 1024, 8>, &occupancy_seg<64, 1024, 8>, true, false},
-    {"staged128_rows1024", 128, 1024, &launch_seg<128, 1024, 8>, &occupancy_seg<128, 1024, 8>, true, false},
-    {"tile32_rows8", 32, 8, &launch_variant<32, 8>, &occupancy_variant<32, 8>, false, false},
-    {"twopass_cells256", 256, 1, &launch_twopass, &occupancy_twopass, false, true},
+    {"tile64_rows16", 64, 16, &launch_variant<64, 16>, &occupancy_variant<64, 16>, false, false, false},
+    {"tile32_rows16", 32, 16, &launch_variant<32, 16>, &occupancy_variant<32, 16>, false, false, false},
+    {"tile32_rows32", 32, 32, &launch_variant<32, 32>, &occupancy_variant<32, 32>, false, false, false},
+    {"tile64_rows8", 64, 8, &launch_variant<64, 8>, &occupancy_variant<64, 8>, false, false, false},
+    {"tile64_rows32", 64, 32, &launch_variant<64, 32>, &occupancy_variant<64, 32>, false, false, false},
+    {"tile128_rows16", 128, 16, &launch_variant<128, 16>, &occupancy_variant<128, 16>, false, false, false},
+    {"tile128_rows32", 128, 32, &launch_variant<128, 32>, &occupancy_variant<128, 32>, false, false, false},
+    {"staged64_rows32", 64, 32, &launch_seg<64, 32, 8>, &occupancy_seg<64, 32, 8>, true, false, false},
+    {"staged128_rows32", 128, 32, &launch_seg<128, 32, 8>, &occupancy_seg<128, 32, 8>, true, false, false},
+    {"staged128_rows64", 128, 64, &launch_seg<128, 64, 8>, &occupancy_seg<128, 64, 8>, true, false, false},
+    {"staged256_rows64", 256, 64, &launch_seg<256, 64, 8>, &occupancy_seg<256, 64, 8>, true, false, false},
+    {"staged64_rows1024", 64, 1024, &launch_seg<64, 1024, 8>, &occupancy_seg<64, 1024, 8>, true, false, false},
+    {"staged128_rows1024", 128, 1024, &launch_seg<128, 1024, 8>, &occupancy_seg<128, 1024, 8>, true, false, false},
+    {"tile32_rows8", 32, 8, &launch_variant<32, 8>, &occupancy_variant<32, 8>, false, false, false},
+    {"twopass_cells256", 256, 1, &launch_twopass, &occupancy_twopass, false, true, false},
+    {"resident_cluster", 0, 0, nullptr, nullptr, false, false, true},
 };
 constexpr int kNumBatchVariants = sizeof(kBatchVariants) / sizeof(kBatchVariants[0]);
 constexpr int kMinTX = 32, kMinZC = 8;  // smallest tile and chunk of the table (item buffer size)
@@ -766,9 +1267,58 @@ constexpr int kMinTX = 32, kMinZC = 8;  // smallest tile and chunk of the table 
         }                                                                                              \
     } while (0)
 
+// Work of the resident shape: active domains grouped by cluster size, largest first.
+// While the blocks would leave more than half of the SMs idle, domains spread over
+// twice, four times, ... as many.
+int rebuild_resident(lbm_batch* b)
+{
+    int nsm = 0;
+    LBM_BCK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
+    std::vector<int> C(b->n, 0);
+    for (int spread = 1; spread <= kResMaxCluster; spread *= 2) {
+        std::vector<int> Cs(b->n, 0);
+        int blocks = 0;
+        for (int d = 0; d < b->n; ++d) {
+            const BatchDom& m = b->doms[d];
+            if (!m.active) continue;
+            Cs[d] = resident_cluster(m.nx, m.ny, radius_of(m.order), spread);
+            blocks += Cs[d];
+        }
+        if (spread > 1 && blocks > nsm) break;
+        C = Cs;
+        if (2 * blocks > nsm) break;
+    }
+    std::vector<int> list;
+    b->res.clear();
+    for (int c = kResMaxCluster; c >= 1; --c) {
+        lbm_batch::ResClass k{c, static_cast<int>(list.size()), 0, 0};
+        for (int d = 0; d < b->n; ++d)
+            if (C[d] == c) {
+                const BatchDom& m = b->doms[d];
+                list.push_back(d);
+                ++k.count;
+                k.bytes = std::max(k.bytes, resident_bytes(m.nx, (m.ny + c - 1) / c, radius_of(m.order)));
+            }
+        if (k.count) b->res.push_back(k);
+    }
+    if (!b->ev_fork) LBM_BCK(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
+    for (size_t i = 0; i < b->res.size(); ++i)
+        if (!b->aux[i]) {
+            LBM_BCK(cudaStreamCreateWithFlags(&b->aux[i], cudaStreamNonBlocking));
+            LBM_BCK(cudaEventCreateWithFlags(&b->ev_join[i], cudaEventDisableTiming));
+        }
+    if (!list.empty())
+        LBM_BCK(cudaMemcpyAsync(b->d_list, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, b->stream));
+    LBM_BCK(cudaStreamSynchronize(b->stream));
+    b->nitems = static_cast<int>(list.size());
+    return LBM_OK;
+}
+
 int rebuild_items(lbm_batch* b)
 {
     const BatchVariant& v = kBatchVariants[b->var];
+    // a captured graph holds the classes; domains that retire are skipped by their flag
+    if (v.resident) return b->graph[0] ? LBM_OK : rebuild_resident(b);
     std::vector<int4> items;
     for (int d = 0; d < b->n; ++d) {
         BatchDom& m = b->doms[d];
@@ -795,9 +1345,14 @@ int rebuild_items(lbm_batch* b)
     return LBM_OK;
 }
 
-cudaError_t launch_step(lbm_batch* b, int parity)
+// n steps of every active domain from pool[parity]; the state ends in pool[parity ^ (n & 1)].
+cudaError_t launch_steps(lbm_batch* b, int parity, int64_t n)
 {
-    return kBatchVariants[b->var].launch(b, parity);
+    if (kBatchVariants[b->var].resident) return launch_resident(b, parity, n);
+    cudaError_t e = cudaSuccess;
+    for (int64_t i = 0; i < n && e == cudaSuccess; ++i)
+        e = kBatchVariants[b->var].launch(b, (parity + static_cast<int>(i & 1)) & 1);
+    return e;
 }
 
 // Makes shape v current: persistent grid = SMs x resident CTAs, work list rebuilt,
@@ -807,7 +1362,8 @@ int select_variant(lbm_batch* b, int v)
     b->var = v;
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device);
-    b->grid = std::max(1, nsm * std::max(1, kBatchVariants[v].occupancy(b->fp32)));
+    if (!kBatchVariants[v].resident)
+        b->grid = std::max(1, nsm * std::max(1, kBatchVariants[v].occupancy(b->fp32)));
     for (int k = 0; k < 2; ++k)
         if (b->graph[k]) {
             cudaGraphExecDestroy(b->graph[k]);
@@ -868,18 +1424,21 @@ int autotune(lbm_batch* b, bool again = false)
     int best = 0;
     for (int v = 0; v < kNumBatchVariants && rc == LBM_OK; ++v) {
         if (kBatchVariants[v].staged && !(b->fp32 && nx4)) continue;
+        if (kBatchVariants[v].resident && !resident_applies(b)) continue;
         if (int r = select_variant(b, v)) {
             rc = r;
             break;
         }
-        for (int i = 0; i < kWarm; ++i) ck(launch_step(b, (b->cur + i) & 1));
+        // a resident launch reads and writes the state once for all its steps
+        const int timed = kBatchVariants[v].resident ? 8 * kTimed : kTimed;
+        ck(launch_steps(b, b->cur, kWarm));
         ck(cudaEventRecord(e0, b->stream));
-        for (int i = 0; i < kTimed; ++i) ck(launch_step(b, (b->cur + kWarm + i) & 1));
+        ck(launch_steps(b, (b->cur + kWarm) & 1, timed));
         ck(cudaEventRecord(e1, b->stream));
         ck(cudaEventSynchronize(e1));
         float ms = 0.f;
         ck(cudaEventElapsedTime(&ms, e0, e1));
-        b->tune_ms[v] = ms / kTimed;
+        b->tune_ms[v] = ms / timed;
         if (b->tune_ms[v] < b->tune_ms[best]) best = v;
         ck(copy_states(false));
     }
@@ -912,6 +1471,34 @@ cudaError_t launch_obs(lbm_batch* b, int only_active = 0)
             b->d_doms, static_cast<const double*>(b->pool[0]), b->d_cur_of, stride / es, b->d_partials,
             b->d_res, b->n, only_active);
     }
+    return cudaGetLastError();
+}
+
+// Device area for one domain's populations in double, kept for the next call.
+int ensure_io(lbm_batch* b, size_t bytes)
+{
+    if (b->io_bytes >= bytes) return LBM_OK;
+    b->dfree(b->io);
+    b->io_bytes = 0;
+    b->io = b->dalloc(bytes);
+    if (!b->io) return set_last_error(LBM_ENOMEM, "lbm_batch: scratch allocation failed");
+    b->io_bytes = bytes;
+    return LBM_OK;
+}
+
+template <bool GET>
+cudaError_t launch_io(lbm_batch* b, int d)
+{
+    const BatchDom& m = b->doms[d];
+    const long long n = static_cast<long long>(kQ9) * m.nx * m.ny;
+    void* state = static_cast<char*>(b->pool[b->cur_of[d]]) + (b->fp32 ? 4 : 8) * m.off;
+    const unsigned grid = static_cast<unsigned>((n + 255) / 256);
+    if (b->fp32)
+        k_batch_io<GET, float><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, static_cast<float*>(state),
+                                                            static_cast<double*>(b->io));
+    else
+        k_batch_io<GET, double><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, static_cast<double*>(state),
+                                                             static_cast<double*>(b->io));
     return cudaGetLastError();
 }
 
@@ -1019,6 +1606,7 @@ int lbm_batch_create(const lbm_params* ps, const double* init, int n, lbm_batch*
     b->psi_pool = b->dalloc(es * poff);
     b->d_doms = static_cast<BatchDom*>(b->dalloc(sizeof(BatchDom) * n));
     b->d_items = static_cast<int4*>(b->dalloc(sizeof(int4) * items));
+    b->d_list = static_cast<int*>(b->dalloc(sizeof(int) * n));
     b->d_nitems = static_cast<int*>(b->dalloc(256));
     b->d_cur_of = static_cast<int*>(b->dalloc(sizeof(int) * n));
     b->d_init = static_cast<double*>(b->dalloc(sizeof(double) * 4 * n));
@@ -1027,7 +1615,7 @@ int lbm_batch_create(const lbm_params* ps, const double* init, int n, lbm_batch*
     b->d_prev = static_cast<double*>(b->dalloc(sizeof(double) * n));
     b->d_newly = static_cast<int*>(b->dalloc(256));
     b->d_err = static_cast<unsigned*>(b->dalloc(256));
-    if (!b->pool[0] || !b->pool[1] || !b->psi_pool || !b->d_doms || !b->d_items || !b->d_nitems || !b->d_cur_of || !b->d_init ||
+    if (!b->pool[0] || !b->pool[1] || !b->psi_pool || !b->d_doms || !b->d_items || !b->d_list || !b->d_nitems || !b->d_cur_of || !b->d_init ||
         !b->d_partials || !b->d_res || !b->d_prev || !b->d_newly || !b->d_err) {
         lbm_batch_destroy(b);
         return set_last_error(LBM_ENOMEM, "lbm_batch_create: device allocation failed");
@@ -1077,6 +1665,13 @@ int lbm_batch_destroy(lbm_batch* b)
     b->dfree(b->psi_pool);
     b->dfree(b->d_doms);
     b->dfree(b->d_items);
+    b->dfree(b->d_list);
+    b->dfree(b->io);
+    for (int k = 0; k < kResMaxCluster; ++k) {
+        if (b->aux[k]) cudaStreamDestroy(b->aux[k]);
+        if (b->ev_join[k]) cudaEventDestroy(b->ev_join[k]);
+    }
+    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     b->dfree(b->d_nitems);
     b->dfree(b->d_cur_of);
     b->dfree(b->d_init);
@@ -1100,10 +1695,8 @@ int lbm_batch_step(lbm_batch* b, int64_t n)
     LBM_BCK(cudaSetDevice(b->device));
     if (n > 0)
         if (int rc = autotune(b)) return rc;
-    for (int64_t i = 0; i < n; ++i) {
-        LBM_BCK(launch_step(b, b->cur));
-        b->cur ^= 1;
-    }
+    LBM_BCK(launch_steps(b, b->cur, n));
+    b->cur ^= static_cast<int>(n & 1);
     b->global_step += n;
     for (int d = 0; d < b->n; ++d)
         if (b->doms[d].active) {
@@ -1133,7 +1726,7 @@ int lbm_batch_run_to_steady(lbm_batch* b, double tol, int64_t max_steps, int64_t
         cudaGraph_t g = nullptr;
         LBM_BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
-        for (int i = 0; i < K && e == cudaSuccess; ++i) e = launch_step(b, (b->cur + i) & 1);
+        e = launch_steps(b, b->cur, K);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_newly, 0, sizeof(int), b->stream);
         if (e == cudaSuccess) e = launch_obs(b, 1);
         if (e == cudaSuccess) {
@@ -1246,6 +1839,8 @@ int lbm_batch_set_schedule(lbm_batch* b, const char* name)
         if (std::strcmp(kBatchVariants[v].name, name) == 0) {
             if (kBatchVariants[v].staged && !(b->fp32 && nx4))
                 return set_last_error(LBM_EINVAL, "lbm_batch_set_schedule: staged shapes need FP32 and nx % 4 == 0");
+            if (kBatchVariants[v].resident && !resident_applies(b))
+                return set_last_error(LBM_EINVAL, "lbm_batch_set_schedule: the resident shape needs FP32 and domains that fit a cluster");
             b->tuned = true;
             b->pinned = true;
             return select_variant(b, v);
@@ -1287,29 +1882,10 @@ int lbm_batch_set_populations(lbm_batch* b, int d, const double* f_host)
 {
     if (!b || !f_host || d < 0 || d >= b->n) return set_last_error(LBM_EINVAL, "lbm_batch_set_populations: bad argument");
     LBM_BCK(cudaSetDevice(b->device));
-    const BatchDom& m = b->doms[d];
-    const long long N = (long long)m.nx * m.ny;
-    const size_t es = b->fp32 ? 4 : 8;
-    std::vector<unsigned char> raw(es * kQ9 * N);
-    static const int cx[9] = {0, 1, -1, 0, 0, 1, -1, 1, -1};
-    static const int cy[9] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
-    static const double w[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
-    // stream on the host: A_b(y) = f_b(y + c_b)
-    for (int q = 0; q < kQ9; ++q)
-        for (int y = 0; y < m.ny; ++y)
-            for (int x = 0; x < m.nx; ++x) {
-                const int xs = (x + cx[q] + m.nx) % m.nx, ys = (y + cy[q] + m.ny) % m.ny;
-                const double v = f_host[(long long)q * N + (long long)ys * m.nx + xs];
-                const long long i = (long long)q * N + (long long)y * m.nx + x;
-                if (b->fp32) {
-                    const float fv = static_cast<float>(v - w[q] * m.rho_bar);
-                    std::memcpy(&raw[4 * i], &fv, 4);
-                } else {
-                    std::memcpy(&raw[8 * i], &v, 8);
-                }
-            }
-    char* dst = static_cast<char*>(b->pool[b->cur_of[d]]) + es * m.off;
-    LBM_BCK(cudaMemcpyAsync(dst, raw.data(), raw.size(), cudaMemcpyHostToDevice, b->stream));
+    const size_t bytes = sizeof(double) * kQ9 * (size_t)b->doms[d].nx * b->doms[d].ny;
+    if (int rc = ensure_io(b, bytes)) return rc;
+    LBM_BCK(cudaMemcpyAsync(b->io, f_host, bytes, cudaMemcpyHostToDevice, b->stream));
+    LBM_BCK(launch_io<false>(b, d));
     LBM_BCK(cudaStreamSynchronize(b->stream));
     return LBM_OK;
 }
@@ -1319,32 +1895,11 @@ int lbm_batch_get_populations(lbm_batch* b, int d, double* f_host)
 {
     if (!b || !f_host || d < 0 || d >= b->n) return set_last_error(LBM_EINVAL, "lbm_batch_get_populations: bad argument");
     LBM_BCK(cudaSetDevice(b->device));
-    const BatchDom& m = b->doms[d];
-    const long long N = (long long)m.nx * m.ny;
-    const size_t es = b->fp32 ? 4 : 8;
-    std::vector<unsigned char> raw(es * kQ9 * N);
-    const char* src = static_cast<const char*>(b->pool[b->cur_of[d]]) + es * m.off;
-    LBM_BCK(cudaMemcpyAsync(raw.data(), src, raw.size(), cudaMemcpyDeviceToHost, b->stream));
+    const size_t bytes = sizeof(double) * kQ9 * (size_t)b->doms[d].nx * b->doms[d].ny;
+    if (int rc = ensure_io(b, bytes)) return rc;
+    LBM_BCK(launch_io<true>(b, d));
+    LBM_BCK(cudaMemcpyAsync(f_host, b->io, bytes, cudaMemcpyDeviceToHost, b->stream));
     LBM_BCK(cudaStreamSynchronize(b->stream));
-    // un-stream on the host: f_b(x) = A_b(x - c_b)
-    static const int cx[9] = {0, 1, -1, 0, 0, 1, -1, 1, -1};
-    static const int cy[9] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
-    static const double w[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
-    for (int q = 0; q < kQ9; ++q)
-        for (int y = 0; y < m.ny; ++y)
-            for (int x = 0; x < m.nx; ++x) {
-                const int xs = ((x - cx[q]) % m.nx + m.nx) % m.nx, ys = ((y - cy[q]) % m.ny + m.ny) % m.ny;
-                const long long i = (long long)q * N + (long long)ys * m.nx + xs;
-                double v;
-                if (b->fp32) {
-                    float fv;
-                    std::memcpy(&fv, &raw[4 * i], 4);
-                    v = (double)fv + w[q] * m.rho_bar;
-                } else {
-                    std::memcpy(&v, &raw[8 * i], 8);
-                }
-                f_host[(long long)q * N + (long long)y * m.nx + x] = v;
-            }
     return LBM_OK;
 }
 

@@ -272,7 +272,7 @@ __device__ __forceinline__ float psi_exp(float r) { return -expm1f(-r); }
 // is n / D, and sqrt(n / D) = |n| / sqrt(n D): one reciprocal square root where
 // the terms taken one by one need three divisions and a square root, all on the
 // FP64 pipe (2 lanes per cycle and SM).
-__device__ __forceinline__ double psi_pr(double rho, const DevParams& p, double cs2)
+__device__ __forceinline__ double psi_pr(double rho, const DevParams64& p, double cs2)
 {
     const double br = kPrB * rho;
     const double d1 = 1.0 - br;
@@ -289,12 +289,15 @@ __device__ __forceinline__ double psi_pr(double rho, const DevParams& p, double 
     return fabs(n) * rsqrt(q);
 }
 
-template <int LAT, class Real>
-__device__ __forceinline__ Real psi_of(Real rho, const DevParams& p)
+template <int LAT>
+__device__ __forceinline__ float psi_of(float rho, const DevParams&)
 {
-    if (std::is_same<Real, double>::value && p.psi_kind == 1)
-        return static_cast<Real>(psi_pr(static_cast<double>(rho), p, Lattice<LAT>::cs2));
     return psi_exp(rho);
+}
+template <int LAT>
+__device__ __forceinline__ double psi_of(double rho, const DevParams64& p)
+{
+    return p.psi_kind == 1 ? psi_pr(rho, p, Lattice<LAT>::cs2) : psi_exp(rho);
 }
 
 // Writes psi of cell (x, y, z) and its periodic images into the ghosted buffer.
@@ -303,7 +306,8 @@ __device__ __forceinline__ void store_psi(Real* __restrict__ psi, const DevParam
 {
     const int g = p.g;
     const int gz = (D == 3) ? g : 0;
-    if (x >= kGhostX && x < p.nx - kGhostX && y >= g && y < p.ny - g && (D == 2 || (z >= g && z < p.nz - g))) {
+    if (std::is_same<Real, double>::value && x >= kGhostX && x < p.nx - kGhostX && y >= g && y < p.ny - g &&
+        (D == 2 || (z >= g && z < p.nz - g))) {
         psi[(static_cast<long long>(z + gz) * p.psy + (y + g)) * p.psx + (x + kGhostX)] = v;  // no image is a ghost
         return;
     }
@@ -345,7 +349,7 @@ __device__ __forceinline__ void force_add(ForceSum<Real>& F, Real d)
         constexpr int i = decltype(iI)::value;
         constexpr int e = S::T.v[A][i];
         if constexpr (k64 && axis && e == 1) F.a[i] = d;
-        else if constexpr (e != 0) F.a[i] += Real(w * e) * d;
+        else if constexpr (e != 0) F.a[i] = vfma(Real(w * e), d, F.a[i]);
     });
 }
 
@@ -700,7 +704,7 @@ Coll64 fill_c64(const DevParams& p)
     return c;
 }
 template <int LAT, int ORD, int COLL>
-DevParams params64(DevParams p)
+DevParams64 params64(DevParams64 p)
 {
     p.c64 = fill_c64<LAT, ORD, COLL>(p);
     return p;
@@ -717,7 +721,7 @@ constexpr int mrt_first(int b, int parity)
 
 template <int LAT, int COLL, bool ONE>
 __device__ __forceinline__ void collide64_at(double (&f)[Lattice<LAT>::Q], const ForceSum<double>& F, double rho,
-                                             const DevParams& p)
+                                             const DevParams64& p)
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q, D = L::D, NP = (Q - 1) / 2;
@@ -861,7 +865,7 @@ __device__ __forceinline__ void collide64_at(double (&f)[Lattice<LAT>::Q], const
 
 template <int LAT, int COLL>
 __device__ __forceinline__ void collide64(double (&f)[Lattice<LAT>::Q], const ForceSum<double>& F, double rho,
-                                          const DevParams& p)
+                                          const DevParams64& p)
 {
     if (p.omega == 1.0)
         collide64_at<LAT, COLL, true>(f, F, rho, p);
@@ -986,7 +990,8 @@ __device__ __forceinline__ void collide32(float (&f)[Lattice<LAT>::Q], const For
 // f holds pre-collision populations (FP32: deviations); on return the
 // post-collision ones.
 template <int LAT, int COLL, class Real>
-__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const ForceSum<Real>& F, const DevParams& p)
+__device__ __forceinline__ void collide(Real (&f)[Lattice<LAT>::Q], const ForceSum<Real>& F,
+                                        const typename ParamsOf<Real>::T& p)
 {
     if constexpr (std::is_same<Real, double>::value) collide64<LAT, COLL>(f, F, sum_f<LAT>(f), p);
     else collide32<LAT, COLL>(f, F, p);
@@ -1096,7 +1101,7 @@ struct CellXYZ {
     int x, y, z;
 };
 template <int D>
-__device__ __forceinline__ CellXYZ cell_xyz(const DevParams& p, unsigned i)
+__device__ __forceinline__ CellXYZ cell_xyz(const DevParams64& p, unsigned i)
 {
     const unsigned r = p.dnx.div(i);
     CellXYZ c;
@@ -1108,7 +1113,7 @@ __device__ __forceinline__ CellXYZ cell_xyz(const DevParams& p, unsigned i)
 
 template <int LAT>
 __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, double* __restrict__ psi,
-                                               double* __restrict__ rho, DevParams p)
+                                               double* __restrict__ rho, DevParams64 p)
 {
     using L = Lattice<LAT>;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1128,7 +1133,7 @@ __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, dou
 // Solid nodes (y < wall_rows, 2-D) bounce back: f*_b = f_{-b}.
 template <int LAT, int ORD, int COLL>
 __global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, const double* __restrict__ psi,
-                                                 const double* __restrict__ rho, double* __restrict__ B, DevParams p)
+                                                 const double* __restrict__ rho, double* __restrict__ B, DevParams64 p)
 {
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;
@@ -1281,7 +1286,7 @@ __device__ __forceinline__ void gather_off(const Pops<Real, Lattice<LAT>::Q>& P,
 // 1 = registers (R = 1 only), 2 = dynamic shared memory, [R + 1][Q][TX*TY].
 template <int LAT, int ORD, int COLL, class Real, int TX, int TY, int ZC, int MINB, int ST>
 __global__ void __launch_bounds__(TX * TY, MINB)
-    k_onepass(const __grid_constant__ Pops<Real, Lattice<LAT>::Q> P, DevParams p, int ntx, int nty)
+    k_onepass(const __grid_constant__ Pops<Real, Lattice<LAT>::Q> P, typename ParamsOf<Real>::T p, int ntx, int nty)
 {
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;
@@ -3856,8 +3861,9 @@ cudaError_t launch_onepass(const LaunchArgs& a, cudaStream_t s)
     const int nm = k3 ? a.p.nz : a.p.ny;
     const long long nblocks = static_cast<long long>(ntx) * nty * ((nm + ZC - 1) / ZC);
     const auto P = make_pops<Real, Lattice<LAT>::Q>(a.fin, a.fout, a.p.N);
-    kern<<<static_cast<unsigned>(nblocks), TX * TY, dyn, s>>>(
-        P, std::is_same<Real, double>::value ? params64<LAT, ORD, COLL>(a.p) : a.p, ntx, nty);
+    typename ParamsOf<Real>::T p = a.p;
+    if constexpr (std::is_same<Real, double>::value) p = params64<LAT, ORD, COLL>(a.p);
+    kern<<<static_cast<unsigned>(nblocks), TX * TY, dyn, s>>>(P, p, ntx, nty);
     return cudaGetLastError();
 }
 

@@ -82,7 +82,7 @@ __device__ __forceinline__ double centre_offset(int i, int n)
 }
 
 // Periodic distance of cell i to the centre node.
-__device__ __forceinline__ double centre_distance(const DevParams& p, int dim, long long i)
+__device__ __forceinline__ double centre_distance(const DevParams64& p, int dim, long long i)
 {
     const unsigned c = static_cast<unsigned>(i);
     const unsigned r = p.dnx.div(c);
@@ -151,7 +151,7 @@ __device__ void search_update(RadiusSearch& s, const double (&m)[3])
 // updates the search, so a round is two launches and no host read.  Bounded by
 // the FP64 distance and interpolation of 3 candidates per cell, whose distance
 // is formed once.
-__global__ void __launch_bounds__(256) k_search_round(DevParams p, int dim, const float* __restrict__ tables, int T,
+__global__ void __launch_bounds__(256) k_search_round(DevParams64 p, int dim, const float* __restrict__ tables, int T,
                                                       double dmax, RadiusSearch* st, double* partials)
 {
     __shared__ double sh[256];
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(256) k_search_round(DevParams p, int dim, cons
     }
 }
 
-__global__ void k_search_field(DevParams p, int dim, const float* __restrict__ tables, int T, double dmax,
+__global__ void k_search_field(DevParams64 p, int dim, const float* __restrict__ tables, int T, double dmax,
                                const RadiusSearch* __restrict__ st, double* __restrict__ rho0)
 {
     const double R = st->Re, shift = st->m0 - st->mm;
@@ -216,7 +216,7 @@ cudaError_t launch_search_start(RadiusSearch* st, const double* res, double lo, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_search_round(const DevParams& p, int dim, const float* tables, int T, double dmax,
+cudaError_t launch_search_round(const DevParams64& p, int dim, const float* tables, int T, double dmax,
                                 RadiusSearch* st, double* partials, int nblocks_max, cudaStream_t s)
 {
     long long nb = (p.N + 255) / 256;
@@ -225,7 +225,7 @@ cudaError_t launch_search_round(const DevParams& p, int dim, const float* tables
     return cudaGetLastError();
 }
 
-cudaError_t launch_search_field(const DevParams& p, int dim, const float* tables, int T, double dmax,
+cudaError_t launch_search_field(const DevParams64& p, int dim, const float* tables, int T, double dmax,
                                 const RadiusSearch* st, double* rho0, cudaStream_t s)
 {
     const long long nb = (p.N + 255) / 256;

@@ -176,3 +176,37 @@ def test_batch_staged_shapes_match_oracle_and_each_other(lbm):
     with pytest.raises(lbm.LbmError):
         b.set_schedule(staged[0])
     b.close()
+
+
+RESIDENT_DOMAINS = STAGED_DOMAINS + [
+    dict(nx=8, ny=8, G=-4.5, tau=1.0, stencil=10, rho_l=1.4, rho_g=0.3, R=2.0, width=2.0),    # bands of 4 rows
+    dict(nx=38, ny=45, G=-5.5, tau=0.6, stencil=10, rho_l=2.2, rho_g=0.1, R=9.0, width=2.0),  # odd rows, 19 pairs
+    dict(nx=70, ny=33, G=-4.6, tau=0.7, stencil=4, rho_l=1.6, rho_g=0.22, R=10.0, width=2.0),
+    dict(nx=256, ny=256, G=-5.0, tau=0.8, stencil=10, rho_l=2.0, rho_g=0.15, R=60.0, width=2.0),  # 16 blocks
+    dict(nx=192, ny=190, G=-4.9, tau=1.0, stencil=8, rho_l=2.0, rho_g=0.15, R=40.0, width=2.0),   # uneven bands
+    dict(nx=500, ny=20, G=-4.9, tau=0.9, stencil=6, rho_l=2.0, rho_g=0.15, R=6.0, width=2.0),
+]
+
+
+@pytest.mark.parametrize("doms", [RESIDENT_DOMAINS, RESIDENT_DOMAINS[4:5], RESIDENT_DOMAINS[7:9]])
+def test_batch_resident_shape_is_bitwise_the_tiled_one(lbm, doms):
+    """The cluster-resident shape against the tiled one after odd and even numbers
+    of steps (the state changes pools), bit for bit, with few domains (spread over
+    more blocks) and many; odd nx and FP64 are refused."""
+    outs = {}
+    for name in ("tile64_rows16", "resident_cluster"):
+        b = lbm.Batch(doms, precision=1)
+        b.set_schedule(name)
+        b.step(7)
+        first = [b.get_f(i) for i in range(len(doms))]
+        b.step(12)
+        outs[name] = (first, [b.get_f(i) for i in range(len(doms))])
+        b.close()
+    for a, c in zip(*outs.values()):
+        for i, (x, y) in enumerate(zip(a, c)):
+            assert np.array_equal(x, y), i
+    for bad, precision in ((DOMAINS[2:3], 1), (doms, 0)):
+        b = lbm.Batch(bad, precision=precision)
+        with pytest.raises(lbm.LbmError):
+            b.set_schedule("resident_cluster")
+        b.close()
