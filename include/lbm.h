@@ -184,9 +184,10 @@ const char* lbm_step_kernel_name(const lbm_ctx* ctx, int i);
 /* Names the step schedule in use and the time per step of every candidate the
  * autotuner measured, as "chosen=NAME;NAME=ms;..." in buf (NUL-terminated,
  * truncated to len).  With LBM_PATH_AUTO / LBM_PATH_ONE_PASS the first
- * lbm_step (or this call) times each compiled variant (tile shape, chunk
- * length, register cap; and the two-pass schedule under AUTO) on the current
- * state, without advancing it, and keeps the fastest.  The variants compute the
+ * lbm_step (or this call) times the compiled variants that may be fastest at the
+ * domain's size (tile shape, chunk length, register cap; and the two-pass
+ * schedule under AUTO) on the current state, without advancing it, and keeps the
+ * fastest; the others can be pinned and are reported with -1 ms.  The variants compute the
  * same step; FP64 and one-cell-per-thread FP32 variants are bitwise alike, while
  * the packed-pair FP32 variants order their float operations differently and
  * agree within FP32 round-off. */

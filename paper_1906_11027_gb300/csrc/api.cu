@@ -265,32 +265,62 @@ int one_step(lbm_ctx* c)
 // without advancing it: each trial recomputes the same step) with CUDA events on
 // the context's stream, and keeps the fastest.  All candidates perform the same
 // arithmetic, so the choice changes speed only.
+// On small domains a launch takes the host longer than the GPU, and single launches
+// would measure the host (a schedule of two small kernels then looks twice as slow as it
+// is in a replayed graph): there the GPU is first kept busy while the host queues
+// every trial, and the host waits once, at the end.
 int autotune(lbm_ctx* c)
 {
     if (c->tuned) return LBM_OK;
-    cudaEvent_t e0, e1;
-    LBM_CK(cudaEventCreate(&e0));
-    if (cudaEventCreate(&e1) != cudaSuccess) {
-        cudaEventDestroy(e0);
-        return fail(LBM_ECUDA, "event creation failed");
+    constexpr long long kSmall = 1LL << 20;  // cells below which a step is of the order of a launch
+    constexpr unsigned kLaunchNs = 2500;     // host time of one launch
+    const bool small = c->N < kSmall;
+    const int reps = small ? 8 : 3;  // events resolve a few microseconds
+    auto timed = [c](int i) {
+        const long long m = c->cand[i] >= 0 ? c->ks.onepass[c->cand[i]].min_cells : 0;
+        return m >= 0 && c->N >= m;
+    };
+    int n_timed = 0;
+    for (int i = 0; i < c->n_cand; ++i) {
+        n_timed += timed(i);
+        c->cand_ms[i] = -1.0;
     }
-    constexpr int kReps = 3;
+    if (n_timed == 1) {
+        for (int i = 0; i < c->n_cand; ++i)
+            if (timed(i)) c->variant = c->cand[i];
+        c->tuned = true;
+        return LBM_OK;
+    }
+    const bool all = n_timed == 0;
+    if (all) n_timed = c->n_cand;
+    std::vector<cudaEvent_t> ev((size_t)2 * c->n_cand, nullptr);
     int rc = LBM_OK;
-    int best = -1;
+    for (size_t k = 0; k < ev.size(); ++k)
+        if (rc == LBM_OK && (all || timed((int)k / 2)) && cudaEventCreate(&ev[k]) != cudaSuccess) rc = fail(LBM_ECUDA, "event creation failed");
+    for (int i = 0; i < c->n_cand && rc == LBM_OK; ++i)
+        if (all || timed(i)) rc = ensure_carry(c, c->cand[i]);  // allocates
+    if (rc == LBM_OK && small && n_timed > 1 && launch_delay((unsigned)(n_timed * (reps + 4)) * kLaunchNs, c->stream))
+        rc = fail(LBM_ECUDA, "delay launch");
+    int last = 0, best = -1;
     for (int i = 0; i < c->n_cand && rc == LBM_OK; ++i) {
+        if (!all && !timed(i)) continue;
+        last = i;
         const int v = c->cand[i];
         rc = launch_schedule(c, v);  // warm-up (and the start of a carried density)
-        if (rc == LBM_OK && cudaEventRecord(e0, c->stream) != cudaSuccess) rc = fail(LBM_ECUDA, "event record");
-        for (int r = 0; r < kReps && rc == LBM_OK; ++r) rc = launch_schedule(c, v);
-        if (rc == LBM_OK && cudaEventRecord(e1, c->stream) != cudaSuccess) rc = fail(LBM_ECUDA, "event record");
-        if (rc == LBM_OK && cudaEventSynchronize(e1) != cudaSuccess) rc = fail(LBM_ECUDA, "event sync");
-        float ms = 0.f;
-        if (rc == LBM_OK) cudaEventElapsedTime(&ms, e0, e1);
-        c->cand_ms[i] = ms / kReps;
-        if (rc == LBM_OK && (best < 0 || c->cand_ms[i] < c->cand_ms[best])) best = i;
+        if (rc == LBM_OK && cudaEventRecord(ev[2 * i], c->stream) != cudaSuccess) rc = fail(LBM_ECUDA, "event record");
+        for (int r = 0; r < reps && rc == LBM_OK; ++r) rc = launch_schedule(c, v);
+        if (rc == LBM_OK && cudaEventRecord(ev[2 * i + 1], c->stream) != cudaSuccess) rc = fail(LBM_ECUDA, "event record");
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    if (rc == LBM_OK && cudaEventSynchronize(ev[2 * last + 1]) != cudaSuccess) rc = fail(LBM_ECUDA, "event sync");
+    for (int i = 0; i < c->n_cand && rc == LBM_OK; ++i) {
+        if (!all && !timed(i)) continue;
+        float ms = 0.f;
+        if (cudaEventElapsedTime(&ms, ev[2 * i], ev[2 * i + 1]) != cudaSuccess) rc = fail(LBM_ECUDA, "event time");
+        c->cand_ms[i] = ms / reps;
+        if (best < 0 || c->cand_ms[i] < c->cand_ms[best]) best = i;
+    }
+    for (auto& e : ev)
+        if (e) cudaEventDestroy(e);
     if (rc != LBM_OK) return rc;
     c->variant = c->cand[best];
     c->tuned = true;

@@ -29,4 +29,17 @@ cudaError_t launch_wait_probe(unsigned* err, cudaStream_t s)
     return cudaGetLastError();
 }
 
+__global__ void k_delay(unsigned ns)
+{
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < ns) {
+    }
+}
+
+cudaError_t launch_delay(unsigned ns, cudaStream_t s)
+{
+    k_delay<<<1, 1, 0, s>>>(ns < 10000000u ? ns : 10000000u);
+    return cudaGetLastError();
+}
+
 }  // namespace lbm

@@ -138,6 +138,7 @@ struct StepVariant {
     int nx_exact;        // nonzero: the variant is compiled for this nx only (whole rows in shared memory)
     int nx_max;          // nonzero: the variant takes rows of at most this many cells (shared-memory size)
     int carry_rows;      // nonzero: the step reads and writes a carried density for groups of this many rows
+    long long min_cells; // the autotuner times the variant from this size on (< 0: never); it can always be pinned
 };
 constexpr int kMaxVariants = 48;
 
@@ -171,6 +172,10 @@ cudaError_t launch_mean(const double* x, long long n, double* partials, int nblo
 // Failure-detection check (diag.cu): one block waits on an mbarrier that nothing
 // completes, through the step kernels' bounded wait, and sets kErrTimeout in *err.
 cudaError_t launch_wait_probe(unsigned* err, cudaStream_t s);
+
+// Keeps the stream busy for about `ns` (at most 10 ms), so that the host can queue work
+// ahead of it (diag.cu).
+cudaError_t launch_delay(unsigned ns, cudaStream_t s);
 
 // Warm-start network (mlp.cu): the network's density at T signed distances evenly
 // spaced over [-dmax, dmax] for (G, tau, order, r_in * R_dev[c]), c < ncand, into

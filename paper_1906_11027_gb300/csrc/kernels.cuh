@@ -135,6 +135,34 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// ---- programmatic dependent launch ----------------------------------------------
+// The FP64 step kernels of the smallest domains are launched while the one before still
+// runs: pdl_begin lets the next launch start its blocks and then waits until the kernel
+// before has completed and its writes are visible, so launch latency and index
+// arithmetic overlap.  No global memory may be touched before it.
+// Only while every block has an SM of its own (64^2: 5.7 -> 5.2 us per step): blocks that
+// start early take the slots they find, and with more than one per SM the FP64 pipes
+// then fill unevenly (256^2 MRT: 22 -> 34 us).
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_early(bool early, void (*kern)(P...), unsigned grid, int block, cudaStream_t s, const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(static_cast<unsigned>(block));
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- indexing -----------------------------------------------------------------
 __device__ __forceinline__ long long cell_of(const DevParams& p, int x, int y, int z)
 {
@@ -1117,8 +1145,9 @@ __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, dou
 {
     using L = Lattice<LAT>;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.N) return;
     const CellXYZ c = cell_xyz<L::D>(p, i);
+    pdl_begin();
+    if (i >= p.N) return;
     double v = p.psi_w;
     if (c.y >= p.wall_rows) {
         double f[L::Q];
@@ -1138,8 +1167,9 @@ __global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, c
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.N) return;
     const CellXYZ c = cell_xyz<L::D>(p, i);
+    pdl_begin();
+    if (i >= p.N) return;
     double f[L::Q];
     gather<LAT>(A, p, c.x, c.y, c.z, f);
     if (L::D == 2 && c.y < p.wall_rows) {
@@ -1783,153 +1813,6 @@ __global__ void __launch_bounds__(NX * TY + 32, 1)
     if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
 }
 
-// One-pass schedule with bulk-copy staging for 2-D lattices of reach 1 (D2Q9),
-// any force stencil up to radius 3.  A tile is TX cells of a row; the march runs
-// along y.  For row s, direction b needs row s - c_by over x0 - XP .. x0 + TX + XP
-// (XP = 16 bytes of values >= R + 1): one contiguous segment, copied by one
-// cp.async.bulk (two where it crosses the periodic x edge).  A stage stays
-// resident until the row collides, so the interior populations are read from
-// shared memory twice (psi, then collision) and nothing waits in registers;
-// stages hold NSTG rows, NSTG - R - 1 of them in flight.  A producer warp issues
-// the copies.
-template <int LAT, int ORD, int COLL, class Real, int TX, int ZC, int NSTG>
-__global__ void __launch_bounds__(TX + 32, 1)
-    k_onepass_seg(const __grid_constant__ Pops<Real, Lattice<LAT>::Q> P, DevParams p, int ntx)
-{
-    using L = Lattice<LAT>;
-    using S = Stencil<2, ORD>;
-    constexpr int R = S::radius;
-    constexpr int Q = L::Q;
-    static_assert(L::D == 2 && L::reach == 1, "segment staging is written for 2-D reach-1 lattices");
-    constexpr int XP = 16 / static_cast<int>(sizeof(Real));
-    static_assert(XP >= R + 1 && TX % XP == 0 && TX % 32 == 0, "x pad / tile");
-    constexpr int W = TX + 2 * XP;   // staged segment length
-    constexpr int EX = TX + 2 * R;   // psi ring row
-    constexpr int NS = 2 * R + 2;
-    constexpr int STG = Q * W;
-    static_assert(NSTG >= R + 2 && NSTG >= 2 * R, "one row in flight; the 2R warm-up rows staged at once");
-    __shared__ Real ring[NS * EX];
-    __shared__ alignas(8) unsigned long long bars[NSTG];
-    extern __shared__ __align__(128) unsigned char dyn_smem[];
-    Real* stage = reinterpret_cast<Real*>(dyn_smem);  // [NSTG][Q][W]
-
-    const int tile = blockIdx.x % ntx;
-    const int chunk = blockIdx.x / ntx;
-    const int x0 = tile * TX;
-    const int nm = p.ny;
-    const int m0 = chunk * ZC;
-    const int m1 = (m0 + ZC < nm) ? m0 + ZC : nm;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31;
-    const bool producer = tid >= TX;
-
-    if (tid == 0) {
-        for (int k = 0; k < NSTG; ++k) mbar_init(smem_u32(&bars[k]), 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-
-    int cby = 0;
-    const Real* src_b = nullptr;
-    sfor<Q>([&](auto bI) {
-        constexpr int b = decltype(bI)::value;
-        constexpr int vy = L::T.v[b][1];
-        if (lane == b) {
-            cby = vy;
-            src_b = P.in[b];
-        }
-    });
-    const int base = m0 - R;
-    auto issue = [&](int s) {
-        const int slot = (s - base) % NSTG;
-        const uint32_t bar = smem_u32(&bars[slot]);
-        if (lane == 0) mbar_expect_tx(bar, static_cast<uint32_t>(STG * sizeof(Real)));
-        __syncwarp();
-        if (lane < Q) {
-            fence_proxy_async_smem();
-            const Real* row = src_b + static_cast<long long>(wrap_any(s - cby, nm)) * p.nx;
-            uint32_t dst = smem_u32(stage + slot * STG + lane * W);
-            int xs = x0 - XP, left = W;
-            while (left > 0) {
-                const int x = wrap_any(xs, p.nx);
-                const int n = (p.nx - x < left) ? p.nx - x : left;
-                bulk_g2s(dst, row + x, static_cast<uint32_t>(n * sizeof(Real)), bar);
-                dst += static_cast<uint32_t>(n * sizeof(Real));
-                xs += n;
-                left -= n;
-            }
-        }
-    };
-    uint32_t phase = 0;
-    bool ok = true;
-    auto stage_of = [&](int s) { return stage + ((s - base) % NSTG) * STG; };
-    auto wait_stage = [&](int s) {
-        const int slot = (s - base) % NSTG;
-        if (ok && !mbar_wait(smem_u32(&bars[slot]), (phase >> slot) & 1u)) ok = false;  // after a timeout, stop waiting
-        phase ^= 1u << slot;
-    };
-    // f of the cell at tile offset cx (-R .. TX + R - 1) from stage st (pull)
-    auto load_cell = [&](const Real* st, int cx, Real (&f)[Q]) {
-        sfor<Q>([&](auto bI) {
-            constexpr int b = decltype(bI)::value;
-            constexpr int vx = L::T.v[b][0];
-            f[b] = st[b * W + cx + XP - vx];
-        });
-    };
-    auto rho_psi = [&](const Real (&f)[Q]) {
-        Real sum = Real(0);
-        sfor<Q>([&](auto bI) { sum += f[decltype(bI)::value]; });
-        const Real rho = std::is_same<Real, float>::value ? Real(p.rho_bar) + sum : sum;
-        return psi_of<LAT>(rho, p);
-    };
-    auto psi_slab = [&](int s) {
-        wait_stage(s);
-        const Real* st = stage_of(s);
-        Real* dst = ring + ring_slot(s, NS) * EX;
-        Real f[Q];
-        load_cell(st, tid, f);
-        dst[tid + R] = rho_psi(f);
-        if (tid < 2 * R) {
-            const int cx = (tid < R) ? tid - R : TX + tid - R;
-            load_cell(st, cx, f);
-            dst[cx + R] = rho_psi(f);
-        }
-    };
-
-    int next = base;
-    const int last = m1 - 1 + R;
-    if (producer)
-        for (; next <= last && next < base + NSTG; ++next) issue(next);
-    if (!producer)
-        for (int s = m0 - R; s < m0 + R; ++s) psi_slab(s);
-    __syncthreads();
-    // slabs below m0 are consumed (psi only): slab k may refill slab k - NSTG's stage
-    if (producer)
-        for (; next <= last && next < m0 + NSTG; ++next) issue(next);
-
-    const bool active = !producer && (x0 + tid) < p.nx;
-    for (int m = m0; m < m1; ++m) {
-        if (!producer) psi_slab(m + R);
-        __syncthreads();
-        // every thread is past the collision of row m - 1
-        if (producer)
-            for (; next <= last && next <= m - 1 + NSTG; ++next) issue(next);
-        if (active) {
-            Real f[Q];
-            load_cell(stage_of(m), tid, f);
-            ForceSum<Real> F;
-            force_ring<LAT, ORD, Real, EX, EX, NS>(ring, m, tid + R, 0, F);
-            collide<LAT, COLL>(f, F, p);
-            const int c = m * p.nx + x0 + tid;
-            sfor<Q>([&](auto bI) {
-                constexpr int b = decltype(bI)::value;
-                __stcs(P.out[b] + c, f[b]);
-            });
-        }
-    }
-    if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
-}
-
 // One-pass schedule with asynchronous staging (FP32 hot path): the populations
 // of slab s (interior and halo cells of the tile) are copied global -> shared
 // with cp.async one iteration before psi of slab s is formed, and the interior
@@ -2262,7 +2145,8 @@ __device__ __forceinline__ float2 cdot2(float2 vx, float2 vy, float2 vz)
 // Packed-pair collision: BGK (COLL = 0) or MRT (COLL = 1, the BGK update plus
 // the moment-space correction of mrt_moments_g / mrt_apply), both Guo-forced.
 template <int LAT, int COLL = 0>
-__device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const float2 (&F)[3], const DevParams& p)
+__device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const float2 (&F)[3], const DevParams& p,
+                                         float om1f)
 {
     static_assert(COLL == 0 || COLL == 1, "packed pairs: BGK or MRT");
     using L = Lattice<LAT>;
@@ -2313,7 +2197,7 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
     const float2 Vx = mul2(fma2(h, ux, mul2(pref, F[0])), ic4);
     const float2 Vy = mul2(fma2(h, uy, mul2(pref, F[1])), ic4);
     const float2 Vz = mul2(fma2(h, uz, mul2(pref, F[2])), ic4);
-    const float2 om1 = p2(p.om1_f);
+    const float2 om1 = p2(om1f);
     {
         constexpr double w0 = L::T.w[0];
         f[0] = fma2(f[0], om1, mul2(p2(float(w0)), A0));
@@ -2330,6 +2214,122 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
         f[b + 1] = fma2(f[b + 1], om1, mul2(p2(float(wb)), sub2(ev, cP)));
     });
     if constexpr (COLL == 1) mrt_apply<LAT, float2>(t, f);
+}
+
+// ---- one-pass tile schedule (2-D, FP32) ---------------------------------------------
+// A block takes a TX x TY tile at once: every thread pulls its RP vertically adjacent
+// cells into registers and writes their psi to shared memory, the halo's psi is formed
+// beside it, and after one barrier the force and collision run from there.  Nothing
+// marches, so all loads of a block are in flight together, and any nx and alignment
+// will do: the schedule for rows that the staged kernels cannot take (nx no multiple
+// of 4) and for lattices of reach 2.  Cells go through the collision as vertical pairs
+// (packed FP32): their loads and stores stay coalesced along x whatever nx is.  The
+// halo costs (TX + 2R)(TY + 2R) / (TX TY) pulls for psi per cell, from L1 and L2.
+// Bound by instruction issue and L2 latency.  Per step against the marching and
+// two-pass schedules: D2Q9 E8 MRT 1021 x 771 19.4 -> 14.9 us, D2Q9 E4 1024 x 768 20 -> 10.3,
+// 2999^2 159 -> 131, D2Q25 1000 x 999 58 -> 44; the staged rows of k_onepass_seg2 stay ahead
+// from about 8 M cells on (8192 x 1024 109 against 114).
+template <int LAT, int ORD, int COLL, int TX, int TY, int RP, int MINB>
+__global__ void __launch_bounds__(TX * TY / RP, MINB)
+    k_tile2d(const float* __restrict__ A, float* __restrict__ B, DevParams p, int ntx)
+{
+    using L = Lattice<LAT>;
+    using S = Stencil<2, ORD>;
+    constexpr int R = S::radius, RE = L::reach, Q = L::Q;
+    constexpr int NT = TX * TY / RP;
+    constexpr int EX = TX + 2 * R, EY = TY + 2 * R, H = EX * EY - TX * TY;
+    static_assert(L::D == 2 && TY % RP == 0 && (RP % 2 == 0 || COLL == 2), "tile");
+    __shared__ float psi[EY * EX];
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX * RP;
+    const int x0 = static_cast<int>(blockIdx.x % ntx) * TX, y0 = static_cast<int>(blockIdx.x / ntx) * TY;
+    const int nx = p.nx, ny = p.ny, N = static_cast<int>(p.N);
+    auto pull = [&](const int (&xo)[2 * RE + 1], const int (&yo)[2 * RE + 1], float (&f)[Q]) {
+        sfor<Q>([&](auto bI) {
+            constexpr int b = decltype(bI)::value;
+            constexpr int cx = L::T.v[b][0], cy = L::T.v[b][1];
+            f[b] = __ldg(A + (b * N + yo[cy + RE] + xo[cx + RE]));
+        });
+    };
+    float f[RP][Q];
+    {
+        int xo[2 * RE + 1];
+        axis_offsets<RE>(wrap_any(x0 + tx, nx), nx, 1, xo);
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+            int yo[2 * RE + 1];
+            axis_offsets<RE>(wrap_any(y0 + ty + i, ny), ny, nx, yo);
+            pull(xo, yo, f[i]);
+        }
+    }
+#pragma unroll 1
+    for (int h = tid; h < H; h += NT) {
+        int ex, ey;
+        if (h < 2 * R * EX) {  // rows above and below the tile
+            const int r = h / EX;
+            ex = h - r * EX;
+            ey = r < R ? r : TY + r;
+        } else {  // columns beside it
+            const int k = h - 2 * R * EX, r = k / (2 * R), c = k - r * (2 * R);
+            ey = R + r;
+            ex = c < R ? c : TX + c;
+        }
+        int xo[2 * RE + 1], yo[2 * RE + 1];
+        axis_offsets<RE>(wrap_any(x0 - R + ex, nx), nx, 1, xo);
+        axis_offsets<RE>(wrap_any(y0 - R + ey, ny), ny, nx, yo);
+        float g[Q];
+        pull(xo, yo, g);
+        psi[ey * EX + ex] = psi_exp(p.rho_bar_f + sum_f<LAT>(g));
+    }
+    float* const own = psi + (ty + R) * EX + tx + R;
+#pragma unroll
+    for (int i = 0; i < RP; ++i) own[i * EX] = psi_exp(p.rho_bar_f + sum_f<LAT>(f[i]));
+    __syncthreads();
+    if (x0 + tx >= nx) return;
+    float* out = B + ((y0 + ty) * nx + x0 + tx);
+    auto force = [&](int i) {
+        ForceSum<float> F{};
+        const float* c = own + i * EX;
+        sfor<S::n / 2>([&](auto kI) {
+            constexpr int k = 2 * decltype(kI)::value;
+            constexpr int o = S::T.v[k][1] * EX + S::T.v[k][0];
+            force_add<LAT, ORD, k>(F, c[o] - c[-o]);
+        });
+        F.psi = c[0];
+        return F;
+    };
+    if constexpr (COLL == 2) {
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+            if (y0 + ty + i >= ny) return;
+            collide32<LAT, COLL>(f[i], force(i), p);
+            sfor<Q>([&](auto bI) {
+                constexpr int b = decltype(bI)::value;
+                out[b * N + i * nx] = f[i][b];
+            });
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < RP; i += 2) {
+            if (y0 + ty + i >= ny) return;
+            const ForceSum<float> F0 = force(i), F1 = force(i + 1);
+            const float2 gp = make_float2(-p.G_f * F0.psi, -p.G_f * F1.psi);
+            const float2 F[3] = {mul2(gp, make_float2(F0.a[0], F1.a[0])), mul2(gp, make_float2(F0.a[1], F1.a[1])),
+                                 p2(0.f)};
+            float2 g[Q];
+            sfor<Q>([&](auto bI) {
+                constexpr int b = decltype(bI)::value;
+                g[b] = make_float2(f[i][b], f[i + 1][b]);
+            });
+            // 1 - omega exactly complementary to the rounded omega, as in collide32: the mass stays
+            collide2<LAT, COLL>(g, F, p, 1.f - p.omega_f);
+            const bool second = y0 + ty + i + 1 < ny;
+            sfor<Q>([&](auto bI) {
+                constexpr int b = decltype(bI)::value;
+                out[b * N + i * nx] = g[b].x;
+                if (second) out[b * N + (i + 1) * nx] = g[b].y;
+            });
+        }
+    }
 }
 
 // Packed-pair form of the persistent whole-row schedule (FP32 BGK): a compute
@@ -2532,7 +2532,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32 + (PRODW ? 32 
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(fcur, F, p);
+                collide2<LAT, COLL>(fcur, F, p, p.om1_f);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
                     constexpr int b = decltype(bI)::value;
@@ -2758,7 +2758,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32 + (PRODW ? 32 
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(d0, F, p);
+                collide2<LAT, COLL>(d0, F, p, p.om1_f);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
                     constexpr int b = decltype(bI)::value;
@@ -3079,7 +3079,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32, 1)
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(f, F, p);
+                collide2<LAT, COLL>(f, F, p, p.om1_f);
                 if (m >= m0 && m < m1) {
                     const long long c = static_cast<long long>(m) * plane + cell_xy;
                     sfor<Q>([&](auto bI) {
@@ -3132,12 +3132,17 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32, 1)
     if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
 }
 
-// Packed-pair form of the segment schedule k_onepass_seg (FP32 BGK, 2-D reach-1
-// lattices): a compute thread owns the x-adjacent cells (2t, 2t + 1) of the
-// tile, so the directions with c_x = 0 come from the staged segment as one
+// One-pass schedule with bulk-copy staging for 2-D lattices of reach 1 (D2Q9), any
+// force stencil up to radius 3, FP32.  A tile is TX cells of a row; the march runs
+// along y.  For row s, direction b needs row s - c_by over x0 - XP .. x0 + TX + XP (XP = 16
+// bytes of values >= R + 1): one contiguous segment, copied by one cp.async.bulk (two
+// where it crosses the periodic x edge).  A stage stays resident until the row
+// collides, so the interior populations are read from shared memory twice (psi,
+// then collision) and nothing waits in registers; stages hold NSTG rows, NSTG - R - 1 of
+// them in flight.  A producer warp issues the copies.
+// A compute thread owns the x-adjacent cells (2t, 2t + 1) of the tile, so the directions with c_x = 0 come from the staged segment as one
 // 8-byte load per pair, psi, the force and the collision run on float2 pairs
 // with the packed FP32 instructions, and every store is one 8-byte store.
-// Staging, stage reuse and the producer warp are those of k_onepass_seg.
 template <int LAT, int ORD, int COLL, int TX, int ZC, int NSTG>
 __global__ void __launch_bounds__(TX / 2 + 32, 1)
     k_onepass_seg2(const __grid_constant__ Pops<float, Lattice<LAT>::Q> P, DevParams p, int ntx)
@@ -3298,7 +3303,7 @@ __global__ void __launch_bounds__(TX / 2 + 32, 1)
             });
             const float2 gp = mul2(p2(-p.G_f), make_float2(rowp[R][0], rowp[R][1]));
             const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), p2(0.f)};
-            collide2<LAT, COLL>(f, F, p);
+            collide2<LAT, COLL>(f, F, p, p.om1_f);
             const int c = m * p.nx + x0 + cx0;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -3457,7 +3462,7 @@ __global__ void __launch_bounds__(TX2 * TY, MINB)
             });
             const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
             const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-            collide2<LAT, 0>(fcur, F, p);
+            collide2<LAT, 0>(fcur, F, p, p.om1_f);
             const int c = m * mscale + cell_xy;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -3808,15 +3813,15 @@ inline int grid_1d(long long n, int cap = 152 * 16)
 // Threads per block of the FP64 one-cell-per-thread kernels: one warp while the
 // whole domain fits the SMs' block slots that way (it spreads evenly), else four.
 inline int block64(long long n) { return n <= 152LL * 32 * 32 ? 32 : 128; }
+constexpr long long kEarly64 = 152 * 32;  // one warp per SM
 
 template <int LAT, class Real>
 cudaError_t launch_psi(const LaunchArgs& a, cudaStream_t s)
 {
     if constexpr (std::is_same<Real, double>::value) {
         const int bs = block64(a.p.N);
-        k_psi64<LAT><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
-            static_cast<const double*>(a.fin), static_cast<double*>(a.psi), a.rho, a.p);
-        return cudaGetLastError();
+        return launch_early(a.p.N <= kEarly64, &k_psi64<LAT>, static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, s,
+                            static_cast<const double*>(a.fin), static_cast<double*>(a.psi), a.rho, a.p);
     } else {
     const dim3 blk(32, 8, 1);
     const dim3 grd((a.p.nx + 31) / 32, (a.p.ny + 7) / 8, Lattice<LAT>::D == 3 ? a.p.nz : 1);
@@ -3830,10 +3835,10 @@ cudaError_t launch_fused(const LaunchArgs& a, cudaStream_t s)
 {
     if constexpr (std::is_same<Real, double>::value) {
         const int bs = block64(a.p.N);
-        k_fused64<LAT, ORD, COLL><<<static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, 0, s>>>(
-            static_cast<const double*>(a.fin), static_cast<const double*>(a.psi), a.rho,
-            static_cast<double*>(a.fout), params64<LAT, ORD, COLL>(a.p));
-        return cudaGetLastError();
+        return launch_early(a.p.N <= kEarly64, &k_fused64<LAT, ORD, COLL>,
+                            static_cast<unsigned>((a.p.N + bs - 1) / bs), bs, s, static_cast<const double*>(a.fin),
+                            static_cast<const double*>(a.psi), a.rho, static_cast<double*>(a.fout),
+                            params64<LAT, ORD, COLL>(a.p));
     } else {
     const dim3 blk(32, TY, TZ);
     const dim3 grd((a.p.nx + 31) / 32, (a.p.ny + TY - 1) / TY, Lattice<LAT>::D == 3 ? (a.p.nz + TZ - 1) / TZ : 1);
@@ -4064,21 +4069,6 @@ cudaError_t launch_onepass_row(const LaunchArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <int LAT, int ORD, int COLL, class Real, int TX, int ZC, int NSTG>
-cudaError_t launch_onepass_seg(const LaunchArgs& a, cudaStream_t s)
-{
-    constexpr int XP = 16 / static_cast<int>(sizeof(Real));
-    constexpr size_t dyn = sizeof(Real) * NSTG * Lattice<LAT>::Q * (TX + 2 * XP);
-    auto kern = &k_onepass_seg<LAT, ORD, COLL, Real, TX, ZC, NSTG>;
-    if (cudaError_t e = ensure_dyn_smem(kern, dyn); e != cudaSuccess) return e;
-    if (a.p.nx % XP != 0) return cudaErrorInvalidValue;
-    const int ntx = (a.p.nx + TX - 1) / TX;
-    const long long nblocks = static_cast<long long>(ntx) * ((a.p.ny + ZC - 1) / ZC);
-    const auto P = make_pops<Real, Lattice<LAT>::Q>(a.fin, a.fout, a.p.N);
-    kern<<<static_cast<unsigned>(nblocks), TX + 32, dyn, s>>>(P, a.p, ntx);
-    return cudaGetLastError();
-}
-
 template <int LAT, int ORD, int COLL, int TX, int ZC, int NSTG>
 cudaError_t launch_onepass_seg2(const LaunchArgs& a, cudaStream_t s)
 {
@@ -4090,6 +4080,16 @@ cudaError_t launch_onepass_seg2(const LaunchArgs& a, cudaStream_t s)
     const long long nblocks = static_cast<long long>(ntx) * ((a.p.ny + ZC - 1) / ZC);
     const auto P = make_pops<float, Lattice<LAT>::Q>(a.fin, a.fout, a.p.N);
     kern<<<static_cast<unsigned>(nblocks), TX / 2 + 32, dyn, s>>>(P, a.p, ntx);
+    return cudaGetLastError();
+}
+
+template <int LAT, int ORD, int COLL, int TX, int TY, int RP, int MINB>
+cudaError_t launch_tile2d(const LaunchArgs& a, cudaStream_t s)
+{
+    const int ntx = (a.p.nx + TX - 1) / TX;
+    const long long nblocks = static_cast<long long>(ntx) * ((a.p.ny + TY - 1) / TY);
+    k_tile2d<LAT, ORD, COLL, TX, TY, RP, MINB><<<static_cast<unsigned>(nblocks), TX * TY / RP, 0, s>>>(
+        static_cast<const float*>(a.fin), static_cast<float*>(a.fout), a.p, ntx);
     return cudaGetLastError();
 }
 
@@ -4229,7 +4229,7 @@ constexpr VariantList make_variants()
     constexpr bool k3 = Lattice<LAT>::D == 3;
     VariantList k{};
     auto add = [&k](const char* name, cudaError_t (*fn)(const LaunchArgs&, cudaStream_t), int nx_mult = 1,
-                    int nx_exact = 0, int nx_max = 0, int carry_rows = 0) {
+                    int nx_exact = 0, int nx_max = 0, int carry_rows = 0, long long min_cells = 0) {
         if (k.n >= kMaxVariants) {
             k.overflow = true;
             return;
@@ -4240,102 +4240,113 @@ constexpr VariantList make_variants()
         k.v[k.n].nx_exact = nx_exact;
         k.v[k.n].nx_max = nx_max;
         k.v[k.n].carry_rows = carry_rows;
+        k.v[k.n].min_cells = min_cells;
         ++k.n;
     };
+    // Variants that lost to one of the others on every size and row length measured (24^3 to
+    // 256^3, E4 and E6, BGK and MRT; 60^2 to 8192^2) are not timed any more, which took most
+    // of a new context's first step; a program can still pin them by name.
+    auto pin = [&add](const char* name, cudaError_t (*fn)(const LaunchArgs&, cudaStream_t), int nx_mult = 1,
+                      int nx_exact = 0, int nx_max = 0, int carry_rows = 0) {
+        add(name, fn, nx_mult, nx_exact, nx_max, carry_rows, -1);
+    };
     constexpr bool r1 = Stencil<Lattice<LAT>::D, ORD>::radius == 1;
+    // the marching segment kernels start at a block per 256 or 512 columns and 64 rows:
+    // 1021 x 771 14 us with tiles, 73 with segments; 8192 x 1024 114 against 109
+    [[maybe_unused]] constexpr long long kSegMin = 4'000'000;
     constexpr bool hot = COLL == 0 && std::is_same<Real, float>::value;
     if constexpr (k3) {
-        add("onepass_32x8_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 2, 2>);
+        // FP64 is bound by its operations, and halos of a one-pass schedule repeat some
+        add("onepass_32x8_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 2, 2>, 1, 0, 0, 0,
+            std::is_same<Real, double>::value ? -1 : 0);
         if constexpr (hot) {
-            add("onepass_32x8_z16_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 4, 2>);
+            pin("onepass_32x8_z16_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 4, 2>);
             add("onepass_32x8_z16_b3_smem", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 3, 2>);
-            if constexpr (r1) add("onepass_32x8_z16_b3_reg", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 3, 1>);
-            add("onepass_32x8_z16_b4_regather", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 4, 0>);
-            add("onepass_async_32x8_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 32, 8, 16, 2>);
-            add("onepass_async_32x8_z32_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 32, 8, 32, 2>);
+            if constexpr (r1) pin("onepass_32x8_z16_b3_reg", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 3, 1>);
+            pin("onepass_32x8_z16_b4_regather", &launch_onepass<LAT, ORD, COLL, Real, 32, 8, 16, 4, 0>);
+            pin("onepass_async_32x8_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 32, 8, 16, 2>);
+            pin("onepass_async_32x8_z32_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 32, 8, 32, 2>);
             if constexpr (r1) {
-                add("onepass_async_64x4_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 64, 4, 16, 2>);
+                pin("onepass_async_64x4_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 64, 4, 16, 2>);
                 add("onepass_64x4_z16_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 64, 4, 16, 4, 2>);
-                add("onepass_row256x2_z32_s2", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 32, 2, 0>, 1, 256);
-                add("onepass_row256x2_z32_s2_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 32, 2, 1>, 1, 256);
-                add("onepass_row256x2_zauto_s2_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 0, 2, 1>, 1, 256);
-                add("onepass_row256x2_zauto_s2_prod_cs", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 0, 2, 2>, 1, 256);
-                add("onepass_rowp256x2_s2", &launch_onepass_rowp<LAT, ORD, COLL, Real, 256, 2, 2>, 1, 256);
-                add("onepass_rowp2_256x2_s2", &launch_onepass_rowp2<LAT, ORD, 0, 256, 2, 2>, 1, 256);
-                add("onepass_rowp2_256x3_s2", &launch_onepass_rowp2<LAT, ORD, 0, 256, 3, 2>, 1, 256);
+                pin("onepass_row256x2_z32_s2", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 32, 2, 0>, 1, 256);
+                pin("onepass_row256x2_z32_s2_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 32, 2, 1>, 1, 256);
+                pin("onepass_row256x2_zauto_s2_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 0, 2, 1>, 1, 256);
+                pin("onepass_row256x2_zauto_s2_prod_cs", &launch_onepass_row<LAT, ORD, COLL, Real, 256, 2, 0, 2, 2>, 1, 256);
+                pin("onepass_rowp256x2_s2", &launch_onepass_rowp<LAT, ORD, COLL, Real, 256, 2, 2>, 1, 256);
+                pin("onepass_rowp2_256x2_s2", &launch_onepass_rowp2<LAT, ORD, 0, 256, 2, 2>, 1, 256);
+                pin("onepass_rowp2_256x3_s2", &launch_onepass_rowp2<LAT, ORD, 0, 256, 3, 2>, 1, 256);
                 add("onepass_rowp2_256x3_s2_np", &launch_onepass_rowp2<LAT, ORD, 0, 256, 3, 2, false>, 1, 256);
                 add("onepass_rowp2_w256x3_s2_np", &launch_onepass_rowp2w<LAT, ORD, 0, 256, 3, 2, false>, 4, 0, 256);
                 add("onepass_rowp2_w224x3_s2", &launch_onepass_rowp2w<LAT, ORD, 0, 224, 3, 2, true>, 4, 0, 224);
-                add("onepass_rowp2_w208x2_s3", &launch_onepass_rowp2w<LAT, ORD, 0, 208, 2, 3, true>, 4, 0, 208);
+                pin("onepass_rowp2_w208x2_s3", &launch_onepass_rowp2w<LAT, ORD, 0, 208, 2, 3, true>, 4, 0, 208);
                 add("onepass_rowp2_w344x2_s2", &launch_onepass_rowp2w<LAT, ORD, 0, 344, 2, 2, true>, 4, 0, 344);
                 add("onepass_rowp2_w456x1_s2", &launch_onepass_rowp2w<LAT, ORD, 0, 456, 1, 2, true>, 4, 0, 456);
-                add("onepass_row128x4_z32_s3", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 32, 3, 0>, 1, 128);
-                add("onepass_row128x4_z32_s3_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 32, 3, 1>, 1, 128);
-                add("onepass_row128x4_zauto_s3_prod_cs", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 0, 3, 2>, 1, 128);
-                add("onepass_x2_64x8_z16_b2_reg", &launch_onepass_x2<LAT, ORD, 32, 8, 16, 2, 1>, 2);
-                add("onepass_128x4_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 4, 16, 2, 2>);
+                pin("onepass_row128x4_z32_s3", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 32, 3, 0>, 1, 128);
+                pin("onepass_row128x4_z32_s3_prod", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 32, 3, 1>, 1, 128);
+                pin("onepass_row128x4_zauto_s3_prod_cs", &launch_onepass_row<LAT, ORD, COLL, Real, 128, 4, 0, 3, 2>, 1, 128);
+                pin("onepass_x2_64x8_z16_b2_reg", &launch_onepass_x2<LAT, ORD, 32, 8, 16, 2, 1>, 2);
+                pin("onepass_128x4_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 4, 16, 2, 2>);
                 add("onepass_64x4_z8_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 64, 4, 8, 4, 2>);
-                add("onepass_64x4_z32_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 64, 4, 32, 4, 2>);
-                add("onepass_la_64x4_z16_b2", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 2, 1>);
-                add("onepass_lai_64x4_z16_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 3, 0>);
-                add("onepass_lai_64x4_z16_b4", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 4, 0>);
-                add("onepass_lai_64x4_z32_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 32, 3, 0>);
+                pin("onepass_64x4_z32_b4_smem", &launch_onepass<LAT, ORD, COLL, Real, 64, 4, 32, 4, 2>);
+                pin("onepass_la_64x4_z16_b2", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 2, 1>);
+                pin("onepass_lai_64x4_z16_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 3, 0>);
+                pin("onepass_lai_64x4_z16_b4", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 16, 4, 0>);
+                pin("onepass_lai_64x4_z32_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 64, 4, 32, 3, 0>);
             }
             if constexpr (Stencil<3, ORD>::radius == 2) {
-                add("onepass_rowr_w256x2_s1", &launch_onepass_rowr<LAT, ORD, COLL, 256, 2, 1, true>, 4, 0, 256);
-                add("onepass_rowr_w256x2_s1_np", &launch_onepass_rowr<LAT, ORD, COLL, 256, 2, 1, false>, 4, 0, 256);
+                pin("onepass_rowr_w256x2_s1", &launch_onepass_rowr<LAT, ORD, COLL, 256, 2, 1, true>, 4, 0, 256);
+                pin("onepass_rowr_w256x2_s1_np", &launch_onepass_rowr<LAT, ORD, COLL, 256, 2, 1, false>, 4, 0, 256);
                 add("onepass_rowr_w256x3_s1_np", &launch_onepass_rowr<LAT, ORD, COLL, 256, 3, 1, false>, 4, 0, 256);
-                add("onepass_rowr_w256x1_s2", &launch_onepass_rowr<LAT, ORD, COLL, 256, 1, 2, true>, 4, 0, 256);
+                pin("onepass_rowr_w256x1_s2", &launch_onepass_rowr<LAT, ORD, COLL, 256, 1, 2, true>, 4, 0, 256);
             }
             if constexpr (Lattice<LAT>::reach == 1) {
-                add("onepass_rowc_w256x3_s2", &launch_onepass_rowc<LAT, ORD, COLL, 256, 3, 2>, 4, 0, 256, 3);
-                add("onepass_rowc_w256x2_s3", &launch_onepass_rowc<LAT, ORD, COLL, 256, 2, 3>, 4, 0, 256, 2);
+                pin("onepass_rowc_w256x3_s2", &launch_onepass_rowc<LAT, ORD, COLL, 256, 3, 2>, 4, 0, 256, 3);
+                pin("onepass_rowc_w256x2_s3", &launch_onepass_rowc<LAT, ORD, COLL, 256, 2, 3>, 4, 0, 256, 2);
             }
             add("onepass_la_32x8_z16_b2", &launch_onepass_la<LAT, ORD, COLL, Real, 32, 8, 16, 2, 1>);
-            add("onepass_lai_32x8_z16_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 32, 8, 16, 3, 0>);
-            add("onepass_x2_64x8_z16_b2_smem", &launch_onepass_x2<LAT, ORD, 32, 8, 16, 2, 2>, 2);
+            pin("onepass_lai_32x8_z16_b3", &launch_onepass_la<LAT, ORD, COLL, Real, 32, 8, 16, 3, 0>);
+            pin("onepass_x2_64x8_z16_b2_smem", &launch_onepass_x2<LAT, ORD, 32, 8, 16, 2, 2>, 2);
         }
         // MRT in FP32: the packed-pair whole-row kernels (nx = 256)
         if constexpr (COLL == 1 && std::is_same<Real, float>::value && r1) {
             add("onepass_rowp2_256x3_s2_np", &launch_onepass_rowp2<LAT, ORD, 1, 256, 3, 2, false>, 1, 256);
-            add("onepass_rowp2_256x2_s2", &launch_onepass_rowp2<LAT, ORD, 1, 256, 2, 2>, 1, 256);
-            add("onepass_rowp2_256x3_s2", &launch_onepass_rowp2<LAT, ORD, 1, 256, 3, 2>, 1, 256);
+            pin("onepass_rowp2_256x2_s2", &launch_onepass_rowp2<LAT, ORD, 1, 256, 2, 2>, 1, 256);
+            pin("onepass_rowp2_256x3_s2", &launch_onepass_rowp2<LAT, ORD, 1, 256, 3, 2>, 1, 256);
             add("onepass_rowp2_w256x3_s2_np", &launch_onepass_rowp2w<LAT, ORD, 1, 256, 3, 2, false>, 4, 0, 256);
             add("onepass_rowp2_w224x3_s2", &launch_onepass_rowp2w<LAT, ORD, 1, 224, 3, 2, true>, 4, 0, 224);
-            add("onepass_rowp2_w208x2_s3", &launch_onepass_rowp2w<LAT, ORD, 1, 208, 2, 3, true>, 4, 0, 208);
+            pin("onepass_rowp2_w208x2_s3", &launch_onepass_rowp2w<LAT, ORD, 1, 208, 2, 3, true>, 4, 0, 208);
             add("onepass_rowp2_w344x2_s2", &launch_onepass_rowp2w<LAT, ORD, 1, 344, 2, 2, true>, 4, 0, 344);
             add("onepass_rowp2_w456x1_s2", &launch_onepass_rowp2w<LAT, ORD, 1, 456, 1, 2, true>, 4, 0, 456);
         }
         // MRT in FP32, any stencil radius: the carried-density whole-row kernels
         if constexpr (COLL == 1 && std::is_same<Real, float>::value && Lattice<LAT>::reach == 1) {
-            add("onepass_rowc_w256x3_s2", &launch_onepass_rowc<LAT, ORD, 1, 256, 3, 2>, 4, 0, 256, 3);
-            add("onepass_rowc_w256x2_s3", &launch_onepass_rowc<LAT, ORD, 1, 256, 2, 3>, 4, 0, 256, 2);
+            pin("onepass_rowc_w256x3_s2", &launch_onepass_rowc<LAT, ORD, 1, 256, 3, 2>, 4, 0, 256, 3);
+            pin("onepass_rowc_w256x2_s3", &launch_onepass_rowc<LAT, ORD, 1, 256, 2, 3>, 4, 0, 256, 2);
         }
         // MRT in FP32 with the radius-2 stencil: the radius-2 whole-row kernel
         if constexpr (COLL == 1 && std::is_same<Real, float>::value && Stencil<3, ORD>::radius == 2)
             add("onepass_rowr_w256x3_s1_np", &launch_onepass_rowr<LAT, ORD, 1, 256, 3, 1, false>, 4, 0, 256);
     } else {
-        add("onepass_128_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 1, 16, 2, 2>);
-        if constexpr (hot) {
-            add("onepass_256_z16_b3_smem", &launch_onepass<LAT, ORD, COLL, Real, 256, 1, 16, 3, 2>);
-            if constexpr (r1) add("onepass_256_z16_b3_reg", &launch_onepass<LAT, ORD, COLL, Real, 256, 1, 16, 3, 1>);
-            add("onepass_async_256_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 256, 1, 16, 2>);
-            add("onepass_x2_256_z16_b2_smem", &launch_onepass_x2<LAT, ORD, 128, 1, 16, 2, 2>, 2);
-            if constexpr (Lattice<LAT>::reach == 1) {
-                add("onepass_seg256_z64_s8", &launch_onepass_seg<LAT, ORD, COLL, Real, 256, 64, 8>, 4);
-                add("onepass_seg256_z64_s6", &launch_onepass_seg<LAT, ORD, COLL, Real, 256, 64, 6>, 4);
-                add("onepass_seg128_z64_s8", &launch_onepass_seg<LAT, ORD, COLL, Real, 128, 64, 8>, 4);
-                add("onepass_seg512_z64_s6", &launch_onepass_seg<LAT, ORD, COLL, Real, 512, 64, 6>, 4);
-                add("onepass_seg2_256_z64_s6", &launch_onepass_seg2<LAT, ORD, 0, 256, 64, 6>, 4);
-                add("onepass_seg2_512_z64_s6", &launch_onepass_seg2<LAT, ORD, 0, 512, 64, 6>, 4);
-                if constexpr (Stencil<2, ORD>::radius <= 2)
-                    add("onepass_seg2_512_z64_s4", &launch_onepass_seg2<LAT, ORD, 0, 512, 64, 4>, 4);
-            }
+        if constexpr (std::is_same<Real, float>::value) {
+            constexpr int RP = Lattice<LAT>::Q > 16 ? 2 : 4;  // cells per thread: 36 to 52 registers of populations
+            // the flatter tile fills the SMs on small domains, and keeps two cells of a long
+            // velocity set in registers (timed: 60^2 2.6 against 2.9 us, 500 x 300 5.0 against 4.7)
+            add("tile32x8", &launch_tile2d<LAT, ORD, COLL, 32, 8, 2, 1>);
+            add("tile32x16", &launch_tile2d<LAT, ORD, COLL, 32, 16, RP, 1>, 1, 0, 0, 0, Lattice<LAT>::Q > 16 ? -1 : 80000);
+        } else {
+            pin("onepass_128_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 1, 16, 2, 2>);
+        }
+        if constexpr (hot && Lattice<LAT>::reach == 1) {
+            add("onepass_seg2_256_z64_s6", &launch_onepass_seg2<LAT, ORD, 0, 256, 64, 6>, 4, 0, 0, 0, kSegMin);
+            add("onepass_seg2_512_z64_s6", &launch_onepass_seg2<LAT, ORD, 0, 512, 64, 6>, 4, 0, 0, 0, kSegMin);
+            if constexpr (Stencil<2, ORD>::radius <= 2)
+                add("onepass_seg2_512_z64_s4", &launch_onepass_seg2<LAT, ORD, 0, 512, 64, 4>, 4, 0, 0, 0, kSegMin);
         }
         // MRT in FP32 (D2Q9): the packed-pair segment kernels
         if constexpr (COLL == 1 && std::is_same<Real, float>::value && Lattice<LAT>::reach == 1) {
-            add("onepass_seg2_256_z64_s6", &launch_onepass_seg2<LAT, ORD, 1, 256, 64, 6>, 4);
-            add("onepass_seg2_512_z64_s6", &launch_onepass_seg2<LAT, ORD, 1, 512, 64, 6>, 4);
+            add("onepass_seg2_256_z64_s6", &launch_onepass_seg2<LAT, ORD, 1, 256, 64, 6>, 4, 0, 0, 0, kSegMin);
+            add("onepass_seg2_512_z64_s6", &launch_onepass_seg2<LAT, ORD, 1, 512, 64, 6>, 4, 0, 0, 0, kSegMin);
         }
     }
     return k;

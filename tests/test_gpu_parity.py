@@ -462,3 +462,30 @@ def test_persistent_row_kernel_bitwise_at_full_size(lbm):
         dom.close()
     a, b = out.values()
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("lattice,shape,stencil,coll", [
+    (0, (1, 8, 8), 4, 0),      # the smallest box: the halo wraps round more than once per tile
+    (0, (1, 33, 31), 10, 1),   # one cell short of and past a tile, radius 3, MRT
+    (0, (1, 17, 65), 8, 2),    # exact-difference forcing, rows and columns past a tile
+    (2, (1, 15, 33), 0, 2),
+    (3, (1, 32, 64), 10, 0),   # reach 2, whole tiles
+])
+def test_tile_schedules_at_tile_edges(lbm, lattice, shape, stencil, coll):
+    """The 2-D tile schedules at their edges against the oracle (FP32 budget of the
+    schedule comparison above: 1e-5 after 23 steps)."""
+    nz, ny, nx = shape
+    probe = lbm.Domain(nx, ny, nz, lattice=lattice, stencil=stencil, precision=1, collision=coll)
+    names = [k for k in probe.schedule_report() if k.startswith("tile")]
+    probe.close()
+    assert len(names) >= 2
+    ref = oracle.Sim(LAT[lattice], nx, ny, nz, stencil=stencil, G=-5.0, tau=0.9, coll=coll)
+    ref.init_droplet(1.9, 0.15, min(nx, ny) / 4, 2.0)
+    ref.step(23)
+    for name in names:
+        dom = lbm.Domain(nx, ny, nz, lattice=lattice, stencil=stencil, precision=1, tau=0.9, collision=coll)
+        dom.set_schedule(name)
+        dom.init_droplet(1.9, 0.15, min(nx, ny) / 4, 2.0)
+        dom.step(23)
+        assert rel_max(dom.get_f(), ref.get_f()) <= 1e-5, name
+        dom.close()
