@@ -747,14 +747,20 @@ int lbm_init_droplet_learned(lbm_ctx* c, lbm_mlp* net, double R, double rho_l, d
     if (dim == 3) nmin = std::min(nmin, c->prm.nz);
     // 36 halvings of a bracket of at most a few hundred cells leave R_eff within
     // 1e-8; the uniform shift removes the remaining mass difference.  Two halvings
-    // per round on the device: 19 rounds of two launches without a host read take
-    // 1.0 ms where 39 host-driven evaluations took 1.9 ms (256 x 256).
+    // per round on the device: 19 rounds of two launches with one host read make the
+    // call 0.37 ms where 39 host-driven evaluations made it 1.90 ms (256 x 256).
     constexpr int kRounds = 1 + 36 / 2;
     LBM_CK(launch_search_start(st, c->res, 1.0, 0.5 * nmin, c->stream));
     for (int k = 0; k < kRounds; ++k) {
         LBM_CK(mlp_profile_tables(net, c->prm.G, c->prm.tau, (double)c->order, st->cand, r_in, 3, T, kDmax, tables,
                                   c->stream));
         LBM_CK(launch_search_round(a.p, dim, tables, T, kDmax, st, c->partials, kNBlocksMax, c->stream));
+        if (k == 0) {  // a bracket without the wanted mass: no search, the tanh start stays
+            int valid = 0;
+            LBM_CK(cudaMemcpyAsync(&valid, &st->ok, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+            LBM_CK(cudaStreamSynchronize(c->stream));
+            if (!valid) break;
+        }
     }
     LBM_CK(launch_search_field(a.p, dim, tables, T, kDmax, st, rho0.d(), c->stream));
     std::vector<char> host(sizeof(RadiusSearch) + sizeof(float) * 3 * T);

@@ -139,7 +139,7 @@ struct TrainBuf {  // per batch row; what the weight and bias gradients read
     float* dZ32[4];  // the same in f32, for the bias gradients
     float* err;      // y - t
     float* dY;       // 2 (y - t) / rows
-    bf16* dYb;
+    bf16* dYb;       // [rows][kOutPad], column 0: a 16-byte row for the asynchronous copies
 };
 
 struct PassSmem {
@@ -166,10 +166,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(NetView net, PassI
     // weights: rows of 256 bytes, 16 copies each
     for (int i = tid; i < kInPad * 16; i += kPassThreads)
         cp16(s32(&sm.w1[i >> 4][(i & 15) * 8]), net.W[0] + (i >> 4) * kH + (i & 15) * 8, 16);
-    for (int l = 0; l < 3; ++l)
+    cp_commit();
+    for (int l = 0; l < 3; ++l) {  // a group per layer: the first layer starts on its own weights
         for (int i = tid; i < kH * 16; i += kPassThreads)
             cp16(s32(&sm.w[l][i >> 4][(i & 15) * 8]), net.W[l + 1] + (i >> 4) * kH + (i & 15) * 8, 16);
-    cp_commit();
+        cp_commit();
+    }
     if (tid < kH) sm.w5[tid] = net.W[4][tid * kOutPad];
 
     // acc = A W (A: 32 x K tile of activations) for this warp's 16 x 32 piece
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(NetView net, PassI
                 if (TRAIN && r < rows) tb.Xp[(long long)r * kInPad + c] = v;
             }
         }
-        cp_wait<0>();  // the weights, first time round
+        cp_wait<3>();  // the first layer's weights, first time round
         __syncthreads();
         int cur = 0;
 #pragma unroll
@@ -258,6 +260,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(NetView net, PassI
                 }
             }
             cur ^= 1;
+            if (l == 0) cp_wait<2>();
+            if (l == 1) cp_wait<1>();
+            if (l == 2) cp_wait<0>();
             __syncthreads();
         }
         if (wn == 0) {  // output column, one warp per 16 rows
@@ -285,7 +290,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(NetView net, PassI
                             gr = 2.f * e / rows;
                             tb.err[r] = e;
                             tb.dY[r] = gr;
-                            tb.dYb[r] = __float2bfloat16(gr);
+                            uint4 row = make_uint4(0u, 0u, 0u, 0u);
+                            row.x = __bfloat16_as_ushort(__float2bfloat16(gr));
+                            *reinterpret_cast<uint4*>(tb.dYb + (long long)r * kOutPad) = row;
                         }
                     }
                     if (TRAIN) sm.g[rl] = __bfloat162float(__float2bfloat16(gr));
@@ -339,15 +346,19 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(NetView net, PassI
 // of the batch through shared memory (cp.async, chunks of 64 rows): 74 blocks, so
 // all layers run at once and a sum still runs over the rows in order.  Bounded by
 // that order: 256 dependent mma steps for a dW, 4096 dependent additions for a db.
-// Training step of 4096 rows, all kernels and copies: 1.9 ms -> 0.08 ms.
-constexpr int kChunk = 64, kGStages = 4, kCPitch = 40;
+// Eight chunks of 64 rows are in flight per block, and all parts
+// come by asynchronous copies; W5's, a value a row, were loaded and stored by the
+// threads, a memory latency per chunk.  Two training steps of 4096 rows, all kernels
+// and copies: 3.94 ms -> 0.22 ms.
+constexpr int kChunk = 64, kGStages = 8, kCPitch = 40;
+constexpr size_t kGradBytes = sizeof(bf16) * kGStages * 2 * kChunk * kCPitch;  // 80 KB in flight per block
 constexpr int kGradGemms = 3 * 16 + 4 + 4;  // 32 x 32 pieces of W2..W4, W1, W5
 constexpr int kGradJobs = kGradGemms + 4 * 4 + 1 + 1;
 
 __global__ void __launch_bounds__(128) k_mlp_grad(TrainBuf tb, int rows, float* __restrict__ grad,
                                                   double* __restrict__ loss)
 {
-    __shared__ __align__(16) unsigned char buf[kGStages * 2 * kChunk * kCPitch * sizeof(bf16)];
+    extern __shared__ __align__(128) unsigned char buf[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int job = blockIdx.x;
     const int nchunk = (rows + kChunk - 1) / kChunk;
@@ -371,7 +382,7 @@ __global__ void __launch_bounds__(128) k_mlp_grad(TrainBuf tb, int rows, float* 
         const bf16* Bm = l == 4 ? tb.dYb : tb.dZ[l];
         bf16(*As)[kChunk][kCPitch] = reinterpret_cast<bf16(*)[kChunk][kCPitch]>(buf);
         bf16(*Bs)[kChunk][kCPitch] = As + kGStages;
-        if (l == 4) {  // one valid column
+        if (l == 4) {  // one column, copied with its zero neighbours; zeros beyond
             for (int i = tid; i < kGStages * kChunk * kCPitch; i += 128) (&Bs[0][0][0])[i] = __float2bfloat16(0.f);
             __syncthreads();
         }
@@ -389,7 +400,7 @@ __global__ void __launch_bounds__(128) k_mlp_grad(TrainBuf tb, int rows, float* 
                 }
                 if (l == 4 && tid < kChunk) {
                     const long long gr = (long long)c * kChunk + tid;
-                    Bs[st][tid][0] = gr < rows ? Bm[gr] : __float2bfloat16(0.f);
+                    cp16(s32(&Bs[st][tid][0]), gr < rows ? Bm + gr * kOutPad : Bm, gr < rows ? 16 : 0);
                 }
             }
             cp_commit();
@@ -619,7 +630,7 @@ int ensure_train(lbm_mlp* n, int rows)
     free_train(n);
     const size_t cap = (std::max(rows, 1024) + 63) / 64 * 64;  // every part starts on 128 bytes
     const size_t bytes = cap * (sizeof(float) * (kIn + 1) + sizeof(bf16) * kInPad + 8 * sizeof(bf16) * kH +
-                                4 * sizeof(float) * kH + 2 * sizeof(float) + sizeof(bf16)) + 256;
+                                4 * sizeof(float) * kH + 2 * sizeof(float) + sizeof(bf16) * kOutPad) + 256;
     bool ok = cudaMalloc(&n->train, bytes) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k)
         ok = cudaMallocHost(&n->stage[k], sizeof(float) * (kIn + 1) * cap) == cudaSuccess &&
@@ -645,7 +656,7 @@ int ensure_train(lbm_mlp* n, int rows)
     }
     n->tb.err = static_cast<float*>(take(sizeof(float) * cap));
     n->tb.dY = static_cast<float*>(take(sizeof(float) * cap));
-    n->tb.dYb = static_cast<bf16*>(take(sizeof(bf16) * cap));
+    n->tb.dYb = static_cast<bf16*>(take(sizeof(bf16) * kOutPad * cap));
     n->tcap = (int)cap;
     return LBM_OK;
 }
@@ -692,7 +703,7 @@ int loss_and_grad(lbm_mlp* n, int rows)
     tb.t = n->Xt + (size_t)rows * kIn;
     k_mlp_pass<true><<<pass_grid(n, rows), kPassThreads, kTrainBytes, n->stream>>>(n->view(), in, rows, nullptr, tb);
     MCK(cudaGetLastError());
-    k_mlp_grad<<<kGradJobs, 128, 0, n->stream>>>(tb, rows, n->grad, n->loss);
+    k_mlp_grad<<<kGradJobs, 128, kGradBytes, n->stream>>>(tb, rows, n->grad, n->loss);
     MCK(cudaGetLastError());
     return LBM_OK;
 }
@@ -725,6 +736,8 @@ int lbm_mlp_create(lbm_mlp** out, uint64_t seed)
               cudaMalloc(&n->m, sizeof(float) * kNParam) == cudaSuccess &&
               cudaMalloc(&n->v, sizeof(float) * kNParam) == cudaSuccess &&
               cudaFuncSetAttribute(k_mlp_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassBytes) ==
+                  cudaSuccess &&
+              cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradBytes) ==
                   cudaSuccess &&
               cudaFuncSetAttribute(k_mlp_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainBytes) ==
                   cudaSuccess;
