@@ -270,7 +270,8 @@ int lbm_batch_set_populations(lbm_batch* b, int d, const double* f_host);
 /* Tile shape of the batch step kernel (cells per tile along x by rows per work
  * item): "tileTX_rowsZC" shapes gather populations per thread; "stagedTX_rowsZC"
  * shapes stage each row segment in shared memory with bulk copies (FP32 batches
- * whose every nx is a multiple of 4 only).  The first lbm_batch_step /
+ * whose every nx is a multiple of 4 only); "resident_cluster" keeps a domain in the
+ * shared memory of a thread-block cluster (FP32, even nx).  The first lbm_batch_step /
  * lbm_batch_run_to_steady (or this call) times every applicable shape for a few
  * steps on the batch's current state, restores the state, and keeps the
  * fastest; all shapes perform the same per-cell arithmetic, so results are
