@@ -220,3 +220,23 @@ def test_learned_start_saves_steps_on_a_large_droplet(lbm, sweep_net):
     d = dict(nx=512, ny=512, G=-5.0, tau=1.0, stencil=4, rho_l=2.0, rho_g=0.15, R=100.0, width=2.0)
     plain, warm = plain_and_warm(lbm, sweep_net, d)
     assert warm < plain, (plain, warm)
+
+
+@pytest.mark.parametrize("rows", [1, 31, 33, 65, 129])
+def test_rows_at_the_edges_of_a_tile(lbm, rows):
+    """Batches that end inside a tile of 32 rows or a chunk of 64.  A row's output does not
+    depend on the other rows.  Rows whose target is their output add exact zeros to every
+    gradient sum, and doubling the rows halves the mean exactly, so the gradients of a batch
+    are twice those of the batch with as many such rows behind it; a row lost or counted
+    twice would move them by a share of 1 / rows, and FP32 sums by some 1e-7."""
+    net = lbm.MLP(seed=17)
+    rng = np.random.default_rng(rows)
+    X = rng.uniform(-1.5, 1.5, size=(2 * rows, 5)).astype(np.float32)
+    y = net.predict(X)
+    assert np.array_equal(net.predict(X[:rows]), y[:rows])
+    t = y.copy()
+    t[:rows] = rng.normal(size=rows).astype(np.float32)
+    loss, g = net.loss_grad(X[:rows], t[:rows])
+    loss2, g2 = net.loss_grad(X, t)
+    assert loss2 == pytest.approx(0.5 * loss, rel=1e-5)
+    assert np.abs(2.0 * g2 - g).max() <= 1e-5 * np.abs(g).max()
