@@ -575,8 +575,9 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     const int psy = p->ny + 2 * g;
     c->psi_bytes = (size_t)psx * psy * (nz + 2 * gz) * c->elem;
     const size_t fbytes = (size_t)li.Q * c->N * c->elem;
-    c->buf[0] = c->dalloc(fbytes);
-    c->buf[1] = c->dalloc(fbytes);
+    // 32 spare bytes: the copies of k_onepass_rowu take whole 16 bytes past a row's end
+    c->buf[0] = c->dalloc(fbytes + 32);
+    c->buf[1] = c->dalloc(fbytes + 32);
     // psi and, in FP64, the density after it
     const size_t psi_room = (c->psi_bytes + 255) / 256 * 256;
     c->psi = c->dalloc(fp32 ? c->psi_bytes : psi_room + sizeof(double) * c->N);

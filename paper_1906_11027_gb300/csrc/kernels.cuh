@@ -2547,6 +2547,228 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32 + (PRODW ? 32 
     if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
 }
 
+// Whole-row packed-pair schedule for rows of any length, of which none need start on
+// 16 bytes.  A direction's rows are one contiguous run, or two across the periodic y
+// edge; its bulk copy starts at the 16-byte boundary before the run and ends past it
+// (the population buffers end in 32 spare bytes), and the reader skips the 0 to 3 values
+// in front, which follow from the run's offset.  (A copy per row is 133 requests a slab
+// at 131 cells a row, some 47 cycles each: 98 us per step.)  A thread owns the
+// cells (t, t + half) of a row instead of two adjacent ones, so its scalar loads and
+// stores have stride one in a warp whatever the alignment; with an odd nx the last
+// thread's second cell does not exist.  Staging, item walk, producer and ring are those
+// of k_onepass_rowp2.  131 x 117 x 97, MRT: 87 us per step (two-pass) -> 67 us, 226 MB at
+// 3.4 TB/s; bound by the 11 warps a block of this shared memory size has.
+template <int LAT, int ORD, int COLL, int TY, int NSTG, int HMAX>
+__global__ void __launch_bounds__((HMAX * TY + 31) / 32 * 32 + 32, 1)
+    k_onepass_rowu(const __grid_constant__ Pops<float, Lattice<LAT>::Q> P, DevParams p, int zc, int nitems)
+{
+    using L = Lattice<LAT>;
+    using S = Stencil<3, ORD>;
+    constexpr int R = S::radius;
+    constexpr int Q = L::Q;
+    static_assert(L::D == 3 && R == 1 && L::reach == 1, "row staging is written for 3-D radius-1 stencils");
+    constexpr int EY = TY + 2 * R;
+    constexpr int NS = 2 * R + 2;
+    static_assert(NSTG >= 2 * R && NSTG <= 32, "stages");
+    const int nx = p.nx, ny = p.ny, nm = p.nz;
+    const int half = (nx + 1) / 2;
+    const int REG = (EY * nx + 15) & ~3;  // a direction's run, or two with their rounding
+    const int NT = (half * TY + 31) / 32 * 32;  // compute threads, whole warps
+    const int EX = nx + 2 * R;
+    const int E = EX * EY;
+    const int STG = Q * REG;
+    __shared__ alignas(8) unsigned long long bars[NSTG];
+    extern __shared__ __align__(128) unsigned char dyn_smem[];
+    float* stage = reinterpret_cast<float*>(dyn_smem);  // [NSTG][Q][REG]
+    float* ring = stage + NSTG * STG;                   // [NS][E]
+
+    const int nty = (ny + TY - 1) / TY;
+    const int plane = nx * ny;
+    const int tid = threadIdx.x;
+    const int x0 = tid % half, ty = tid / half;  // ty >= TY: idle lane
+    const bool two = x0 + half < nx;
+    const int x1 = two ? x0 + half : x0;  // without a second cell the first one twice
+    const int lane = tid & 31;
+    const bool producer = tid >= NT;
+
+    if (tid == 0) {
+        for (int k = 0; k < NSTG; ++k) mbar_init(smem_u32(&bars[k]), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+
+    int cby = 0, cbz = 0;
+    const float* src_b = nullptr;
+    sfor<Q>([&](auto bI) {
+        constexpr int b = decltype(bI)::value;
+        constexpr int vy = L::T.v[b][1], vz = L::T.v[b][2];
+        if (lane == b) {
+            cby = vy;
+            cbz = vz;
+            src_b = P.in[b];
+        }
+    });
+    int p_it = blockIdx.x, p_y0 = 0, p_next = 0, p_last = -1;
+    auto p_load_item = [&]() {
+        if (p_it >= nitems) return;
+        const int m0 = (p_it / nty) * zc;
+        const int m1 = (m0 + zc < nm) ? m0 + zc : nm;
+        p_y0 = (p_it % nty) * TY;
+        p_next = m0 - R;
+        p_last = m1 - 1 + R;
+    };
+    p_load_item();
+    long long issued = 0;
+    auto issue_next = [&]() {
+        const int slot = static_cast<int>(issued % NSTG);
+        const uint32_t bar = smem_u32(&bars[slot]);
+        // rows [y, y + n1) of the plane, then rows [0, EY - n1); EY <= ny
+        const int y = wrap_near(p_y0 - R - cby, ny);
+        const int n1 = ny - y < EY ? ny - y : EY;
+        const uint32_t c1 = static_cast<uint32_t>((n1 * nx + 6) & ~3) * 4u;
+        const uint32_t c2 = n1 < EY ? static_cast<uint32_t>(((EY - n1) * nx + 6) & ~3) * 4u : 0u;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, lane < Q ? c1 + c2 : 0u);
+        if (lane == 0) mbar_expect_tx(bar, total);
+        __syncwarp();
+        if (lane < Q) {
+            fence_proxy_async_smem();
+            const float* pl = src_b + static_cast<long long>(wrap_near(p_next - cbz, nm)) * plane;
+            const uint32_t dst = smem_u32(stage + slot * STG + lane * REG);
+            auto copy = [&](uint32_t to, const float* from, uint32_t bytes) {
+                bulk_g2s(to, reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(from) & ~uintptr_t(15)), bytes, bar);
+            };
+            copy(dst, pl + static_cast<long long>(y) * nx, c1);
+            if (c2) copy(dst + c1, pl, c2);
+        }
+        __syncwarp();
+        ++issued;
+        if (++p_next > p_last) {
+            p_it += gridDim.x;
+            p_load_item();
+        }
+    };
+    auto issue_upto = [&](long long consumed) {
+        while (p_it < nitems && issued < consumed + NSTG) issue_next();
+    };
+
+    uint32_t phase = 0;
+    bool ok = true;
+    long long consumed = 0;
+    auto wait_seq = [&](long long q) -> const float* {
+        const int slot = static_cast<int>(q % NSTG);
+        if (ok && !mbar_wait(smem_u32(&bars[slot]), (phase >> slot) & 1u)) ok = false;  // after a timeout, stop waiting
+        phase ^= 1u << slot;
+        return stage + slot * STG;
+    };
+    // pull columns for c_x = +1 (x - 1) and c_x = -1 (x + 1), periodic
+    const int xl0 = x0 == 0 ? nx - 1 : x0 - 1, xr0 = x0 + 1 == nx ? 0 : x0 + 1;
+    const int xl1 = x1 == 0 ? nx - 1 : x1 - 1, xr1 = x1 + 1 == nx ? 0 : x1 + 1;
+    // The values in front of a run: its offset b N + z nx ny + y nx modulo 4 (the buffer
+    // starts on 16 bytes), y = 0 for the run after the periodic edge.
+    const int n4 = static_cast<int>(p.N & 3);
+    auto load_pair = [&](const float* st, int s, int y0, int fy, float2 (&f)[Q]) {
+        int zo[3], yo[3], ro[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            zo[k] = wrap_near(s - (k - 1), nm) * (plane & 3);
+            const int y = wrap_near(y0 - R - (k - 1), ny);
+            const int n1 = ny - y;
+            const bool first = fy < n1;
+            yo[k] = first ? y * (nx & 3) : 0;
+            ro[k] = first ? fy * nx : ((n1 * nx + 6) & ~3) + (fy - n1) * nx;
+        }
+        sfor<Q>([&](auto bI) {
+            constexpr int b = decltype(bI)::value;
+            constexpr int vx = L::T.v[b][0], vy = L::T.v[b][1], vz = L::T.v[b][2];
+            const float* rb = st + b * REG + ro[vy + 1] + ((b * n4 + zo[vz + 1] + yo[vy + 1]) & 3);
+            f[b] = vx == 0 ? make_float2(rb[x0], rb[x1])
+                 : vx > 0  ? make_float2(rb[xl0], rb[xl1])
+                           : make_float2(rb[xr0], rb[xr1]);
+        });
+    };
+    auto rho_psi2 = [&](const float2 (&f)[Q]) {
+        float2 sum = p2(0.f);
+        sfor<Q>([&](auto bI) { sum = add2(sum, f[decltype(bI)::value]); });
+        const float rb = static_cast<float>(p.rho_bar);
+        return make_float2(psi_of<LAT>(rb + sum.x, p), psi_of<LAT>(rb + sum.y, p));
+    };
+    float2 fcur[Q], fnxt[Q];
+    auto put_psi2 = [&](float* dst, int fy, float2 v) {
+        float* row = dst + fy * EX;
+        row[x0 + R] = v.x;
+        if (two) row[x1 + R] = v.y;
+        if (x0 == 0) row[nx + R] = v.x;                   // wrapped column right of the row
+        if (two && x1 + 1 == nx) row[0] = v.y;            // wrapped column left of the row
+    };
+    auto psi_slab = [&](int s, int y0, long long q) {
+        const float* st = wait_seq(q);
+        if (ty >= TY) return;  // idle lane: keeps the barrier phases only
+        float* dst = ring + ring_slot(s, NS) * E;
+        load_pair(st, s, y0, ty + R, fnxt);
+        put_psi2(dst, ty + R, rho_psi2(fnxt));
+        for (int k = ty; k < 2 * R; k += TY) {
+            const int fy = (k < R) ? k : EY - 2 * R + k;
+            float2 f[Q];
+            load_pair(st, s, y0, fy, f);
+            put_psi2(dst, fy, rho_psi2(f));
+        }
+    };
+
+    if (producer) issue_upto(0);
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const int y0 = (it % nty) * TY;
+        const int m0 = (it / nty) * zc;
+        const int m1 = (m0 + zc < nm) ? m0 + zc : nm;
+        if (!producer)
+            for (int s = m0 - R; s < m0 + R; ++s) psi_slab(s, y0, consumed + (s - (m0 - R)));
+        consumed += 2 * R;
+#pragma unroll
+        for (int b = 0; b < Q; ++b) fcur[b] = fnxt[b];
+        __syncthreads();
+        if (producer) issue_upto(consumed);
+        const bool active = !producer && ty < TY && (y0 + ty) < ny;
+        const int cell_xy = (y0 + ty) * nx + x0;
+        for (int m = m0; m < m1; ++m) {
+            if (!producer) psi_slab(m + R, y0, consumed);
+            ++consumed;
+            __syncthreads();
+            if (producer) issue_upto(consumed);
+            if (active) {
+                const int d = x1 - x0;
+                const float* base[2 * R + 1];
+#pragma unroll
+                for (int k = 0; k < 2 * R + 1; ++k) base[k] = ring + ring_slot(m - R + k, NS) * E + (ty + R) * EX + x0 + R;
+                float2 ax = p2(0.f), ay = p2(0.f), az = p2(0.f);
+                sfor<S::n / 2>([&](auto kI) {
+                    constexpr int a = 2 * decltype(kI)::value;
+                    constexpr int ex = S::T.v[a][0], ey = S::T.v[a][1], ez = S::T.v[a][2];
+                    constexpr double wt = S::T.w[a] * L::cs2;
+                    const float* pp = base[ez + R] + ey * EX + ex;
+                    const float* pm = base[R - ez] - ey * EX - ex;
+                    const float2 df = sub2(make_float2(pp[0], pp[d]), make_float2(pm[0], pm[d]));
+                    if (ex != 0) ax = fma2(p2(float(wt * ex)), df, ax);
+                    if (ey != 0) ay = fma2(p2(float(wt * ey)), df, ay);
+                    if (ez != 0) az = fma2(p2(float(wt * ez)), df, az);
+                });
+                const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][d]));
+                const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
+                // 1 - omega exactly complementary to the rounded omega, as in collide32: the mass stays
+                collide2<LAT, COLL>(fcur, F, p, 1.f - p.omega_f);
+                const int c = m * plane + cell_xy;
+                sfor<Q>([&](auto bI) {
+                    constexpr int b = decltype(bI)::value;
+                    __stcs(P.out[b] + c, fcur[b].x);
+                    if (two) __stcs(P.out[b] + c + half, fcur[b].y);
+                });
+            }
+#pragma unroll
+            for (int b = 0; b < Q; ++b) fcur[b] = fnxt[b];
+        }
+        __syncthreads();
+    }
+    if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
+}
+
 // Whole-row packed-pair schedule for stencils of radius R >= 2 (D3Q19 with the
 // 6th-order stencil): the staging, item walk and packed collision of
 // k_onepass_rowp2, with the row length read at run time (nx <= NXMAX, a
@@ -3942,6 +4164,33 @@ cudaError_t launch_onepass_rowp2w(const LaunchArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Whole rows of any length 8 <= nx <= 2 HMAX (k_onepass_rowu); every domain has ny >= 8.
+template <int LAT, int ORD, int COLL, int TY, int NSTG, int HMAX>
+cudaError_t launch_onepass_rowu(const LaunchArgs& a, cudaStream_t s)
+{
+    constexpr int Q = Lattice<LAT>::Q;
+    constexpr int EY = TY + 2;
+    static_assert(EY <= 8, "a tile with its halo wraps round the smallest domain once");
+    auto dyn_of = [](int nx) {
+        return sizeof(float) * (static_cast<size_t>(NSTG) * Q * ((EY * nx + 15) & ~3) + 4 * static_cast<size_t>(nx + 2) * EY);
+    };
+    auto kern = &k_onepass_rowu<LAT, ORD, COLL, TY, NSTG, HMAX>;
+    if (cudaError_t e = ensure_dyn_smem(kern, dyn_of(2 * HMAX)); e != cudaSuccess) return e;
+    const int nx = a.p.nx;
+    if (nx < 8 || nx > 2 * HMAX || (reinterpret_cast<uintptr_t>(a.fin) & 15) != 0) return cudaErrorInvalidValue;
+    const int nty = (a.p.ny + TY - 1) / TY;
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int zc = rowp_chunk(a.p.nz, nty, nsm);
+    const int nitems = nty * ((a.p.nz + zc - 1) / zc);
+    const int grid = nitems < nsm ? nitems : nsm;
+    const int threads = ((nx + 1) / 2 * TY + 31) / 32 * 32 + 32;
+    const auto P = make_pops<float, Q>(a.fin, a.fout, a.p.N);
+    kern<<<grid, threads, dyn_of(nx), s>>>(P, a.p, zc, nitems);
+    return cudaGetLastError();
+}
+
 // Radius-2 whole-row schedule (k_onepass_rowr), any row length nx <= NXMAX
 // that is a multiple of 4.
 template <int LAT, int ORD, int COLL, int NXMAX, int TY, int NSTG, bool PRODW>
@@ -4318,6 +4567,14 @@ constexpr VariantList make_variants()
             pin("onepass_rowp2_w208x2_s3", &launch_onepass_rowp2w<LAT, ORD, 1, 208, 2, 3, true>, 4, 0, 208);
             add("onepass_rowp2_w344x2_s2", &launch_onepass_rowp2w<LAT, ORD, 1, 344, 2, 2, true>, 4, 0, 344);
             add("onepass_rowp2_w456x1_s2", &launch_onepass_rowp2w<LAT, ORD, 1, 456, 1, 2, true>, 4, 0, 456);
+        }
+        // Rows of any length, as many of them per tile as two stages and 11 warps allow.  us per
+        // step, MRT, 117 x 97 rows of 64: 37.0 against 40.4 (two-pass); of 109: 55.9, 71.8; of 131:
+        // 66.9, 86.7; of 132: 66.2 against 70.3 (rowp2_w224x3); of 201: 100 against 118
+        if constexpr (COLL <= 1 && std::is_same<Real, float>::value && r1 && Lattice<LAT>::reach == 1) {
+            add("onepass_rowu_w116x6_s2", &launch_onepass_rowu<LAT, ORD, COLL, 6, 2, 58>, 1, 0, 116);
+            add("onepass_rowu_w140x5_s2", &launch_onepass_rowu<LAT, ORD, COLL, 5, 2, 70>, 1, 0, 140);
+            add("onepass_rowu_w232x3_s2", &launch_onepass_rowu<LAT, ORD, COLL, 3, 2, 116>, 1, 0, 232);
         }
         // MRT in FP32, any stencil radius: the carried-density whole-row kernels
         if constexpr (COLL == 1 && std::is_same<Real, float>::value && Lattice<LAT>::reach == 1) {

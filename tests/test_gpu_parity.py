@@ -489,3 +489,53 @@ def test_tile_schedules_at_tile_edges(lbm, lattice, shape, stencil, coll):
         dom.step(23)
         assert rel_max(dom.get_f(), ref.get_f()) <= 1e-5, name
         dom.close()
+
+
+@pytest.mark.parametrize("lattice,shape,coll,top", [
+    (0, (1, 8, 9), 0, 17.0),     # densities on both sides of the table's end (15.5)
+    (0, (1, 64, 76), 1, 2.0),    # 4864 cells: the last size of the early launch
+    (0, (1, 60, 82), 0, 2.0),    # 4920: past it
+    (0, (1, 389, 401), 1, 2.0),  # 155,989: blocks of more than one warp, a ragged last one
+    (2, (1, 9, 11), 2, 17.0),
+    (3, (1, 13, 9), 2, 17.0),
+    (1, (9, 11, 10), 1, 17.0),
+])
+def test_fp64_kernels_at_their_edges(lbm, lattice, shape, coll, top):
+    """FP64 step where its psi table ends and its launch shape changes, against the oracle:
+    3 steps from densities spread over [0.1, top] stay within 1e-12 (operations of 1e-16
+    each, some hundreds in a row)."""
+    dom, ref = pair(lbm, lattice, shape, coll=coll, G=-0.5, path=1)
+    rho = 0.1 + (top - 0.1) * np.random.default_rng(5).random(shape)
+    for d in (dom, ref):
+        d.init_from_rho(rho)
+        d.step(3)
+    assert rel_max(dom.get_f(), ref.get_f()) <= 1e-12
+    dom.close()
+
+
+@pytest.mark.parametrize("shape,coll", [
+    ((8, 8, 8), 0),       # the smallest box: the halo wraps round in every tile
+    ((9, 11, 9), 1),      # odd rows: every alignment of a row occurs, the last pair has one cell
+    ((8, 13, 86), 1),     # rows of 8-byte alignment
+    ((10, 9, 139), 0),    # the longest odd rows of the five-row tile
+    ((8, 9, 231), 1),     # and of the three-row tile, buffer ends off 16 bytes
+    ((161, 16, 12), 0),   # items of several chunks along z
+])
+def test_unaligned_row_schedules(lbm, shape, coll):
+    """Whole-row schedules for rows that start on no 16-byte boundary against the oracle
+    (FP32 budget of the schedule comparison above: 1e-5 after 23 steps)."""
+    nz, ny, nx = shape
+    probe = lbm.Domain(nx, ny, nz, lattice=lbm.LBM_D3Q19, stencil=4, precision=1, collision=coll)
+    names = [k for k in probe.schedule_report() if k.startswith("onepass_rowu")]
+    probe.close()
+    assert names
+    ref = oracle.Sim(LAT[lbm.LBM_D3Q19], nx, ny, nz, stencil=4, G=-5.0, tau=0.9, coll=coll)
+    ref.init_droplet(1.9, 0.15, min(nx, ny, nz) / 4, 2.0)
+    ref.step(23)
+    for name in names:
+        dom = lbm.Domain(nx, ny, nz, lattice=lbm.LBM_D3Q19, stencil=4, precision=1, tau=0.9, collision=coll)
+        dom.set_schedule(name)
+        dom.init_droplet(1.9, 0.15, min(nx, ny, nz) / 4, 2.0)
+        dom.step(23)
+        assert rel_max(dom.get_f(), ref.get_f()) <= 1e-5, name
+        dom.close()
