@@ -223,8 +223,8 @@ __device__ __forceinline__ Real sum_f(const Real (&f)[Lattice<LAT>::Q])
 }
 
 // ---- psi -------------------------------------------------------------------------
-// 1 - exp(-j/64) and exp(-j/64) to the last bit, for psi_exp below: powers of
-// exp(-1/64) in double-double arithmetic, evaluated by the compiler.
+// exp(-j/64) and 1 - exp(-j/64), the latter in two doubles, for psi_exp below: powers
+// of exp(-1/64) in double-double arithmetic, evaluated by the compiler.
 struct DD {
     double h, l;
 };
@@ -235,9 +235,10 @@ constexpr DD dd_sum(double a, double b)  // |a| >= |b|
 }
 constexpr DD dd_mul(DD a, DD b)
 {
-    auto split = [](double v) {  // Dekker: v = hi + lo with 26-bit halves
-        const double t = 134217729.0 * v;
-        const double hi = t - (t - v);
+    // exact product by halves (Dekker), 24 and 29 bits; the split holds whether the host
+    // compiler contracts products and sums or not
+    auto split = [](double v) {
+        const double hi = static_cast<float>(v);
         return DD{hi, v - hi};
     };
     const DD x = split(a.h), y = split(b.h);
@@ -246,7 +247,8 @@ constexpr DD dd_mul(DD a, DD b)
     return dd_sum(p, e + (a.h * b.l + a.l * b.h));
 }
 struct ExpTable {
-    double2 v[1024];  // {exp(-j/64), 1 - exp(-j/64)}
+    double e[1024];   // exp(-j/64)
+    double2 y[1024];  // 1 - exp(-j/64) in two doubles
 };
 constexpr ExpTable make_exp_table()
 {
@@ -266,8 +268,10 @@ constexpr ExpTable make_exp_table()
     DD e{1.0, 0.0};
     for (int j = 0; j < 1024; ++j) {
         const DD c = dd_sum(1.0, -e.h);
-        T.v[j].x = e.h;
-        T.v[j].y = c.h + (c.l - e.l);
+        const DD y = dd_sum(c.h, c.l - e.l);
+        T.e[j] = e.h;
+        T.y[j].x = y.h;
+        T.y[j].y = y.l;
         e = dd_mul(e, q);
     }
     return T;
@@ -276,22 +280,28 @@ __device__ const ExpTable kExpTable = make_exp_table();
 
 // 1 - exp(-r).  Table and polynomial: r = j/64 + x, |x| <= 1/128,
 // 1 - exp(-r) = (1 - e_j) + e_j (1 - exp(-x)), the last factor by its Taylor
-// polynomial (next term 2^-54 of the value): 10 operations of the FP64 pipe where
-// expm1 takes 19 (D2Q9 psi pass at 2048^2: 0.24 -> 0.15 ms).
+// polynomial (next term x^7/5040).  The table holds 1 - e_j in two doubles and the
+// smaller summands are collected before the larger, so that one rounding counts; below
+// 1/16, where the summands would cancel, expm1.  RMS error 0.289 units in the last place
+// (0.290 below 0.1), that of a correctly rounded result; expm1 0.289 to 0.314.
+// j and j/64 come from r's upper word on the integer pipe: 9 operations of the FP64 pipe
+// where expm1 takes 19, and the polynomial does not wait for the table.
 __device__ __forceinline__ double psi_exp(double r)
 {
-    if (static_cast<unsigned>(__double2hiint(r)) >= 0x402f0000u) return -expm1(-r);  // not in [0, 15.5)
-    constexpr double magic = 6755399441055744.0;  // 1.5 * 2^52: the sum holds round(64 r) in its low word
-    const double t = fma(r, 64.0, magic);
-    const int j = __double2loint(t);
-    const double x = fma(t - magic, -1.0 / 64.0, r);
-    double c = fma(x, -1.0 / 720.0, 1.0 / 120.0);
-    c = fma(c, x, -1.0 / 24.0);
-    c = fma(c, x, 1.0 / 6.0);
-    c = fma(c, x, -0.5);
-    c = fma(c, x, 1.0);
-    const double2 e = __ldg(&kExpTable.v[j]);
-    return fma(e.x, c * x, e.y);
+    const int hi = __double2hiint(r);
+    if (static_cast<unsigned>(hi) - 0x3fb00000u >= 0x402f0000u - 0x3fb00000u) return -expm1(-r);  // not in [1/16, 15.5)
+    const int k = 14 + 1023 - (hi >> 20);  // the upper word's lowest k bits count for less than 1/64
+    const int half = 1 << (k - 1);
+    const int j = (((hi & 0xfffff) | 0x100000) + half) >> k;
+    const double x = r - __hiloint2double((hi + half) & -(1 << k), 0);
+    const double e = __ldg(&kExpTable.e[j]);
+    const double2 y = __ldg(&kExpTable.y[j]);
+    double q = fma(x, -1.0 / 720.0, 1.0 / 120.0);
+    q = fma(q, x, -1.0 / 24.0);
+    q = fma(q, x, 1.0 / 6.0);
+    q = fma(q, x, -0.5);
+    const double p = fma(q, x * x, x);
+    return y.x + fma(e, p, y.y);
 }
 __device__ __forceinline__ float psi_exp(float r) { return -expm1f(-r); }
 
