@@ -44,12 +44,12 @@ inline FastDiv make_fast_div(unsigned d)
 // the host.  w: weight of the lattice's largest shell, w1: first force weight
 // times c_s^2 (the force sums come divided by it).
 struct Coll64 {
-    double g, gh;    // -G w1, half of it
-    double k0, k1;   // w omega / (2 c_s^2), -G w1 w pref / c_s^2
-    double w, omega, om1;  // w, omega, 1 - omega
-    double kb, kj;   // exact difference: w / c_s^2, w (1 - omega) / c_s^2
-    double hT;       // exact difference: w / (2 c_s^2)
-    double dmn[19];  // MRT: (omega - s_k) / |M_k|^2
+    double gh, k0;      // -G w1 / 2, w omega / (2 c_s^2)
+    double k1, k1l;     // -G w1 w pref / c_s^2, in two terms
+    double omega, om1;  // omega, 1 - omega
+    double g, gl;       // exact difference: -G w1, in two terms
+    double kb, hT;      // exact difference: w / c_s^2, w / (2 c_s^2)
+    double dmn[19];     // MRT: (omega - s_k) / |M_k|^2
 };
 
 // Runtime constants of one domain, passed by value to every kernel.
