@@ -657,23 +657,21 @@ __device__ __forceinline__ V cdot(V vx, V vy, V vz)
 // lattice, stencil and collision, 40 to 100 steps, over that of the plain form (terms as
 // printed, no sharing): 0.92 on average (geometric), 0.67 to 1.08 by lattice and collision.
 
-// x * 2^K on the integer pipe.  Zero, a result below 2^-1022 (to zero), infinities
-// and NaN are kept apart.
+// x * 2^K on the integer pipe, where x and the result are normal numbers.  scale2_room is
+// below scale2_normal where they are; the values of a cell are tested together, and the
+// others (zero, subnormal, overflow, infinity, NaN) are multiplied.
+constexpr unsigned kExpOne = 1u << 20, kExpMask = 0x7ff00000u;
+template <int K>
+constexpr unsigned scale2_normal = (K < 0 ? kExpMask : kExpMask - kExpOne * K) - kExpOne * (K < 0 ? 1 - K : 1);
+template <int K>
+__device__ __forceinline__ unsigned scale2_room(double x)
+{
+    return (static_cast<unsigned>(__double2hiint(x)) & kExpMask) - kExpOne * (K < 0 ? 1 - K : 1);
+}
 template <int K>
 __device__ __forceinline__ double scale2(double x)
 {
-    if constexpr (K == 0) return x;
-    const int hi = __double2hiint(x);
-    const int e = hi & 0x7ff00000;
-    const bool live = K < 0 ? e > (-K << 20) : e != 0;
-    int h = live ? hi + K * (1 << 20) : hi & 0x80000000;
-    int lo = live ? __double2loint(x) : 0;
-    const bool big = K < 0 ? e == 0x7ff00000 : e >= 0x7ff00000 - (K << 20);
-    if (big) {
-        h = K > 0 && e != 0x7ff00000 ? (hi & 0x80000000) | 0x7ff00000 : hi;
-        lo = K > 0 && e != 0x7ff00000 ? 0 : __double2loint(x);
-    }
-    return __hiloint2double(h, lo);
+    return __hiloint2double(__double2hiint(x) + K * static_cast<int>(kExpOne), __double2loint(x));
 }
 // x * r for a compile-time r
 constexpr int log2_of(double r)
@@ -904,11 +902,22 @@ __device__ __forceinline__ void collide64_at(double (&f)[Lattice<LAT>::Q], const
     const double orho = ONE ? rho : c.omega * rho;
     const double A0 = fma(W.h, orho, W.l != 0.0 ? fma(W.l, orho, -tr) : -tr);
     auto relax = [&](double fb, double x) { return ONE ? x : fma(c.om1, fb, x); };
+    // shells scaled by a power of two wait for the test of all their values
+    auto power = [](auto bI) {
+        constexpr int k = log2_of(weight_ratio<LAT>(decltype(bI)::value));
+        return std::integral_constant<int, k == 99 ? 0 : k>{};
+    };
+    double up[NP], dn[NP];
+    unsigned room = 0, normal = ~0u;  // (all of a lattice's powers fall into the smallest room)
+    auto hold = [&](auto kI, double x) {
+        constexpr int k = decltype(kI)::value;
+        const unsigned m = scale2_room<k>(x);
+        room = m > room ? m : room;
+        normal = scale2_normal<k> < normal ? scale2_normal<k> : normal;
+    };
     auto ratio = [&](auto bI, double x) {
         constexpr double r = weight_ratio<LAT>(decltype(bI)::value);
-        constexpr int k = log2_of(r);
-        if constexpr (k != 99) return scale2<k>(x);
-        else return r * x;
+        return r == 1.0 ? x : r * x;
     };
     sfor<NP>([&](auto kI) {
         constexpr int b = 1 + 2 * decltype(kI)::value;
@@ -937,14 +946,51 @@ __device__ __forceinline__ void collide64_at(double (&f)[Lattice<LAT>::Q], const
             if constexpr (ko >= 0) o = r == 1.0 ? o + O : fma(r, o, O); else o = ratio(std::integral_constant<int, b>{}, o);
             f[b] = relax(f[b], e + o);
             f[b + 1] = relax(f[b + 1], e - o);
+        } else if constexpr (decltype(power(std::integral_constant<int, b>{}))::value != 0) {
+            constexpr auto k = decltype(power(std::integral_constant<int, b>{})){};
+            up[(b - 1) / 2] = e + o;
+            dn[(b - 1) / 2] = e - o;
+            hold(k, up[(b - 1) / 2]);
+            hold(k, dn[(b - 1) / 2]);
         } else {
             f[b] = relax(f[b], ratio(std::integral_constant<int, b>{}, e + o));
             f[b + 1] = relax(f[b + 1], ratio(std::integral_constant<int, b>{}, e - o));
         }
     });
     constexpr DD r0 = weight_ratio2<LAT>(0);
-    if constexpr (r0.l != 0.0) f[0] = relax(f[0], fma(r0.h, A0, r0.l * A0));
-    else f[0] = relax(f[0], ratio(std::integral_constant<int, 0>{}, A0));
+    constexpr auto k0 = decltype(power(std::integral_constant<int, 0>{})){};
+    double rest = A0;
+    if constexpr (r0.l != 0.0) rest = fma(r0.h, A0, r0.l * A0);
+    else if constexpr (k0 != 0) hold(k0, A0);
+    else rest = r0.h * A0;
+    auto scaled = [&](auto by) {
+        if constexpr (COLL != 1)
+            sfor<NP>([&](auto kI) {
+                constexpr int b = 1 + 2 * decltype(kI)::value;
+                constexpr auto k = decltype(power(std::integral_constant<int, b>{})){};
+                if constexpr (k != 0) {
+                    up[decltype(kI)::value] = by(k, up[decltype(kI)::value]);
+                    dn[decltype(kI)::value] = by(k, dn[decltype(kI)::value]);
+                }
+            });
+        if constexpr (k0 != 0) rest = by(k0, rest);
+    };
+    if (room < normal) scaled([](auto kI, double x) { return scale2<decltype(kI)::value>(x); });
+    else
+        scaled([](auto kI, double x) {
+            constexpr int k = decltype(kI)::value;
+            constexpr double by = k < 0 ? 1.0 / (1 << (k < 0 ? -k : 0)) : double(1 << (k < 0 ? 0 : k));
+            return x * by;
+        });
+    if constexpr (COLL != 1)
+        sfor<NP>([&](auto kI) {
+            constexpr int b = 1 + 2 * decltype(kI)::value;
+            if constexpr (decltype(power(std::integral_constant<int, b>{}))::value != 0) {
+                f[b] = relax(f[b], up[decltype(kI)::value]);
+                f[b + 1] = relax(f[b + 1], dn[decltype(kI)::value]);
+            }
+        });
+    f[0] = relax(f[0], rest);
     if constexpr (COLL == 1) {
         double E = 0.0;
         constexpr int ke = mrt_first<LAT>(0, 1);

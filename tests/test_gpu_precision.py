@@ -156,3 +156,21 @@ def test_fp64_psi_at_low_density(lbm):
         return float(np.sqrt((((u - ref) / ref) ** 2).mean()))
 
     assert rms(got["u"][0, 0, 1::3, 0]) <= 1.25 * rms(velocity(np.float64))
+
+
+@pytest.mark.parametrize("lattice", [oracle.D2Q9, oracle.D2Q13, oracle.D2Q25, oracle.D3Q19])
+@pytest.mark.parametrize("rho", [3e-307, 3e-308])
+def test_fp64_populations_below_the_normal_range(lbm, lattice, rho):
+    """A rest state so thin that the outer populations are subnormal: each is a product
+    rounded to a multiple of 2^-1074, so a step moves a population by at most 2^-1074 per
+    operation on it (20) besides the round-off of the normal ones."""
+    shape = (8, 8, 8) if lattice == oracle.D3Q19 else (1, 8, 8)
+    dom = lbm.Domain(*shape[::-1], lattice=lattice, G=-5.0, tau=1.0, precision=0)
+    dom.init_from_rho(np.full(shape, rho))
+    f0 = dom.get_f()
+    dom.step(2)
+    f = dom.get_f()
+    dom.close()
+    _, w, _ = oracle.lattice_table(lattice)
+    assert np.abs(f0 - (w * rho)[:, None, None, None]).max() <= 2 * 5e-324
+    assert np.abs(f - f0).max() <= 40 * 5e-324 + 1e-14 * rho
