@@ -2300,7 +2300,8 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
     const float2 pref = p2(p.pref_f);
     const float2 orho = mul2(omega, rho);
     // A0 = omega s - omega rho usq - pref uF / cs2
-    const float2 A0 = fma2(mul2(pref, p2(float(-1.0 / cs2))), uF, fma2(orho, sub2(p2(0.f), usq), mul2(omega, s)));
+    // (omega s, by far the largest term, is not rounded by itself)
+    const float2 A0 = fma2(mul2(pref, p2(float(-1.0 / cs2))), uF, fma2(omega, s, mul2(vneg(orho), usq)));
     const float2 ic2 = p2(float(1.0 / cs2)), ic4 = p2(float(1.0 / (cs2 * cs2)));
     const float2 Px = mul2(fma2(orho, ux, mul2(pref, F[0])), ic2);
     const float2 Py = mul2(fma2(orho, uy, mul2(pref, F[1])), ic2);
