@@ -75,7 +75,6 @@ struct DevParams {
     // the scalars the FP32 kernels use, so they convert nothing per cell.
     double dmrt[4];
     float omega_f, pref_f, rho_bar_f, G_f;
-    float om1_f;  // 1 - omega, rounded once from double
     float dmrt_f[4];
 };
 
@@ -106,7 +105,6 @@ __host__ __device__ inline void finish_params(DevParams& p)
     p.pref_f = static_cast<float>(p.pref);
     p.rho_bar_f = static_cast<float>(p.rho_bar);
     p.G_f = static_cast<float>(p.G);
-    p.om1_f = static_cast<float>(1.0 - p.omega);
 }
 
 // Everything a launcher may need; unused fields are ignored.

@@ -2257,8 +2257,7 @@ __device__ __forceinline__ float2 cdot2(float2 vx, float2 vy, float2 vz)
 // Packed-pair collision: BGK (COLL = 0) or MRT (COLL = 1, the BGK update plus
 // the moment-space correction of mrt_moments_g / mrt_apply), both Guo-forced.
 template <int LAT, int COLL = 0>
-__device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const float2 (&F)[3], const DevParams& p,
-                                         float om1f)
+__device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const float2 (&F)[3], const DevParams& p)
 {
     static_assert(COLL == 0 || COLL == 1, "packed pairs: BGK or MRT");
     using L = Lattice<LAT>;
@@ -2310,7 +2309,8 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
     const float2 Vx = mul2(fma2(h, ux, mul2(pref, F[0])), ic4);
     const float2 Vy = mul2(fma2(h, uy, mul2(pref, F[1])), ic4);
     const float2 Vz = mul2(fma2(h, uz, mul2(pref, F[2])), ic4);
-    const float2 om1 = p2(om1f);
+    // complementary to the rounded omega, or a density would drift by the difference every step
+    const float2 om1 = p2(1.f - p.omega_f);
     {
         constexpr double w0 = L::T.w[0];
         f[0] = fma2(f[0], om1, mul2(p2(float(w0)), A0));
@@ -2433,8 +2433,7 @@ __global__ void __launch_bounds__(TX * TY / RP, MINB)
                 constexpr int b = decltype(bI)::value;
                 g[b] = make_float2(f[i][b], f[i + 1][b]);
             });
-            // 1 - omega exactly complementary to the rounded omega, as in collide32: the mass stays
-            collide2<LAT, COLL>(g, F, p, 1.f - p.omega_f);
+            collide2<LAT, COLL>(g, F, p);
             const bool second = y0 + ty + i + 1 < ny;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -2645,7 +2644,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32 + (PRODW ? 32 
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(fcur, F, p, p.om1_f);
+                collide2<LAT, COLL>(fcur, F, p);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
                     constexpr int b = decltype(bI)::value;
@@ -2865,8 +2864,7 @@ __global__ void __launch_bounds__((HMAX * TY + 31) / 32 * 32 + 32, 1)
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][d]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                // 1 - omega exactly complementary to the rounded omega, as in collide32: the mass stays
-                collide2<LAT, COLL>(fcur, F, p, 1.f - p.omega_f);
+                collide2<LAT, COLL>(fcur, F, p);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
                     constexpr int b = decltype(bI)::value;
@@ -3093,7 +3091,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32 + (PRODW ? 32 
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(d0, F, p, p.om1_f);
+                collide2<LAT, COLL>(d0, F, p);
                 const int c = m * plane + cell_xy;
                 sfor<Q>([&](auto bI) {
                     constexpr int b = decltype(bI)::value;
@@ -3414,7 +3412,7 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32, 1)
                 });
                 const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
                 const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-                collide2<LAT, COLL>(f, F, p, p.om1_f);
+                collide2<LAT, COLL>(f, F, p);
                 if (m >= m0 && m < m1) {
                     const long long c = static_cast<long long>(m) * plane + cell_xy;
                     sfor<Q>([&](auto bI) {
@@ -3638,7 +3636,7 @@ __global__ void __launch_bounds__(TX / 2 + 32, 1)
             });
             const float2 gp = mul2(p2(-p.G_f), make_float2(rowp[R][0], rowp[R][1]));
             const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), p2(0.f)};
-            collide2<LAT, COLL>(f, F, p, p.om1_f);
+            collide2<LAT, COLL>(f, F, p);
             const int c = m * p.nx + x0 + cx0;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;
@@ -3797,7 +3795,7 @@ __global__ void __launch_bounds__(TX2 * TY, MINB)
             });
             const float2 gp = mul2(p2(-p.G_f), make_float2(base[R][0], base[R][1]));
             const float2 F[3] = {mul2(gp, ax), mul2(gp, ay), mul2(gp, az)};
-            collide2<LAT, 0>(fcur, F, p, p.om1_f);
+            collide2<LAT, 0>(fcur, F, p);
             const int c = m * mscale + cell_xy;
             sfor<Q>([&](auto bI) {
                 constexpr int b = decltype(bI)::value;

@@ -179,12 +179,12 @@ def test_fp64_populations_below_the_normal_range(lbm, lattice, rho):
 @pytest.mark.parametrize("lattice,shape,stencil,coll", [
     (oracle.D2Q9, (1, 96, 128), 4, 0), (oracle.D2Q9, (1, 96, 128), 8, 1), (oracle.D2Q13, (1, 96, 128), 6, 0),
     (oracle.D3Q19, (34, 36, 44), 4, 0), (oracle.D3Q19, (34, 36, 44), 4, 1), (oracle.D3Q19, (34, 36, 44), 6, 0)])
-@pytest.mark.parametrize("tau", [0.8])
+@pytest.mark.parametrize("tau", [0.8, 0.9])
 def test_fp32_schedules_share_one_round_off(lbm, lattice, shape, stencil, coll, tau):
     """Every FP32 schedule rounds the collision's large terms at the same places, so its
     RMS error against an FP64 run, mean of six droplets, is the two-pass schedule's
     within 6% (the order of the small terms differs).  omega is exact in single
-    precision at tau = 0.8."""
+    precision at tau = 0.8 and off by 5e-8 at 0.9, where 1 - omega has to match it."""
     nz, ny, nx = shape
     names, err = None, {}
     for k in range(6):
