@@ -276,7 +276,10 @@ int lbm_batch_set_populations(lbm_batch* b, int d, const double* f_host);
  * steps on the batch's current state, restores the state, and keeps the
  * fastest; all shapes perform the same per-cell arithmetic, so results are
  * bitwise the same whichever is chosen.  The report is "chosen=NAME;NAME=ms;..."
- * in buf (NUL-terminated, truncated to len). */
+ * in buf (NUL-terminated, truncated to len), milliseconds per step of a call of 64
+ * steps ("resident_cluster") or of single steps (the others); NAME is the shape of
+ * calls of 64 steps.  A call of so few steps that loading and storing the resident
+ * domains would not pay takes the fastest of the other shapes instead. */
 int lbm_batch_schedule_report(lbm_batch* b, char* buf, int len);
 
 /* Pins the tile shape to the named one, skipping the autotuner; LBM_EINVAL for

@@ -486,6 +486,7 @@ __global__ void __launch_bounds__(256) k_batch_fused2(const BatchDom* __restrict
 constexpr int kResThreads = 256;
 constexpr int kResRows = 8;       // most rows per thread (144 registers of populations)
 constexpr int kResMaxCluster = 16;
+constexpr int kResTimed = 64;     // steps of the call that the tuner times
 
 // (every thread arrives; the waits end because all blocks of a cluster run together and
 // take the same number of steps)
@@ -993,7 +994,9 @@ struct lbm_batch {
     bool tuned;     // autotuner has run, or a shape was pinned
     bool pinned;    // a shape was pinned by lbm_batch_set_schedule (never re-tuned)
     long long tuned_cells;  // active cells when the shape was last tuned
-    std::vector<double> tune_ms;  // ms per step of each shape (< 0: not timed)
+    std::vector<double> tune_ms;  // ms per step of each shape (< 0: not timed; resident: of a call of kResTimed steps)
+    bool res_tuned;               // the resident shape may take calls from `var`
+    double res_fixed, res_step;   // ms of a resident call of n steps: res_fixed + n res_step
     // resident shape: domains by cluster size, largest first, each class on a stream
     // of its own so that the classes share the GPU
     struct ResClass {
@@ -1310,7 +1313,6 @@ int rebuild_resident(lbm_batch* b)
     if (!list.empty())
         LBM_BCK(cudaMemcpyAsync(b->d_list, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, b->stream));
     LBM_BCK(cudaStreamSynchronize(b->stream));
-    b->nitems = static_cast<int>(list.size());
     return LBM_OK;
 }
 
@@ -1318,7 +1320,7 @@ int rebuild_items(lbm_batch* b)
 {
     const BatchVariant& v = kBatchVariants[b->var];
     // a captured graph holds the classes; domains that retire are skipped by their flag
-    if (v.resident) return b->graph[0] ? LBM_OK : rebuild_resident(b);
+    if (v.resident) return LBM_OK;
     std::vector<int4> items;
     for (int d = 0; d < b->n; ++d) {
         BatchDom& m = b->doms[d];
@@ -1345,10 +1347,21 @@ int rebuild_items(lbm_batch* b)
     return LBM_OK;
 }
 
+// Whether a call of n steps goes to the resident shape.  It reads and writes the state
+// once per call and forks and joins a stream per cluster size, which only many steps pay
+// back: 40 domains of 64^2 to 256^2, us per step, in calls of 1, 4, 16 and 64 steps:
+// resident 107, 38, 24, 20 and tile128_rows16 29, 27, 27, 27; one domain of 64^2: 10, 3.5,
+// 1.6, 1.2 and 14, 13, 12, 12.
+bool takes_resident(const lbm_batch* b, int64_t n)
+{
+    if (kBatchVariants[b->var].resident) return true;
+    return b->res_tuned && b->res_fixed + n * b->res_step < n * b->tune_ms[b->var];
+}
+
 // n steps of every active domain from pool[parity]; the state ends in pool[parity ^ (n & 1)].
 cudaError_t launch_steps(lbm_batch* b, int parity, int64_t n)
 {
-    if (kBatchVariants[b->var].resident) return launch_resident(b, parity, n);
+    if (takes_resident(b, n)) return launch_resident(b, parity, n);
     cudaError_t e = cudaSuccess;
     for (int64_t i = 0; i < n && e == cudaSuccess; ++i)
         e = kBatchVariants[b->var].launch(b, (parity + static_cast<int>(i & 1)) & 1);
@@ -1362,13 +1375,13 @@ int select_variant(lbm_batch* b, int v)
     b->var = v;
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device);
-    if (!kBatchVariants[v].resident)
-        b->grid = std::max(1, nsm * std::max(1, kBatchVariants[v].occupancy(b->fp32)));
     for (int k = 0; k < 2; ++k)
         if (b->graph[k]) {
             cudaGraphExecDestroy(b->graph[k]);
             b->graph[k] = nullptr;
         }
+    if (kBatchVariants[v].resident) return rebuild_resident(b);
+    b->grid = std::max(1, nsm * std::max(1, kBatchVariants[v].occupancy(b->fp32)));
     if (int rc = rebuild_items(b)) return rc;
     // no more persistent blocks than items: the work list only shrinks until the
     // next selection, and the blocks loop over whatever it holds
@@ -1378,7 +1391,8 @@ int select_variant(lbm_batch* b, int v)
 
 // Times every shape on the batch's current state (a few steps each, from a saved
 // copy that is put back afterwards, so the state does not advance) and keeps the
-// fastest.  Without room for the copy the default shape stays.
+// fastest that steps launch by launch and, beside it, the resident shape with what a call
+// and a step of it take.  Without room for the copy the default shape stays.
 int autotune(lbm_batch* b, bool again = false)
 {
     if (b->tuned && !(again && !b->pinned)) return LBM_OK;
@@ -1421,7 +1435,19 @@ int autotune(lbm_batch* b, bool again = false)
     b->tune_ms.assign(kNumBatchVariants, -1.0);
     bool nx4 = true;
     for (const auto& m : b->doms) nx4 = nx4 && m.nx % 4 == 0;
+    // calls of n steps, from an even number of steps after the saved state; ms of one
+    auto timed = [&](int calls, int n) {
+        float ms = 0.f;
+        ck(cudaEventRecord(e0, b->stream));
+        for (int i = 0; i < calls; ++i) ck(launch_steps(b, (b->cur + i * n) & 1, n));
+        ck(cudaEventRecord(e1, b->stream));
+        ck(cudaEventSynchronize(e1));
+        ck(cudaEventElapsedTime(&ms, e0, e1));
+        return static_cast<double>(ms) / calls;
+    };
     int best = 0;
+    bool resident = false;
+    b->res_tuned = false;
     for (int v = 0; v < kNumBatchVariants && rc == LBM_OK; ++v) {
         if (kBatchVariants[v].staged && !(b->fp32 && nx4)) continue;
         if (kBatchVariants[v].resident && !resident_applies(b)) continue;
@@ -1429,17 +1455,17 @@ int autotune(lbm_batch* b, bool again = false)
             rc = r;
             break;
         }
-        // a resident launch reads and writes the state once for all its steps
-        const int timed = kBatchVariants[v].resident ? 8 * kTimed : kTimed;
         ck(launch_steps(b, b->cur, kWarm));
-        ck(cudaEventRecord(e0, b->stream));
-        ck(launch_steps(b, (b->cur + kWarm) & 1, timed));
-        ck(cudaEventRecord(e1, b->stream));
-        ck(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        ck(cudaEventElapsedTime(&ms, e0, e1));
-        b->tune_ms[v] = ms / timed;
-        if (b->tune_ms[v] < b->tune_ms[best]) best = v;
+        if (kBatchVariants[v].resident) {
+            const double many = timed(1, kResTimed), one = timed(kTimed, 1);
+            b->tune_ms[v] = many / kResTimed;
+            b->res_step = std::max(0.0, many - one) / (kResTimed - 1);
+            b->res_fixed = std::max(0.0, one - b->res_step);
+            resident = true;
+        } else {
+            b->tune_ms[v] = timed(1, kTimed) / kTimed;
+            if (b->tune_ms[v] < b->tune_ms[best]) best = v;
+        }
         ck(copy_states(false));
     }
     ck(cudaStreamSynchronize(b->stream));
@@ -1447,6 +1473,7 @@ int autotune(lbm_batch* b, bool again = false)
     if (e1) cudaEventDestroy(e1);
     b->dfree(save);
     if (rc != LBM_OK) return rc;
+    b->res_tuned = resident;
     return select_variant(b, best);
 }
 
@@ -1818,7 +1845,10 @@ int lbm_batch_schedule_report(lbm_batch* b, char* buf, int len)
     if (!b || !buf || len < 1) return set_last_error(LBM_EINVAL, "lbm_batch_schedule_report: bad argument");
     LBM_BCK(cudaSetDevice(b->device));
     if (int rc = autotune(b)) return rc;
-    std::string s = std::string("chosen=") + kBatchVariants[b->var].name;
+    int chosen = b->var;
+    for (int v = 0; v < kNumBatchVariants; ++v)
+        if (kBatchVariants[v].resident && takes_resident(b, kResTimed)) chosen = v;
+    std::string s = std::string("chosen=") + kBatchVariants[chosen].name;
     for (int v = 0; v < kNumBatchVariants && v < (int)b->tune_ms.size(); ++v) {
         if (b->tune_ms[v] < 0) continue;
         char t[96];
@@ -1843,6 +1873,7 @@ int lbm_batch_set_schedule(lbm_batch* b, const char* name)
                 return set_last_error(LBM_EINVAL, "lbm_batch_set_schedule: the resident shape needs FP32 and domains that fit a cluster");
             b->tuned = true;
             b->pinned = true;
+            b->res_tuned = false;
             return select_variant(b, v);
         }
     return set_last_error(LBM_EINVAL, "lbm_batch_set_schedule: unknown tile shape");

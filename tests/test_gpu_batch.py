@@ -210,3 +210,42 @@ def test_batch_resident_shape_is_bitwise_the_tiled_one(lbm, doms):
         with pytest.raises(lbm.LbmError):
             b.set_schedule("resident_cluster")
         b.close()
+
+
+MIXED_SIDES = [64, 96, 128, 192, 256] * 8
+
+
+def mixed_domains():
+    return [dict(nx=n, ny=n, G=-5.0 + 0.01 * i, tau=0.9, R=0.2 * n, stencil=(4, 6, 8, 10)[i % 4], rho_l=2.0,
+                 rho_g=0.15, width=2.0) for i, n in enumerate(MIXED_SIDES)]
+
+
+def test_batch_single_steps_do_not_pay_for_long_calls(lbm):
+    """The tuned batch takes a call of one step about as fast as a pinned per-step shape
+    (a resident call loads and stores every domain and forks a stream per cluster size:
+    3.7 times as slow), and long calls by the faster of the two, whatever came before."""
+    import time
+
+    import torch
+
+    def per_step(b, n, calls):
+        best = float("inf")
+        for _ in range(5):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for _ in range(calls):
+                b.step(n)
+            torch.cuda.synchronize()
+            best = min(best, (time.perf_counter() - t) / (n * calls))
+        return best
+
+    times = {}
+    for name in (None, "tile128_rows16", "resident_cluster"):
+        b = lbm.Batch(mixed_domains(), precision=1)
+        if name:
+            b.set_schedule(name)
+        b.step(2)
+        times[name] = (per_step(b, 1, 100), per_step(b, 2, 50), per_step(b, 128, 4))
+        b.close()
+    for auto, tile, resident in zip(*times.values()):
+        assert auto <= 1.3 * min(tile, resident), times
