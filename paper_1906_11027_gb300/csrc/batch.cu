@@ -1004,6 +1004,7 @@ struct lbm_batch {
         size_t bytes;         // shared memory of a block
     };
     std::vector<ResClass> res;
+    int res_spread;      // how far the listed domains are spread (resident_sizes)
     int* d_list;
     cudaStream_t aux[kResMaxCluster];
     cudaEvent_t ev_fork, ev_join[kResMaxCluster];
@@ -1270,14 +1271,13 @@ constexpr int kMinTX = 32, kMinZC = 8;  // smallest tile and chunk of the table 
         }                                                                                              \
     } while (0)
 
-// Work of the resident shape: active domains grouped by cluster size, largest first.
-// While the blocks would leave more than half of the SMs idle, domains spread over
-// twice, four times, ... as many.
-int rebuild_resident(lbm_batch* b)
+// Cluster sizes of the active domains (0: retired).  While the blocks would leave more
+// than half of the SMs idle, domains spread over twice, four times, ... as many.  Returns
+// the spread.
+int resident_sizes(const lbm_batch* b, int nsm, std::vector<int>& C)
 {
-    int nsm = 0;
-    LBM_BCK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
-    std::vector<int> C(b->n, 0);
+    C.assign(b->n, 0);
+    int taken = 1;
     for (int spread = 1; spread <= kResMaxCluster; spread *= 2) {
         std::vector<int> Cs(b->n, 0);
         int blocks = 0;
@@ -1289,8 +1289,29 @@ int rebuild_resident(lbm_batch* b)
         }
         if (spread > 1 && blocks > nsm) break;
         C = Cs;
+        taken = spread;
         if (2 * blocks > nsm) break;
     }
+    return taken;
+}
+
+// Work of the resident shape: active domains grouped by cluster size, largest first.
+// `only_if_better`: after domains have retired, only when the others would spread
+// further or half of the listed clusters have nothing to do any more (a rebuilt list
+// costs a new captured graph).  *rebuilt: whether the list was made anew.
+int rebuild_resident(lbm_batch* b, bool only_if_better = false, bool* rebuilt = nullptr)
+{
+    int nsm = 0;
+    LBM_BCK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
+    std::vector<int> C;
+    const int spread = resident_sizes(b, nsm, C);
+    int listed = 0, active = 0;
+    for (const auto& k : b->res) listed += k.count;
+    for (const auto& m : b->doms) active += m.active;
+    if (rebuilt) *rebuilt = false;
+    if (only_if_better && spread <= b->res_spread && 2 * active > listed) return LBM_OK;
+    if (rebuilt) *rebuilt = true;
+    b->res_spread = spread;
     std::vector<int> list;
     b->res.clear();
     for (int c = kResMaxCluster; c >= 1; --c) {
@@ -1319,7 +1340,6 @@ int rebuild_resident(lbm_batch* b)
 int rebuild_items(lbm_batch* b)
 {
     const BatchVariant& v = kBatchVariants[b->var];
-    // a captured graph holds the classes; domains that retire are skipped by their flag
     if (v.resident) return LBM_OK;
     std::vector<int4> items;
     for (int d = 0; d < b->n; ++d) {
@@ -1804,6 +1824,17 @@ int lbm_batch_run_to_steady(lbm_batch* b, double tol, int64_t max_steps, int64_t
             nactive = 0;
             for (auto& m : b->doms) nactive += m.active;
             if (int rc = rebuild_items(b)) return rc;
+            // a captured graph holds the resident classes; retired domains are skipped by
+            // their flag, and their clusters go once that is worth a new graph
+            if (nactive > 0 && takes_resident(b, K)) {
+                bool rebuilt = false;
+                if (int rc = rebuild_resident(b, true, &rebuilt)) return rc;
+                if (rebuilt) {
+                    cudaGraphExecDestroy(b->graph[0]);
+                    b->graph[0] = nullptr;
+                    if (int rc = capture()) return rc;
+                }
+            }
             // when the active set has shrunk eightfold, finer items may fill the GPU
             // better: time the shapes again on what is left
             long long cells = 0;

@@ -249,3 +249,65 @@ def test_batch_single_steps_do_not_pay_for_long_calls(lbm):
         b.close()
     for auto, tile, resident in zip(*times.values()):
         assert auto <= 1.3 * min(tile, resident), times
+
+
+def resting(n, k):
+    """Domains of one density: steady at the first check."""
+    return [dict(nx=n, ny=n, G=-4.5, tau=1.0, stencil=4, rho_l=0.7, rho_g=0.7, R=n / 4, width=2.0) for _ in range(k)]
+
+
+def test_batch_resident_survivors_spread_over_freed_sms(lbm):
+    """149 of 150 domains retire at the first check: the last one then runs about as
+    fast as alone, on as many SMs (it stayed on one, among clusters without work)."""
+    import time
+
+    import torch
+
+    drop = dict(nx=64, ny=64, G=-5.0, tau=1.0, stencil=4, rho_l=2.0, rho_g=0.15, R=16.0, width=2.0)
+    times = []
+    for doms in ([drop], [drop] + resting(64, 149)):
+        b = lbm.Batch(doms, precision=1)
+        b.set_schedule("resident_cluster")
+        steps, _, ok = b.run_to_steady(1e-12, 400, 100)
+        assert not ok and list(steps) == [400] + [100] * (len(doms) - 1)
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        b.run_to_steady(1e-12, 4000, 100)
+        times.append(time.perf_counter() - t)
+        b.close()
+    assert times[1] <= 2.0 * times[0], times
+
+
+def test_batch_resident_steady_runs_bitwise_like_the_tiled_shape(lbm):
+    """Clusters of several sizes, forked and joined inside the captured steady block,
+    while domains retire at different checks; then plain steps of what is left, and a
+    call longer than one launch takes (4096 steps) from an odd number of steps on."""
+    doms = [RESIDENT_DOMAINS[k] for k in (0, 1, 6, 8, 9)] + resting(48, 6) + resting(256, 2)
+    doms.append(dict(nx=40, ny=44, G=-5.0, tau=1.0, stencil=4, rho_l=1.93, rho_g=0.16, R=9.0, width=3.0))
+    outs = {}
+    for name in ("tile64_rows16", "resident_cluster"):
+        b = lbm.Batch(doms, precision=1)
+        b.set_schedule(name)
+        b.step(3)
+        steps, obs, ok = b.run_to_steady(2e-7, 1200, 100)
+        again = b.run_to_steady(2e-7, 600, 50)
+        b.step(5)
+        outs[name] = (list(steps), obs, ok, list(again[0]), again[1], [b.get_f(i) for i in range(len(doms))])
+        b.close()
+    a, c = outs.values()
+    assert a[:5] == c[:5]
+    assert len(set(a[0])) >= 3, a[0]  # retired at different checks
+    for i, (x, y) in enumerate(zip(a[5], c[5])):
+        assert np.array_equal(x, y), i
+    long = [dict(nx=8, ny=8, G=-4.5, tau=1.0, stencil=s, rho_l=1.4, rho_g=0.3, R=2.0, width=2.0) for s in (4, 10)]
+    long.append(dict(nx=16, ny=20, G=-4.5, tau=1.0, stencil=6, rho_l=1.4, rho_g=0.3, R=4.0, width=2.0))
+    fs = []
+    for name in ("tile32_rows8", "resident_cluster"):
+        b = lbm.Batch(long, precision=1)
+        b.set_schedule(name)
+        b.step(7)
+        b.step(4097 + 2)
+        fs.append([b.get_f(i) for i in range(len(long))])
+        b.close()
+    for x, y in zip(*fs):
+        assert np.array_equal(x, y)
