@@ -988,6 +988,7 @@ struct lbm_batch {
     cudaGraphExec_t graph[2];
     int graph_k;
     int graph_cur;  // parity the graph was captured from
+    double graph_tol;  // tolerance of its check
     unsigned* d_err;  // device error word (a bounded wait that ran out)
     unsigned* h_err;  // pinned copy, read after every graph block
     int var;        // tile shape in use (index into the variant table)
@@ -1767,7 +1768,7 @@ int lbm_batch_run_to_steady(lbm_batch* b, double tol, int64_t max_steps, int64_t
     // one graph per starting parity is not needed: K is even, so every block of K
     // steps starts from the same parity
     auto capture = [&]() -> int {
-    if (!b->graph[0] || b->graph_k != K || b->graph_cur != b->cur) {
+    if (!b->graph[0] || b->graph_k != K || b->graph_cur != b->cur || b->graph_tol != tol) {
         if (b->graph[0]) cudaGraphExecDestroy(b->graph[0]);
         b->graph[0] = nullptr;
         cudaGraph_t g = nullptr;
@@ -1792,6 +1793,7 @@ int lbm_batch_run_to_steady(lbm_batch* b, double tol, int64_t max_steps, int64_t
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return set_last_error(LBM_ECUDA, cudaGetErrorString(e));
         b->graph_k = K;
+        b->graph_tol = tol;
         b->graph_cur = b->cur;
     }
     return LBM_OK;

@@ -311,3 +311,14 @@ def test_batch_resident_steady_runs_bitwise_like_the_tiled_shape(lbm):
         b.close()
     for x, y in zip(*fs):
         assert np.array_equal(x, y)
+
+
+def test_batch_steady_run_takes_its_own_tolerance(lbm):
+    """A second run with the same check interval and a looser tolerance retires by that
+    tolerance (the captured check kept the first run's)."""
+    b = lbm.Batch(DOMAINS[:1], precision=0)
+    steps, _, ok = b.run_to_steady(1e-14, 200, 100)
+    assert not ok and steps[0] == 200
+    steps, _, ok = b.run_to_steady(1.0, 400, 100)
+    assert ok and steps[0] == 300
+    b.close()
