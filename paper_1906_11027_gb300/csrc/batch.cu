@@ -541,7 +541,7 @@ __host__ __device__ inline int resident_rows_per_thread(int nx, int ny, int C)
 // every working thread has M rows and the compiler may interleave them; rows that two
 // threads share get the same values from both.
 template <int ORD, int M>
-__device__ __forceinline__ void resident_domain(const BatchDom& d, const float* __restrict__ A0, float* __restrict__ B0,
+__device__ __forceinline__ void resident_domain(const BatchDom& d, const float* A0, float* B0,
                                                 float* smem, int rank, int C, int nsteps)
 {
     using L = Lattice<kLatD2Q9>;
@@ -727,10 +727,12 @@ __device__ __forceinline__ void resident_rows(const BatchDom& d, const float* A0
 }
 
 // One cluster per listed domain; every block of a cluster takes the same way through.
+// After an even number of steps a domain goes back to where it came from, so the pools may
+// be one buffer (all of it is read before the first cluster barrier, and written after the
+// last).
 __global__ void __launch_bounds__(kResThreads, 1) k_batch_resident(const BatchDom* __restrict__ doms,
                                                                    const int* __restrict__ list, int C,
-                                                                   const float* __restrict__ pool_in,
-                                                                   float* __restrict__ pool_out, int nsteps)
+                                                                   const float* pool_in, float* pool_out, int nsteps)
 {
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     float* smem = reinterpret_cast<float*>(dyn_smem);
