@@ -2298,17 +2298,19 @@ __device__ __forceinline__ void collide2(float2 (&f)[Lattice<LAT>::Q], const flo
     const float2 omega = p2(p.omega_f);
     const float2 pref = p2(p.pref_f);
     const float2 orho = mul2(omega, rho);
-    // A0 = omega s - omega rho usq - pref uF / cs2
-    // (omega s, by far the largest term, is not rounded by itself)
-    const float2 A0 = fma2(mul2(pref, p2(float(-1.0 / cs2))), uF, fma2(omega, s, mul2(vneg(orho), usq)));
+    // The roundings of the one-cell-per-thread collision, term by term: the large ones
+    // (omega s, which is not rounded by itself) decide how far a run is off, and the small ones
+    // by how much the mass drifts.
     const float2 ic2 = p2(float(1.0 / cs2)), ic4 = p2(float(1.0 / (cs2 * cs2)));
-    const float2 Px = mul2(fma2(orho, ux, mul2(pref, F[0])), ic2);
-    const float2 Py = mul2(fma2(orho, uy, mul2(pref, F[1])), ic2);
-    const float2 Pz = mul2(fma2(orho, uz, mul2(pref, F[2])), ic2);
+    // A0 = omega s - omega rho usq - pref uF / cs2
+    const float2 A0 = fma2(mul2(vneg(pref), uF), ic2, fma2(omega, s, mul2(vneg(orho), usq)));
+    const float2 Px = mul2(fma2(pref, F[0], mul2(orho, ux)), ic2);
+    const float2 Py = mul2(fma2(pref, F[1], mul2(orho, uy)), ic2);
+    const float2 Pz = mul2(fma2(pref, F[2], mul2(orho, uz)), ic2);
     const float2 h = mul2(p2(0.5f), orho);
-    const float2 Vx = mul2(fma2(h, ux, mul2(pref, F[0])), ic4);
-    const float2 Vy = mul2(fma2(h, uy, mul2(pref, F[1])), ic4);
-    const float2 Vz = mul2(fma2(h, uz, mul2(pref, F[2])), ic4);
+    const float2 Vx = mul2(fma2(pref, F[0], mul2(h, ux)), ic4);
+    const float2 Vy = mul2(fma2(pref, F[1], mul2(h, uy)), ic4);
+    const float2 Vz = mul2(fma2(pref, F[2], mul2(h, uz)), ic4);
     // complementary to the rounded omega, or a density would drift by the difference every step
     const float2 om1 = p2(1.f - p.omega_f);
     {
