@@ -139,7 +139,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // The FP64 step kernels of the smallest domains are launched while the one before still
 // runs: pdl_begin lets the next launch start its blocks and then waits until the kernel
 // before has completed and its writes are visible, so launch latency and index
-// arithmetic overlap.  No global memory may be touched before it.
+// arithmetic overlap.  No global memory may be touched before it, and what the kernel
+// before writes is read by ordinary loads, which the wait orders: pointers to it are not
+// __restrict__, or the compiler might take it for read-only for the whole kernel.
 // Only while every block has an SM of its own (64^2: 5.7 -> 5.2 us per step): blocks that
 // start early take the slots they find, and with more than one per SM the FP64 pipes
 // then fill unevenly (256^2 MRT: 22 -> 34 us).
@@ -188,7 +190,7 @@ __device__ __forceinline__ int shift_wrap_fwd(int i, int n)
 
 // Pull gather of the pre-collision populations f_b(x) = A_b(x - c_b).
 template <int LAT, class Real>
-__device__ __forceinline__ void gather(const Real* __restrict__ A, const DevParams& p, int x, int y, int z,
+__device__ __forceinline__ void gather(const Real* A, const DevParams& p, int x, int y, int z,
                                        Real (&f)[Lattice<LAT>::Q])
 {
     using L = Lattice<LAT>;
@@ -351,7 +353,7 @@ __device__ __forceinline__ double psi_of(double rho, const DevParams64& p)
 
 // Writes psi of cell (x, y, z) and its periodic images into the ghosted buffer.
 template <int D, class Real>
-__device__ __forceinline__ void store_psi(Real* __restrict__ psi, const DevParams& p, int x, int y, int z, Real v)
+__device__ __forceinline__ void store_psi(Real* psi, const DevParams& p, int x, int y, int z, Real v)
 {
     const int g = p.g;
     const int gz = (D == 3) ? g : 0;
@@ -1252,8 +1254,7 @@ __device__ __forceinline__ CellXYZ cell_xyz(const DevParams64& p, unsigned i)
 }
 
 template <int LAT>
-__global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, double* __restrict__ psi,
-                                               double* __restrict__ rho, DevParams64 p)
+__global__ void __launch_bounds__(128) k_psi64(const double* A, double* psi, double* rho, DevParams64 p)
 {
     using L = Lattice<LAT>;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1273,8 +1274,8 @@ __global__ void __launch_bounds__(128) k_psi64(const double* __restrict__ A, dou
 
 // Solid nodes (y < wall_rows, 2-D) bounce back: f*_b = f_{-b}.
 template <int LAT, int ORD, int COLL>
-__global__ void __launch_bounds__(128) k_fused64(const double* __restrict__ A, const double* __restrict__ psi,
-                                                 const double* __restrict__ rho, double* __restrict__ B, DevParams64 p)
+__global__ void __launch_bounds__(128) k_fused64(const double* A, const double* psi, const double* rho, double* B,
+                                                 DevParams64 p)
 {
     using L = Lattice<LAT>;
     using S = Stencil<L::D, ORD>;

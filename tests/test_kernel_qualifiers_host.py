@@ -30,3 +30,12 @@ def test_resident_pools_may_be_one_buffer():
             for p in params.split(","):
                 if re.search(r"\b(pool_in|pool_out|A0|B0)\b", p):
                     assert "__restrict__" not in p, (name, p)
+
+
+def test_early_launched_kernels_read_by_ordinary_loads():
+    early = [f for f in functions() if re.search(r"\bpdl_begin\(\);", f[2])]
+    assert len(early) >= 2
+    called = [f for name in ("gather", "store_psi") for f in named(name)]
+    for name, params, body in early + called:
+        assert "__restrict__" not in params, name
+        assert "__ldg(" not in body and "ld.global.nc" not in body, name
