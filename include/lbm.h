@@ -189,9 +189,9 @@ const char* lbm_step_kernel_name(const lbm_ctx* ctx, int i);
  * schedule under AUTO) on the current state, without advancing it, and keeps the
  * fastest; the others can be pinned and are reported with -1 ms.  The variants compute the
  * same step; FP64 variants, 2-D FP32 variants with BGK or MRT and one-cell-per-thread
- * 3-D FP32 variants are bitwise alike, while the packed-pair variants in 3-D and the
- * tiles with exact-difference forcing order some small terms differently and agree
- * within FP32 round-off. */
+ * 3-D FP32 variants are bitwise alike, while the packed-pair variants in 3-D, the tiles
+ * with exact-difference forcing and the "_reg" marches order some small terms
+ * differently and agree within FP32 round-off. */
 int lbm_schedule_report(lbm_ctx* ctx, char* buf, int len);
 
 /* Pins the step schedule to the named candidate (a name lbm_schedule_report

@@ -3468,6 +3468,154 @@ __global__ void __launch_bounds__((NXMAX / 2 * TY + 31) / 32 * 32, 1)
     if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
 }
 
+// One-cell-per-thread form of the segment schedule k_onepass_seg2 below, which it lost to at
+// every size measured; kept for programs that pin it.
+// One-pass schedule with bulk-copy staging for 2-D lattices of reach 1 (D2Q9),
+// any force stencil up to radius 3.  A tile is TX cells of a row; the march runs
+// along y.  For row s, direction b needs row s - c_by over x0 - XP .. x0 + TX + XP
+// (XP = 16 bytes of values >= R + 1): one contiguous segment, copied by one
+// cp.async.bulk (two where it crosses the periodic x edge).  A stage stays
+// resident until the row collides, so the interior populations are read from
+// shared memory twice (psi, then collision) and nothing waits in registers;
+// stages hold NSTG rows, NSTG - R - 1 of them in flight.  A producer warp issues
+// the copies.
+template <int LAT, int ORD, int COLL, class Real, int TX, int ZC, int NSTG>
+__global__ void __launch_bounds__(TX + 32, 1)
+    k_onepass_seg(const __grid_constant__ Pops<Real, Lattice<LAT>::Q> P, DevParams p, int ntx)
+{
+    using L = Lattice<LAT>;
+    using S = Stencil<2, ORD>;
+    constexpr int R = S::radius;
+    constexpr int Q = L::Q;
+    static_assert(L::D == 2 && L::reach == 1, "segment staging is written for 2-D reach-1 lattices");
+    constexpr int XP = 16 / static_cast<int>(sizeof(Real));
+    static_assert(XP >= R + 1 && TX % XP == 0 && TX % 32 == 0, "x pad / tile");
+    constexpr int W = TX + 2 * XP;   // staged segment length
+    constexpr int EX = TX + 2 * R;   // psi ring row
+    constexpr int NS = 2 * R + 2;
+    constexpr int STG = Q * W;
+    static_assert(NSTG >= R + 2 && NSTG >= 2 * R, "one row in flight; the 2R warm-up rows staged at once");
+    __shared__ Real ring[NS * EX];
+    __shared__ alignas(8) unsigned long long bars[NSTG];
+    extern __shared__ __align__(128) unsigned char dyn_smem[];
+    Real* stage = reinterpret_cast<Real*>(dyn_smem);  // [NSTG][Q][W]
+
+    const int tile = blockIdx.x % ntx;
+    const int chunk = blockIdx.x / ntx;
+    const int x0 = tile * TX;
+    const int nm = p.ny;
+    const int m0 = chunk * ZC;
+    const int m1 = (m0 + ZC < nm) ? m0 + ZC : nm;
+    const int tid = threadIdx.x;
+    const int lane = tid & 31;
+    const bool producer = tid >= TX;
+
+    if (tid == 0) {
+        for (int k = 0; k < NSTG; ++k) mbar_init(smem_u32(&bars[k]), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+
+    int cby = 0;
+    const Real* src_b = nullptr;
+    sfor<Q>([&](auto bI) {
+        constexpr int b = decltype(bI)::value;
+        constexpr int vy = L::T.v[b][1];
+        if (lane == b) {
+            cby = vy;
+            src_b = P.in[b];
+        }
+    });
+    const int base = m0 - R;
+    auto issue = [&](int s) {
+        const int slot = (s - base) % NSTG;
+        const uint32_t bar = smem_u32(&bars[slot]);
+        if (lane == 0) mbar_expect_tx(bar, static_cast<uint32_t>(STG * sizeof(Real)));
+        __syncwarp();
+        if (lane < Q) {
+            fence_proxy_async_smem();
+            const Real* row = src_b + static_cast<long long>(wrap_any(s - cby, nm)) * p.nx;
+            uint32_t dst = smem_u32(stage + slot * STG + lane * W);
+            int xs = x0 - XP, left = W;
+            while (left > 0) {
+                const int x = wrap_any(xs, p.nx);
+                const int n = (p.nx - x < left) ? p.nx - x : left;
+                bulk_g2s(dst, row + x, static_cast<uint32_t>(n * sizeof(Real)), bar);
+                dst += static_cast<uint32_t>(n * sizeof(Real));
+                xs += n;
+                left -= n;
+            }
+        }
+    };
+    uint32_t phase = 0;
+    bool ok = true;
+    auto stage_of = [&](int s) { return stage + ((s - base) % NSTG) * STG; };
+    auto wait_stage = [&](int s) {
+        const int slot = (s - base) % NSTG;
+        if (ok && !mbar_wait(smem_u32(&bars[slot]), (phase >> slot) & 1u)) ok = false;  // after a timeout, stop waiting
+        phase ^= 1u << slot;
+    };
+    // f of the cell at tile offset cx (-R .. TX + R - 1) from stage st (pull)
+    auto load_cell = [&](const Real* st, int cx, Real (&f)[Q]) {
+        sfor<Q>([&](auto bI) {
+            constexpr int b = decltype(bI)::value;
+            constexpr int vx = L::T.v[b][0];
+            f[b] = st[b * W + cx + XP - vx];
+        });
+    };
+    auto rho_psi = [&](const Real (&f)[Q]) {
+        const Real sum = sum_f<LAT>(f);
+        const Real rho = std::is_same<Real, float>::value ? Real(p.rho_bar) + sum : sum;
+        return psi_of<LAT>(rho, p);
+    };
+    auto psi_slab = [&](int s) {
+        wait_stage(s);
+        const Real* st = stage_of(s);
+        Real* dst = ring + ring_slot(s, NS) * EX;
+        Real f[Q];
+        load_cell(st, tid, f);
+        dst[tid + R] = rho_psi(f);
+        if (tid < 2 * R) {
+            const int cx = (tid < R) ? tid - R : TX + tid - R;
+            load_cell(st, cx, f);
+            dst[cx + R] = rho_psi(f);
+        }
+    };
+
+    int next = base;
+    const int last = m1 - 1 + R;
+    if (producer)
+        for (; next <= last && next < base + NSTG; ++next) issue(next);
+    if (!producer)
+        for (int s = m0 - R; s < m0 + R; ++s) psi_slab(s);
+    __syncthreads();
+    // slabs below m0 are consumed (psi only): slab k may refill slab k - NSTG's stage
+    if (producer)
+        for (; next <= last && next < m0 + NSTG; ++next) issue(next);
+
+    const bool active = !producer && (x0 + tid) < p.nx;
+    for (int m = m0; m < m1; ++m) {
+        if (!producer) psi_slab(m + R);
+        __syncthreads();
+        // every thread is past the collision of row m - 1
+        if (producer)
+            for (; next <= last && next <= m - 1 + NSTG; ++next) issue(next);
+        if (active) {
+            Real f[Q];
+            load_cell(stage_of(m), tid, f);
+            ForceSum<Real> F;
+            force_ring<LAT, ORD, Real, EX, EX, NS>(ring, m, tid + R, 0, F);
+            collide<LAT, COLL>(f, F, p);
+            const int c = m * p.nx + x0 + tid;
+            sfor<Q>([&](auto bI) {
+                constexpr int b = decltype(bI)::value;
+                __stcs(P.out[b] + c, f[b]);
+            });
+        }
+    }
+    if (!ok && tid == 0) atomicOr(p.err, kErrTimeout);
+}
+
 // One-pass schedule with bulk-copy staging for 2-D lattices of reach 1 (D2Q9), any
 // force stencil up to radius 3, FP32.  A tile is TX cells of a row; the march runs
 // along y.  For row s, direction b needs row s - c_by over x0 - XP .. x0 + TX + XP (XP = 16
@@ -4432,6 +4580,21 @@ cudaError_t launch_onepass_row(const LaunchArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <int LAT, int ORD, int COLL, class Real, int TX, int ZC, int NSTG>
+cudaError_t launch_onepass_seg(const LaunchArgs& a, cudaStream_t s)
+{
+    constexpr int XP = 16 / static_cast<int>(sizeof(Real));
+    constexpr size_t dyn = sizeof(Real) * NSTG * Lattice<LAT>::Q * (TX + 2 * XP);
+    auto kern = &k_onepass_seg<LAT, ORD, COLL, Real, TX, ZC, NSTG>;
+    if (cudaError_t e = ensure_dyn_smem(kern, dyn); e != cudaSuccess) return e;
+    if (a.p.nx % XP != 0) return cudaErrorInvalidValue;
+    const int ntx = (a.p.nx + TX - 1) / TX;
+    const long long nblocks = static_cast<long long>(ntx) * ((a.p.ny + ZC - 1) / ZC);
+    const auto P = make_pops<Real, Lattice<LAT>::Q>(a.fin, a.fout, a.p.N);
+    kern<<<static_cast<unsigned>(nblocks), TX + 32, dyn, s>>>(P, a.p, ntx);
+    return cudaGetLastError();
+}
+
 template <int LAT, int ORD, int COLL, int TX, int ZC, int NSTG>
 cudaError_t launch_onepass_seg2(const LaunchArgs& a, cudaStream_t s)
 {
@@ -4705,8 +4868,20 @@ constexpr VariantList make_variants()
             // velocity set in registers (timed: 60^2 2.6 against 2.9 us, 500 x 300 5.0 against 4.7)
             add("tile32x8", &launch_tile2d<LAT, ORD, COLL, 32, 8, 2, 1>);
             add("tile32x16", &launch_tile2d<LAT, ORD, COLL, 32, 16, RP, 1>, 1, 0, 0, 0, Lattice<LAT>::Q > 16 ? -1 : 80000);
-        } else {
-            pin("onepass_128_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 1, 16, 2, 2>);
+        }
+        // marching and one-cell segment forms
+        pin("onepass_128_z16_b2_smem", &launch_onepass<LAT, ORD, COLL, Real, 128, 1, 16, 2, 2>);
+        if constexpr (hot) {
+            pin("onepass_256_z16_b3_smem", &launch_onepass<LAT, ORD, COLL, Real, 256, 1, 16, 3, 2>);
+            if constexpr (r1) pin("onepass_256_z16_b3_reg", &launch_onepass<LAT, ORD, COLL, Real, 256, 1, 16, 3, 1>);
+            pin("onepass_async_256_z16_b2", &launch_onepass_async<LAT, ORD, COLL, Real, 256, 1, 16, 2>);
+            pin("onepass_x2_256_z16_b2_smem", &launch_onepass_x2<LAT, ORD, 128, 1, 16, 2, 2>, 2);
+        }
+        if constexpr (hot && Lattice<LAT>::reach == 1) {
+            pin("onepass_seg256_z64_s8", &launch_onepass_seg<LAT, ORD, COLL, Real, 256, 64, 8>, 4);
+            pin("onepass_seg256_z64_s6", &launch_onepass_seg<LAT, ORD, COLL, Real, 256, 64, 6>, 4);
+            pin("onepass_seg128_z64_s8", &launch_onepass_seg<LAT, ORD, COLL, Real, 128, 64, 8>, 4);
+            pin("onepass_seg512_z64_s6", &launch_onepass_seg<LAT, ORD, COLL, Real, 512, 64, 6>, 4);
         }
         if constexpr (hot && Lattice<LAT>::reach == 1) {
             add("onepass_seg2_256_z64_s6", &launch_onepass_seg2<LAT, ORD, 0, 256, 64, 6>, 4, 0, 0, 0, kSegMin);

@@ -539,3 +539,30 @@ def test_unaligned_row_schedules(lbm, shape, coll):
         dom.step(23)
         assert rel_max(dom.get_f(), ref.get_f()) <= 1e-5, name
         dom.close()
+
+
+@pytest.mark.parametrize("lattice,shape,stencil,names", [
+    (0, (1, 80, 260), 4, ["onepass_128_z16_b2_smem", "onepass_256_z16_b3_smem", "onepass_256_z16_b3_reg",
+                          "onepass_async_256_z16_b2", "onepass_x2_256_z16_b2_smem", "onepass_seg256_z64_s8",
+                          "onepass_seg256_z64_s6", "onepass_seg128_z64_s8", "onepass_seg512_z64_s6"]),
+    (0, (1, 70, 133), 10, ["onepass_128_z16_b2_smem", "onepass_256_z16_b3_smem", "onepass_async_256_z16_b2"]),
+    (2, (1, 66, 130), 6, ["onepass_128_z16_b2_smem", "onepass_256_z16_b3_smem", "onepass_x2_256_z16_b2_smem"])])
+def test_untimed_2d_schedules_can_still_be_pinned(lbm, lattice, shape, stencil, names):
+    """Schedule names that programs pinned before tiles took over: the step is bitwise
+    that of the two-pass schedule (every one-cell form shares its arithmetic, and the
+    packed pairs round where it does), but for the march that holds a row in registers,
+    which the compiler contracts differently: 40 operations a step, 30 steps."""
+    nz, ny, nx = shape
+    outs = {}
+    for name in ["two_pass"] + names:
+        dom = lbm.Domain(nx, ny, nz, lattice=lattice, stencil=stencil, G=-5.0, tau=0.9, precision=1)
+        dom.init_droplet(2.0, 0.15, 16.0, 2.5)
+        dom.set_schedule(name)
+        dom.step(30)
+        outs[name] = dom.get_f()
+        dom.close()
+    for name in names:
+        if name.endswith("_reg"):
+            assert rel_max(outs[name], outs["two_pass"]) <= 40 * 30 * 2.0 ** -24, name
+        else:
+            assert np.array_equal(outs[name], outs["two_pass"]), name
