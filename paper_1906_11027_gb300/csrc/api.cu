@@ -268,17 +268,26 @@ int one_step(lbm_ctx* c)
 // On small domains a launch takes the host longer than the GPU, and single launches
 // would measure the host (a schedule of two small kernels then looks twice as slow as it
 // is in a replayed graph): there the GPU is first kept busy while the host queues
-// every trial, and the host waits once, at the end.
+// every trial, and the host waits once, at the end.  Calls of many steps replay a graph
+// there, where a launch costs some 3 us less than on a stream, and the two-pass schedule has
+// two: in 3-D it is compared with one launch's difference taken off (24^3, two-pass and
+// onepass_rowu_w116x6_s2: 8.7 and 8.5 us by launches, 4.5 and 7.3 replayed; 64^3: 18.5 and
+// 16.6, 12.6 and 15.0; 80^3: 29.2 and 25.0, 24.8 and 23.2).  In 2-D tiles win either way.
 int autotune(lbm_ctx* c)
 {
     if (c->tuned) return LBM_OK;
     constexpr long long kSmall = 1LL << 20;  // cells below which a step is of the order of a launch
     constexpr unsigned kLaunchNs = 2500;     // host time of one launch
+    constexpr double kReplayMs = 0.003;      // what a launch costs less in a replayed graph
     const bool small = c->N < kSmall;
     const int reps = small ? 8 : 3;  // events resolve a few microseconds
     auto timed = [c](int i) {
         const long long m = c->cand[i] >= 0 ? c->ks.onepass[c->cand[i]].min_cells : 0;
         return m >= 0 && c->N >= m;
+    };
+    const bool less = small && c->graphs_ok && c->li.D == 3;
+    auto replayed = [&](int i) {  // only to compare: the two-pass schedule less its second launch
+        return c->cand_ms[i] - (less && c->cand[i] < 0 ? kReplayMs : 0.0);
     };
     int n_timed = 0;
     for (int i = 0; i < c->n_cand; ++i) {
@@ -317,7 +326,7 @@ int autotune(lbm_ctx* c)
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, ev[2 * i], ev[2 * i + 1]) != cudaSuccess) rc = fail(LBM_ECUDA, "event time");
         c->cand_ms[i] = ms / reps;
-        if (best < 0 || c->cand_ms[i] < c->cand_ms[best]) best = i;
+        if (best < 0 || replayed(i) < replayed(best)) best = i;
     }
     for (auto& e : ev)
         if (e) cudaEventDestroy(e);
