@@ -889,20 +889,20 @@ __global__ void k_batch_init(const BatchDom* __restrict__ doms, const double* __
     }
 }
 
-// State I/O of one domain: f = pre-collision populations in double [9][ny][nx],
-// A the pool's storage (A_b(y) = f_b(y + c_b), FP32 less w_b rho_bar).  On the host the
+// State I/O of one domain, directions [q0, q0 + nq): f = pre-collision populations in double
+// [nq][ny][nx], A the pool's storage of all nine (A_b(y) = f_b(y + c_b), FP32 less w_b rho_bar).  On the host the
 // pull took 1.3 ms per 256 x 256 domain, here 10 us.
 template <bool GET, class Real>
-__global__ void __launch_bounds__(256) k_batch_io(int nx, int ny, double rho_bar, Real* __restrict__ A,
-                                                  double* __restrict__ f)
+__global__ void __launch_bounds__(256) k_batch_io(int nx, int ny, double rho_bar, int q0, int nq,
+                                                  Real* __restrict__ A, double* __restrict__ f)
 {
     using L = Lattice<kLatD2Q9>;
     constexpr bool kDev = std::is_same<Real, float>::value;
     const long long N = static_cast<long long>(nx) * ny;
     const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
-    if (i >= kQ9 * N) return;
-    const int b = static_cast<int>(i / N);
-    const int y = static_cast<int>((i - b * N) / nx), x = static_cast<int>(i - b * N - static_cast<long long>(y) * nx);
+    if (i >= nq * N) return;
+    const int k = static_cast<int>(i / N), b = q0 + k;
+    const int y = static_cast<int>((i - k * N) / nx), x = static_cast<int>(i - k * N - static_cast<long long>(y) * nx);
     int cx = 0, cy = 0;
     double w = 0.0;
     sfor<kQ9>([&](auto bI) {
@@ -919,8 +919,8 @@ __global__ void __launch_bounds__(256) k_batch_io(int nx, int ny, double rho_bar
         const double v = static_cast<double>(A[b * N + static_cast<long long>(wrap_near(y - cy, ny)) * nx + wrap_near(x - cx, nx)]);
         f[i] = kDev ? v + w * rho_bar : v;
     } else {
-        const double v = f[b * N + static_cast<long long>(wrap_near(y + cy, ny)) * nx + wrap_near(x + cx, nx)];
-        A[i] = static_cast<Real>(kDev ? v - w * rho_bar : v);
+        const double v = f[k * N + static_cast<long long>(wrap_near(y + cy, ny)) * nx + wrap_near(x + cx, nx)];
+        A[b * N + i - k * N] = static_cast<Real>(kDev ? v - w * rho_bar : v);
     }
 }
 
@@ -1011,8 +1011,6 @@ struct lbm_batch {
     int* d_list;
     cudaStream_t aux[kResMaxCluster];
     cudaEvent_t ev_fork, ev_join[kResMaxCluster];
-    void* io;            // device copy of one domain's populations in double (state I/O)
-    size_t io_bytes;
 
     void* dalloc(size_t bytes)
     {
@@ -1524,32 +1522,54 @@ cudaError_t launch_obs(lbm_batch* b, int only_active = 0)
     return cudaGetLastError();
 }
 
-// Device area for one domain's populations in double, kept for the next call.
-int ensure_io(lbm_batch* b, size_t bytes)
-{
-    if (b->io_bytes >= bytes) return LBM_OK;
-    b->dfree(b->io);
-    b->io_bytes = 0;
-    b->io = b->dalloc(bytes);
-    if (!b->io) return set_last_error(LBM_ENOMEM, "lbm_batch: scratch allocation failed");
-    b->io_bytes = bytes;
-    return LBM_OK;
-}
-
+// Populations of domain d between its storage and a double host array [9][ny][nx].  They
+// pass through the other pool, which nothing reads between steps where its domains' states
+// lie in this one: all nine directions at once where neighbouring domains leave that much
+// room, else as many as fit (four of an FP32 domain into its own part).  No memory is
+// needed, and a copy costs some 70 us beside its bytes.
 template <bool GET>
-cudaError_t launch_io(lbm_batch* b, int d)
+cudaError_t copy_populations(lbm_batch* b, int d, double* f_host)
 {
     const BatchDom& m = b->doms[d];
-    const long long n = static_cast<long long>(kQ9) * m.nx * m.ny;
-    void* state = static_cast<char*>(b->pool[b->cur_of[d]]) + (b->fp32 ? 4 : 8) * m.off;
-    const unsigned grid = static_cast<unsigned>((n + 255) / 256);
-    if (b->fp32)
-        k_batch_io<GET, float><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, static_cast<float*>(state),
-                                                            static_cast<double*>(b->io));
-    else
-        k_batch_io<GET, double><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, static_cast<double*>(state),
-                                                             static_cast<double*>(b->io));
-    return cudaGetLastError();
+    const long long N = static_cast<long long>(m.nx) * m.ny;
+    const long long es = b->fp32 ? 4 : 8;
+    const long long need = kQ9 * N * static_cast<long long>(sizeof(double));
+    // the longest run of domains whose part of the other pool is free
+    long long at = es * m.off, room = es * kQ9 * N;
+    for (int k = 0, first = 0; k < b->n && room < need; ++k) {
+        if (b->cur_of[k] != b->cur_of[d]) {
+            first = k + 1;
+            continue;
+        }
+        const BatchDom& z = b->doms[k];
+        const long long start = es * b->doms[first].off;
+        const long long bytes = es * (z.off + static_cast<long long>(kQ9) * z.nx * z.ny) - start;
+        if (bytes > room) {
+            room = bytes;
+            at = start;
+        }
+    }
+    const int most = static_cast<int>(std::min<long long>(kQ9, room / (N * static_cast<long long>(sizeof(double)))));
+    void* state = static_cast<char*>(b->pool[b->cur_of[d]]) + es * m.off;
+    double* via = reinterpret_cast<double*>(static_cast<char*>(b->pool[b->cur_of[d] ^ 1]) + at);
+    for (int q0 = 0; q0 < kQ9; q0 += most) {
+        const int nq = std::min(most, kQ9 - q0);
+        const size_t bytes = sizeof(double) * nq * N;
+        cudaError_t e = cudaSuccess;
+        if (!GET) e = cudaMemcpyAsync(via, f_host + q0 * N, bytes, cudaMemcpyHostToDevice, b->stream);
+        if (e != cudaSuccess) return e;
+        const unsigned grid = static_cast<unsigned>((nq * N + 255) / 256);
+        if (b->fp32)
+            k_batch_io<GET, float><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, q0, nq,
+                                                                static_cast<float*>(state), via);
+        else
+            k_batch_io<GET, double><<<grid, 256, 0, b->stream>>>(m.nx, m.ny, m.rho_bar, q0, nq,
+                                                                 static_cast<double*>(state), via);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (GET) e = cudaMemcpyAsync(f_host + q0 * N, via, bytes, cudaMemcpyDeviceToHost, b->stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaStreamSynchronize(b->stream);
 }
 
 double pressure_exp(double rho, double G)
@@ -1716,7 +1736,6 @@ int lbm_batch_destroy(lbm_batch* b)
     b->dfree(b->d_doms);
     b->dfree(b->d_items);
     b->dfree(b->d_list);
-    b->dfree(b->io);
     for (int k = 0; k < kResMaxCluster; ++k) {
         if (b->aux[k]) cudaStreamDestroy(b->aux[k]);
         if (b->ev_join[k]) cudaEventDestroy(b->ev_join[k]);
@@ -1948,11 +1967,7 @@ int lbm_batch_set_populations(lbm_batch* b, int d, const double* f_host)
 {
     if (!b || !f_host || d < 0 || d >= b->n) return set_last_error(LBM_EINVAL, "lbm_batch_set_populations: bad argument");
     LBM_BCK(cudaSetDevice(b->device));
-    const size_t bytes = sizeof(double) * kQ9 * (size_t)b->doms[d].nx * b->doms[d].ny;
-    if (int rc = ensure_io(b, bytes)) return rc;
-    LBM_BCK(cudaMemcpyAsync(b->io, f_host, bytes, cudaMemcpyHostToDevice, b->stream));
-    LBM_BCK(launch_io<false>(b, d));
-    LBM_BCK(cudaStreamSynchronize(b->stream));
+    LBM_BCK(copy_populations<false>(b, d, const_cast<double*>(f_host)));
     return LBM_OK;
 }
 
@@ -1961,11 +1976,7 @@ int lbm_batch_get_populations(lbm_batch* b, int d, double* f_host)
 {
     if (!b || !f_host || d < 0 || d >= b->n) return set_last_error(LBM_EINVAL, "lbm_batch_get_populations: bad argument");
     LBM_BCK(cudaSetDevice(b->device));
-    const size_t bytes = sizeof(double) * kQ9 * (size_t)b->doms[d].nx * b->doms[d].ny;
-    if (int rc = ensure_io(b, bytes)) return rc;
-    LBM_BCK(launch_io<true>(b, d));
-    LBM_BCK(cudaMemcpyAsync(f_host, b->io, bytes, cudaMemcpyDeviceToHost, b->stream));
-    LBM_BCK(cudaStreamSynchronize(b->stream));
+    LBM_BCK(copy_populations<true>(b, d, f_host));
     return LBM_OK;
 }
 

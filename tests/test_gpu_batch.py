@@ -322,3 +322,35 @@ def test_batch_steady_run_takes_its_own_tolerance(lbm):
     steps, _, ok = b.run_to_steady(1.0, 400, 100)
     assert ok and steps[0] == 300
     b.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_batch_state_io_needs_no_memory(lbm, precision):
+    """Reading and writing populations works when the allocator has nothing left, takes
+    nothing from it, and leaves every domain, running or retired, as it was."""
+    b = lbm.Batch(DOMAINS + resting(40, 1), precision=precision, torch_alloc=True)
+    b.step(3)
+    steps, _, _ = b.run_to_steady(1e-9, 100, 50)
+    assert steps[-1] < steps[0]  # the resting domain has retired
+    alloc, live = b._alloc, b._alloc.live
+    torch = alloc._torch
+
+    class Spent:
+        class cuda:
+            @staticmethod
+            def caching_allocator_alloc(*a):
+                raise MemoryError
+
+            caching_allocator_delete = staticmethod(torch.cuda.caching_allocator_delete)
+
+    alloc._torch = Spent
+    fs = [b.get_f(i) for i in range(b.n)]
+    for i, f in enumerate(fs):
+        b.set_f(i, f)
+    for i, f in enumerate(fs):
+        assert np.array_equal(b.get_f(i), f), i
+    assert alloc.live == live
+    b.step(5)
+    assert np.array_equal(b.get_f(b.n - 1), fs[-1]) and not np.array_equal(b.get_f(0), fs[0])
+    b.close()
+    assert alloc.live == 0
