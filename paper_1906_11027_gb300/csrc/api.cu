@@ -133,7 +133,6 @@ struct lbm_ctx {
     int cur;      // index of the buffer holding the current state
     void* psi;
     size_t psi_bytes;
-    double* rho;  // FP64: density written by the psi kernel for the collision (in psi's allocation)
     double* partials;
     double* res;
     unsigned* err;
@@ -182,7 +181,7 @@ struct lbm_ctx {
         a.carry_in = carry[cur];
         a.carry_out = carry[cur ^ 1];
         a.psi = psi;
-        a.rho = rho;
+        a.rho = elem == 8 ? static_cast<double*>(buf[cur ^ 1]) : nullptr;  // until the step's output replaces it
         a.tmap = &tmap;
         a.partials = partials;
         a.nblocks_max = kNBlocksMax;
@@ -585,12 +584,10 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
     c->psi_bytes = (size_t)psx * psy * (nz + 2 * gz) * c->elem;
     const size_t fbytes = (size_t)li.Q * c->N * c->elem;
     // 32 spare bytes: the copies of k_onepass_rowu take whole 16 bytes past a row's end
-    c->buf[0] = c->dalloc(fbytes + 32);
-    c->buf[1] = c->dalloc(fbytes + 32);
-    // psi and, in FP64, the density after it
-    const size_t psi_room = (c->psi_bytes + 255) / 256 * 256;
-    c->psi = c->dalloc(fp32 ? c->psi_bytes : psi_room + sizeof(double) * c->N);
-    if (c->psi && !fp32) c->rho = reinterpret_cast<double*>(static_cast<char*>(c->psi) + psi_room);
+    const size_t spare = fp32 && li.D == 3 ? 32 : 0;
+    c->buf[0] = c->dalloc(fbytes + spare);
+    c->buf[1] = c->dalloc(fbytes + spare);
+    c->psi = c->dalloc(c->psi_bytes);
     c->partials = static_cast<double*>(c->dalloc(sizeof(double) * kNBlocksMax * kObsWidth));
     c->res_len = kResLine + p->nx + 8;
     c->res = static_cast<double*>(c->dalloc(sizeof(double) * c->res_len));

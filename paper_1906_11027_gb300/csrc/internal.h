@@ -117,7 +117,7 @@ struct LaunchArgs {
     double* partials;      // reduction scratch
     int nblocks_max;       // capacity of partials (blocks)
     double* res;           // reduction result (see api.cu for the slots)
-    double* rho;           // density of every cell (FP64 two-pass schedule)
+    double* rho;           // density of every cell (FP64 two-pass schedule; part of fout)
     double* dbuf0;         // double work buffers (N or Q*N)
     double* dbuf1;
     int mode;              // init profile: 0 droplet, 1 flat

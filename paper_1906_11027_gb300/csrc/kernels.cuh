@@ -1235,7 +1235,8 @@ __global__ void __launch_bounds__(32 * TY * TZ)
 // two lanes per cycle and SM: 16 blocks of 256 threads kept 136 SMs idle).  psi
 // comes straight from the ghosted buffer through L1: at two FP64 lanes per
 // cycle the staging of tiles buys nothing.  k_psi64 keeps the density for
-// k_fused64, whose BGK or exact-difference collision needs no sum then.  Per step, with
+// k_fused64, whose BGK or exact-difference collision needs no sum then, where direction 0
+// of the output will be (rho == B: a thread reads its own cell's before it writes it).  Per step, with
 // collide64: D2Q9 64^2 14.3 -> 5.7 us, D2Q25 Peng-Robinson 60^2 32 -> 10.3 us, D2Q9 MRT
 // 256^2 39 -> 22 us, D2Q9 2048^2 1.24 -> 0.58 ms (54 operations where there were 155 in
 // plain form, and 18 for psi where there were 32).

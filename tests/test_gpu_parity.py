@@ -597,3 +597,26 @@ def test_tuned_step_of_a_small_box_is_not_slower_than_two_pass(lbm, side):
         ms[name] = best
         dom.close()
     assert ms[None] <= 1.1 * ms["two_pass"], ms
+
+
+@pytest.mark.parametrize("lattice,shape,radius", [(0, (1, 40, 48), 1), (3, (1, 40, 48), 2), (1, (12, 16, 20), 1)])
+def test_fp64_domain_takes_two_population_buffers_and_psi(lbm, monkeypatch, lattice, shape, radius):
+    """Device memory of an FP64 domain: two buffers of its populations, psi with its
+    ghosts, and what does not grow with the cells; stepping takes no more."""
+    nz, ny, nx = shape
+    sizes = []
+
+    class Counting(lbm.TorchAllocator):
+        def _alloc(self, nbytes, ctx):
+            sizes.append(nbytes)
+            return super()._alloc(nbytes, ctx)
+
+    monkeypatch.setattr(lbm, "TorchAllocator", Counting)
+    dom = lbm.Domain(nx, ny, nz, lattice=lattice, G=-5.0, precision=0, torch_alloc=True)
+    psi = 8 * ((nx + 8 + 3) // 4 * 4) * (ny + 2 * radius) * (nz + (2 * radius if nz > 1 else 0))
+    assert sizes[:3] == [8 * dom.Q * dom.N] * 2 + [psi]
+    dom.init_droplet(2.0, 0.15, 4.0 if nz > 1 else 12.0, 2.0)
+    taken = len(sizes)
+    dom.step(20)
+    assert len(sizes) == taken
+    dom.close()
