@@ -722,6 +722,7 @@ int lbm_init_droplet_learned(lbm_ctx* c, lbm_mlp* net, double R, double rho_l, d
     if (!c || !net || !(R > 0.0) || !(width > 0.0) || !(rho_l > 0.0) || !(rho_g > 0.0))
         return fail(LBM_EINVAL, "bad argument");
     if (c->prm.psi != LBM_PSI_EXP) return fail(LBM_EUNSUPPORTED, "the warm-start network models psi = 1 - exp(-rho)");
+    if (mlp_device(net) != c->device) return fail(LBM_EINVAL, "the network is on device %d, the domain on %d", mlp_device(net), c->device);
     if (int rc = set_device(c)) return rc;
     if (used_fallback) *used_fallback = 0;
     if (c->prm.G > kWarmStartMaxG) {  // near the critical coupling the steady state depends on the start

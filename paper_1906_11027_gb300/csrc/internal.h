@@ -182,6 +182,7 @@ constexpr double kMlpDmax = 24.0;
 }  // namespace lbm
 struct lbm_mlp;
 namespace lbm {
+int mlp_device(const lbm_mlp* n);  // that its parameters are on
 cudaError_t mlp_profile_tables(const lbm_mlp* n, double G, double tau, double order, const double* R_dev, double r_in,
                                int ncand, int T, double dmax, float* tables_dev, cudaStream_t s);
 

@@ -628,7 +628,7 @@ int ensure_train(lbm_mlp* n, int rows)
 {
     if (rows <= n->tcap) return LBM_OK;
     free_train(n);
-    const size_t cap = (std::max(rows, 1024) + 63) / 64 * 64;  // every part starts on 128 bytes
+    const size_t cap = ((size_t)std::max(rows, 1024) + 63) / 64 * 64;  // every part starts on 128 bytes
     const size_t bytes = cap * (sizeof(float) * (kIn + 1) + sizeof(bf16) * kInPad + 8 * sizeof(bf16) * kH +
                                 4 * sizeof(float) * kH + 2 * sizeof(float) + sizeof(bf16) * kOutPad) + 256;
     bool ok = cudaMalloc(&n->train, bytes) == cudaSuccess;
@@ -936,6 +936,8 @@ int lbm_mlp_load(lbm_mlp** out, const char* path)
 
 // ---- evaluation of the network on 1-D tables of signed distances ----------------
 namespace lbm {
+
+int mlp_device(const lbm_mlp* n) { return n->device; }
 
 cudaError_t mlp_profile_tables(const lbm_mlp* n, double G, double tau, double order, const double* R_dev, double r_in,
                                int ncand, int T, double dmax, float* tables_dev, cudaStream_t s)
