@@ -635,20 +635,22 @@ int lbm_create(const lbm_params* p, lbm_ctx** out)
             return cleanup(fail(LBM_EINVAL, "psi of the wall density rho_w is not finite (Peng-Robinson argument below zero)"));
     }
 
-    // TMA descriptor of the ghosted psi buffer; the box is one fused-kernel
-    // tile plus the halo (x: kGhostX each side, y/z: the stencil radius).
-    PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
-    if (!enc) return cleanup(fail(LBM_ECUDA, "cuTensorMapEncodeTiled unavailable"));
-    const CUtensorMapDataType dt = fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-    cuuint64_t dims[3] = {(cuuint64_t)(p->nx + 2 * kGhostX), (cuuint64_t)psy, (cuuint64_t)(nz + 2 * gz)};
-    cuuint64_t strides[2] = {(cuuint64_t)psx * c->elem, (cuuint64_t)psx * psy * c->elem};
-    cuuint32_t box[3] = {(cuuint32_t)(ks.tile_x + 2 * kGhostX), (cuuint32_t)(ks.tile_y + 2 * g),
-                         (cuuint32_t)(ks.tile_z + 2 * gz)};
-    cuuint32_t estr[3] = {1, 1, 1};
-    const cuuint32_t rank = li.D == 3 ? 3 : 2;
-    CUresult cr = enc(&c->tmap, dt, rank, c->psi, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (cr != CUDA_SUCCESS) return cleanup(fail(LBM_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr));
+    // TMA descriptor of the ghosted psi buffer (FP32; the FP64 kernels read it plainly); the
+    // box is one fused-kernel tile plus the halo (x: kGhostX each side, y/z: the stencil radius).
+    if (fp32) {
+        PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
+        if (!enc) return cleanup(fail(LBM_ECUDA, "cuTensorMapEncodeTiled unavailable"));
+        cuuint64_t dims[3] = {(cuuint64_t)(p->nx + 2 * kGhostX), (cuuint64_t)psy, (cuuint64_t)(nz + 2 * gz)};
+        cuuint64_t strides[2] = {(cuuint64_t)psx * c->elem, (cuuint64_t)psx * psy * c->elem};
+        cuuint32_t box[3] = {(cuuint32_t)(ks.tile_x + 2 * kGhostX), (cuuint32_t)(ks.tile_y + 2 * g),
+                             (cuuint32_t)(ks.tile_z + 2 * gz)};
+        cuuint32_t estr[3] = {1, 1, 1};
+        const cuuint32_t rank = li.D == 3 ? 3 : 2;
+        CUresult cr = enc(&c->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, c->psi, dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (cr != CUDA_SUCCESS) return cleanup(fail(LBM_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr));
+    }
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return cleanup(fail(LBM_ECUDA, "create sync failed"));
     *out = c;
     return LBM_OK;

@@ -462,13 +462,6 @@ __device__ __forceinline__ V macc1(V acc, V x)
     else return vmul(vsplat<V>(double(C)), x);
 }
 
-// A scalar parameter in the kernel's precision (FP32 kernels read the FP32 copy).
-template <class Real>
-__device__ __forceinline__ Real par(double d, float f)
-{
-    if constexpr (std::is_same<Real, float>::value) return f; else return d;
-}
-
 // ---- MRT as a correction of the BGK update -------------------------------------
 // With m_eq := M feq and Guo's source in moment space, the MRT update is
 //   m* = m - S (m - m_eq) + (I - S/2) m_src,
@@ -1238,8 +1231,8 @@ __global__ void __launch_bounds__(32 * TY * TZ)
 // k_fused64, whose BGK or exact-difference collision needs no sum then, where direction 0
 // of the output will be (rho == B: a thread reads its own cell's before it writes it).  Per step, with
 // collide64: D2Q9 64^2 14.3 -> 5.7 us, D2Q25 Peng-Robinson 60^2 32 -> 10.3 us, D2Q9 MRT
-// 256^2 39 -> 22 us, D2Q9 2048^2 1.24 -> 0.58 ms (54 operations where there were 155 in
-// plain form, and 18 for psi where there were 32).
+// 256^2 39 -> 22 us, D2Q9 2048^2 1.24 -> 0.58 ms (55 operations where there were 155 in
+// plain form, and 17 for psi where there were 32).
 struct CellXYZ {
     int x, y, z;
 };

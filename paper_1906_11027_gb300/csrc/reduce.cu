@@ -73,18 +73,10 @@ cudaError_t launch_mean(const double* x, long long n, double* partials, int nblo
     return cudaGetLastError();
 }
 
-__device__ __forceinline__ double centre_offset(int i, int n)
-{
-    double d = static_cast<double>(i) - static_cast<double>(n / 2);
-    if (d > 0.5 * n) d -= n;
-    if (d < -0.5 * n) d += n;
-    return d;
-}
-
 // Periodic distance of cell i to the centre node.  The offsets are whole numbers, so
 // their squares are summed as integers and converted by the bits (a conversion
 // instruction takes the FP64 pipe as long as an addition).
-__device__ __forceinline__ int centre_offset_i(int i, int n)
+__device__ __forceinline__ int centre_offset(int i, int n)
 {
     int d = i - n / 2;
     if (2 * d > n) d -= n;
@@ -98,8 +90,8 @@ __device__ __forceinline__ double centre_distance(const DevParams64& p, int dim,
     const int x = static_cast<int>(c - r * p.dnx.d);
     const int z = dim == 3 ? static_cast<int>(p.dny.div(r)) : 0;
     const int y = static_cast<int>(r) - z * p.ny;
-    const long long dx = centre_offset_i(x, p.nx), dy = centre_offset_i(y, p.ny);
-    const long long dz = dim == 3 ? centre_offset_i(z, p.nz) : 0;
+    const long long dx = centre_offset(x, p.nx), dy = centre_offset(y, p.ny);
+    const long long dz = dim == 3 ? centre_offset(z, p.nz) : 0;
     const unsigned long long q = static_cast<unsigned long long>(dx * dx + dy * dy + dz * dz);  // < 2^52
     return sqrt(__longlong_as_double(static_cast<long long>(q | 0x4330000000000000ull)) - 4503599627370496.0);
 }
