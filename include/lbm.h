@@ -187,7 +187,8 @@ const char* lbm_step_kernel_name(const lbm_ctx* ctx, int i);
  * lbm_step (or this call) times the compiled variants that may be fastest at the
  * domain's size (tile shape, chunk length, register cap; and the two-pass
  * schedule under AUTO) on the current state, without advancing it, and keeps the
- * fastest; the others can be pinned and are reported with -1 ms.  The variants compute the
+ * fastest; the others can be pinned and are reported with -1 ms, as is a variant that
+ * would be timed by itself.  The variants compute the
  * same step; FP64 variants, 2-D FP32 variants with BGK or MRT and one-cell-per-thread
  * 3-D FP32 variants are bitwise alike, while the packed-pair variants in 3-D, the tiles
  * with exact-difference forcing and the "_reg" marches order some small terms
